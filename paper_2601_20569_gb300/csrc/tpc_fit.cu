@@ -221,58 +221,77 @@ __global__ void k_st_gather(FrameDev F, KParams P) {
   }
 }
 
-// Sector refit of one track over its kept clusters' positions PS[j], j = j0,
-// j0+dj, ... (nsteps steps).  Each position is loaded one step ahead of the
-// filter, so the load overlaps the arithmetic of the current step.
-__device__ __forceinline__ bool refit_pass(const KParams& P, const float4* PS, int j0, int dj,
-                                           int nsteps, Trk<float>& t) {
-  float4 nxt = PS[j0];
-  for (int s = 0; s < nsteps; ++s) {
-    const float4 cur = nxt;
-    if (s + 1 < nsteps) nxt = PS[j0 + (s + 1) * dj];
-    if (!propagate(t, cur.x, P, P.fit_max_snp)) return false;
-    update(t, residual(t, cur.y, cur.z, P));
-  }
-  return true;
-}
-
+// Sector refit as a per-lane state machine: every loop iteration is one step
+// (propagate to a kept cluster, update) of the lane's current track, and a
+// lane whose track ends takes the next one from the work queue.  A track's
+// 2 nk steps run outward over its kept clusters (innermost first), then, with
+// reset covariance, inward over the same ones; the next position is requested
+// one step ahead of the filter.  One loop body for both passes and all tracks,
+// because what bounds the kernel is the serial chain of a track's steps: as
+// two nested loops per track the lanes of a warp did not reconverge between
+// tracks and passes of unequal length, and a step cost 5 us instead of 0.8.
 __global__ void __launch_bounds__(256) k_sector_refit(FrameDev F, KParams P) {
   const int ns = F.cnt->n_tracks;
   if (F.cnt->err) return;
   const int NR = P.n_rows;
-  for (int q = queue_next(&F.cnt->queue[kQSectorRefit]); q < ns;
-       q = queue_next(&F.cnt->queue[kQSectorRefit])) {
-    const int i = F.st_order[q];
-    const int ti = F.st_tl[i];
-    const int nk = F.tl_nkept[ti];
-    const int* K = F.tl_kept + (long)ti * kMaxRows;  // outermost first
-    const float4* PS = F.st_pos + F.st_off[i];       // same order
-    const int rs = F.srow[K[nk - 1]];
-    F.st_key[i] = F.sid[F.starts[ti]];
-    F.st_sector[i] = rs / NR;
-    F.st_rmin[i] = rs % NR;
-    F.st_rmax[i] = F.srow[K[0]] % NR;
-    F.st_next[i] = -1;
-    F.st_hasprev[i] = 0;
-    F.st_bestB[i] = -1;
-    F.st_bestA[i] = ~0ull;
-    F.st_xbestB[i] = -1;
-    F.st_xbestA[i] = ~0ull;
-    F.st_dz[i] = 0.0f;
-    Trk<float> t;
+  bool busy = false, inward = false;
+  int i = 0, sec = 0, nk = 0, left = 0;
+  const float4* pos = nullptr;
+  float4 nxt;
+  Trk<float> t;
+  for (;;) {
+    if (!busy) {
+      const int q = queue_next(&F.cnt->queue[kQSectorRefit]);
+      if (q >= ns) break;
+      i = F.st_order[q];
+      const int ti = F.st_tl[i];
+      nk = F.tl_nkept[ti];
+      const int* K = F.tl_kept + (long)ti * kMaxRows;  // outermost first
+      pos = F.st_pos + F.st_off[i] + nk - 1;           // same order
+      nxt = *pos;
+      const int rs = F.srow[K[nk - 1]];
+      sec = rs / NR;
+      F.st_key[i] = F.sid[F.starts[ti]];
+      F.st_sector[i] = sec;
+      F.st_rmin[i] = rs % NR;
+      F.st_rmax[i] = F.srow[K[0]] % NR;
+      F.st_next[i] = -1;
+      F.st_hasprev[i] = 0;
+      F.st_bestB[i] = -1;
+      F.st_bestA[i] = ~0ull;
+      F.st_xbestB[i] = -1;
+      F.st_xbestA[i] = ~0ull;
+      F.st_dz[i] = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) t.p[k] = F.tl_par[(long)ti * 5 + k];
-    t.x = F.tl_x[ti];
-    reset_cov(t.c, P);
-    // outward over the kept clusters (innermost first), then inward
-    bool ok = refit_pass(P, PS, nk - 1, -1, nk, t);
-    if (ok) {
-      put_state(F.st_oe + (long)i * kStateF, t, rs / NR);
+      for (int k = 0; k < 5; ++k) t.p[k] = F.tl_par[(long)ti * 5 + k];
+      t.x = F.tl_x[ti];
       reset_cov(t.c, P);
-      ok = refit_pass(P, PS, 0, 1, nk, t);
-      if (ok) put_state(F.st_ie + (long)i * kStateF, t, rs / NR);
+      left = nk;
+      inward = false;
+      busy = true;
+      continue;
     }
-    F.st_ok[i] = ok ? 1 : 0;
+    const float4 cur = nxt;
+    if (--left > 0) {  // (the inward pass starts at the cluster the outward one ends on)
+      pos += inward ? 1 : -1;
+      nxt = *pos;
+    }
+    if (!propagate(t, cur.x, P, P.fit_max_snp)) {
+      F.st_ok[i] = 0;
+      busy = false;
+      continue;
+    }
+    update(t, residual(t, cur.y, cur.z, P));
+    if (left > 0) continue;
+    put_state((inward ? F.st_ie : F.st_oe) + (long)i * kStateF, t, sec);
+    if (inward) {
+      F.st_ok[i] = 1;
+      busy = false;
+    } else {
+      reset_cov(t.c, P);
+      left = nk;
+      inward = true;
+    }
   }
 }
 
