@@ -367,6 +367,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.ft_z0, FT);
   ok &= dalloc(ctx, &F.ft_st_cl, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_st_rs, FT * kMaxRows);
+  ok &= dalloc(ctx, &F.ft_meas, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_store, FT * kMaxRows * 5);
   ok &= dalloc(ctx, &F.ft_flag, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_end2, FT * kStateF);

@@ -216,7 +216,9 @@ __global__ void k_st_gather(FrameDev F, KParams P) {
       }
 #pragma unroll
       for (int u = 0; u < kChunks; ++u)
-        if (c[u] >= 0) out[lane + 32 * u] = make_float4(rx[rr[u] % NR], yz[u].x, yz[u].y, 0.0f);
+        if (c[u] >= 0)
+          out[lane + 32 * u] =
+              make_float4(rx[rr[u] % NR], yz[u].x, yz[u].y, __int_as_float(rr[u]));
     }
   }
 }
@@ -246,15 +248,16 @@ __global__ void __launch_bounds__(256) k_sector_refit(FrameDev F, KParams P) {
       i = F.st_order[q];
       const int ti = F.st_tl[i];
       nk = F.tl_nkept[ti];
-      const int* K = F.tl_kept + (long)ti * kMaxRows;  // outermost first
-      pos = F.st_pos + F.st_off[i] + nk - 1;           // same order
+      pos = F.st_pos + F.st_off[i];  // kept clusters, outermost first
+      const int rs0 = __float_as_int(pos->w);
+      pos += nk - 1;
       nxt = *pos;
-      const int rs = F.srow[K[nk - 1]];
+      const int rs = __float_as_int(nxt.w);
       sec = rs / NR;
       F.st_key[i] = F.sid[F.starts[ti]];
       F.st_sector[i] = sec;
       F.st_rmin[i] = rs % NR;
-      F.st_rmax[i] = F.srow[K[0]] % NR;
+      F.st_rmax[i] = rs0 % NR;
       F.st_next[i] = -1;
       F.st_hasprev[i] = 0;
       F.st_bestB[i] = -1;
@@ -1040,83 +1043,200 @@ __device__ __forceinline__ float zoff(const float* ie) {
   return ie[1] - ie[3] * sqrtf(ie[20] * ie[20] + ie[0] * ie[0]);
 }
 
-// Per fit track, ahead of the fit: the station list, the chain's last
-// segment (whose outer end starts iteration 1), the identity key and the
-// drift-time z offset.  One warp per track: the segments of the chain are
-// taken in order, and the lanes take 32 kept clusters of a segment at a time
-// (innermost first), their loads issued together.  A station is a kept
-// cluster, preceded, on the inner rows of one sector, by an empty station on
-// every row skipped since the previous cluster; a warp scan of the stations
-// each cluster adds gives the places.  Stations beyond kMaxRows are dropped
+// Tracks merged across the central electrode: the measured z of a cluster of
+// sector sec in the frame of the track's first side (zside: the side whose
+// clusters take the shift zsh, -1 for a track on one side), and the window
+// centre cz of that frame in the measured z of sector sec.
+__device__ __forceinline__ int shift_side(const FrameDev& F, int f) {
+  return F.ft_zsh[f] != 0.0f ? 1 - F.ft_side0[f] : -1;
+}
+__device__ __forceinline__ float track_z(float z, int sec, int zside, float zsh, const KParams& P) {
+  return zside >= 0 && ((sec / P.n_phi) & 1) == zside ? z + zsh : z;
+}
+// The shift that applies to the clusters of sector sec (0: none).
+__device__ __forceinline__ float row_shift(int sec, int zside, float zsh, const KParams& P) {
+  return zside >= 0 && ((sec / P.n_phi) & 1) == zside ? zsh : 0.0f;
+}
+
+// A station's measurement for the fit iterations: the cluster's position in
+// the frame of the track's first side, corrected by the map, with the map's x
+// displacement apart (it moves the cluster along the reference of the
+// iteration that uses it).  The correction depends on the row's x, the cluster
+// and the track's z offset, not on the filter state, so it is evaluated once
+// per station here, over all stations at once, instead of in each iteration on
+// its serial chain of steps.
+template <bool kMap>
+__device__ __forceinline__ float4 fit_meas(const MapDev& M, const KParams& P, int rs, float x,
+                                           float y, float z, float z0) {
+  const int sec = rs / P.n_rows, row = rs % P.n_rows;
+  float4 m = make_float4(0.0f, y, z, __uint_as_float((unsigned)sec << 8 | (unsigned)row | kStHave));
+  if (kMap) {
+    float D[3];
+    map_eval(M, P, sec, x, y, z - z0, D);
+    m.x = D[0];
+    m.y = y + D[1];
+    m.z = z + D[2];
+  }
+  return m;
+}
+
+// The measurement (my, mz) of station record m about the reference ref (false:
+// the reference cannot be stepped to the displaced cluster).
+template <bool kMap>
+__device__ __forceinline__ bool meas_at(const float4& m, const KParams& P, const float* ref,
+                                        float& my, float& mz) {
+  my = m.y;
+  mz = m.z;
+  if (kMap && m.x != 0.0f) {
+    StepJ st;
+    if (!helix_step(ref, m.x, P, st, P.fit_max_snp)) return false;
+    my = my - (st.p0 - ref[0]);
+    mz = mz - (st.p1 - ref[1]);
+  }
+  return true;
+}
+
+__device__ __forceinline__ int st_row(const float4& m) { return __float_as_int(m.w) & 0xFF; }
+__device__ __forceinline__ int st_sector(const float4& m) {
+  return (__float_as_int(m.w) >> 8) & 0xFFFF;
+}
+__device__ __forceinline__ bool st_have(const float4& m) {
+  return (__float_as_uint(m.w) & kStHave) != 0u;
+}
+
+// Per fit track, ahead of the fit: the station list with the stations'
+// measurements, the chain's last segment (whose outer end starts iteration 1),
+// the identity key and the drift-time z offset.  A station is a kept cluster,
+// preceded, on the inner rows of one sector, by an empty station on every row
+// skipped since the previous cluster.  Stations beyond kMaxRows are dropped
 // (none are reached: a chain's rows increase along it).
-__global__ void k_fit_stations(FrameDev F, KParams P) {
+//
+// A warp takes 32 tracks.  Its lanes walk their tracks' chains side by side,
+// one segment per round, so that the dependent loads of a segment's header
+// (next segment, tracklet, length, position offset) are in flight for 32 tracks
+// at once; then the warp writes the round's segments one after the other, its
+// lanes over 32 kept clusters at a time (their positions lie in one run, from
+// the sector refit's gather), a warp scan of the stations each cluster adds
+// giving the places.
+template <bool kMap>
+__global__ void __launch_bounds__(kBlock, 3) k_fit_stations(FrameDev F, KParams P, MapDev M) {
+  if (!kMap) M.on = 0;
+  __shared__ float rx[kMaxRows];
+  for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
+  __syncthreads();
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   if (F.cnt->err) return;
   const int NR = P.n_rows;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
-  for (int f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); f < nf; f += nw) {
-    const int head = F.ft_head[f];
-    int* SC = F.ft_st_cl + (long)f * kMaxRows;
-    uint16_t* SR = F.ft_st_rs + (long)f * kMaxRows;
+  // tracks per warp: 32, fewer where that would leave warps without work
+  const int per = max(1, min(32, (nf + nw - 1) / nw));
+  for (int f0 = per * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); f0 < nf;
+       f0 += per * nw) {
+    const int f = f0 + lane;
+    const bool mine = lane < per && f < nf;
+    const int head = mine ? F.ft_head[f] : -1;
     // across the central electrode: the side of the first segment, and the
     // z shift of the clusters on the other side (set at the first segment
     // there, 0 for a chain on one side)
-    const int side0 = (F.st_sector[head] / P.n_phi) & 1;
+    const int side0 = mine ? (F.st_sector[head] / P.n_phi) & 1 : 0;
+    const float z0 = mine ? zoff(F.st_ie + (long)head * kStateF) : 0.0f;
     float zsh = 0.0f;
     bool crossed = false;
-    int last = head, ns = 0, prev = -1;
-    for (int sg = head; sg >= 0; sg = F.st_next[sg]) {
-      last = sg;
-      if (!crossed && ((F.st_sector[sg] / P.n_phi) & 1) != side0) {
-        crossed = true;
-        zsh = F.st_dz[sg];
+    int sg = head, last = head, ns = 0, prev = -1;
+    while (__any_sync(0xffffffffu, sg >= 0)) {
+      int ti = 0, nk = 0, off = 0, nxt = -1;
+      if (sg >= 0) {
+        last = sg;
+        nxt = F.st_next[sg];
+        off = F.st_off[sg];
+        ti = F.st_tl[sg];
+        nk = F.tl_nkept[ti];
+        if (!crossed && ((F.st_sector[sg] / P.n_phi) & 1) != side0) {
+          crossed = true;
+          zsh = F.st_dz[sg];
+        }
       }
-      const int ti = F.st_tl[sg];
-      const int nk = F.tl_nkept[ti];
-      const int* K = F.tl_kept + (long)ti * kMaxRows;  // outermost first
-      for (int j0 = 0; j0 < nk; j0 += 32) {
-        const bool valid = j0 + lane < nk;
-        const int c = valid ? K[nk - 1 - (j0 + lane)] : -1;
-        const int rs = valid ? (int)F.srow[c] : 0;
-        int prs = __shfl_up_sync(0xffffffffu, rs, 1);
-        if (lane == 0) prs = prev;
-        int gap = 0;
-        if (valid && prs >= 0 && prs / NR == rs / NR)
-          gap = max(0, min(rs % NR, P.inner_rows) - (prs % NR + 1));
-        const int add = valid ? gap + 1 : 0;
-        int incl = add;
+      for (unsigned todo = __ballot_sync(0xffffffffu, sg >= 0); todo; todo &= todo - 1) {
+        const int j = __ffs(todo) - 1;
+        const int tj = __shfl_sync(0xffffffffu, ti, j);
+        const int nj = __shfl_sync(0xffffffffu, nk, j);
+        const int oj = __shfl_sync(0xffffffffu, off, j);
+        const int sj = __shfl_sync(0xffffffffu, side0, j);
+        const float z0j = __shfl_sync(0xffffffffu, z0, j);
+        const float zshj = __shfl_sync(0xffffffffu, zsh, j);
+        int nsj = __shfl_sync(0xffffffffu, ns, j);
+        int pj = __shfl_sync(0xffffffffu, prev, j);
+        const int zside = zshj != 0.0f ? 1 - sj : -1;
+        const int* K = F.tl_kept + (long)tj * kMaxRows;  // outermost first
+        int* SC = F.ft_st_cl + (long)(f0 + j) * kMaxRows;
+        uint16_t* SR = F.ft_st_rs + (long)(f0 + j) * kMaxRows;
+        float4* SM = F.ft_meas + (long)(f0 + j) * kMaxRows;
+        for (int j0 = 0; j0 < nj; j0 += 32) {
+          const bool valid = j0 + lane < nj;
+          const int q = nj - 1 - (j0 + lane);
+          const int c = valid ? K[q] : -1;
+          float4 ps = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (valid) {
+            if (oj >= 0) {
+              ps = F.st_pos[oj + q];
+            } else {  // a segment of the edge following
+              const float2 yz = F.syz[c];
+              const int r = F.srow[c];
+              ps = make_float4(rx[r % NR], yz.x, yz.y, __int_as_float(r));
+            }
+          }
+          const int rs = __float_as_int(ps.w);
+          int prs = __shfl_up_sync(0xffffffffu, rs, 1);
+          if (lane == 0) prs = pj;
+          int gap = 0;
+          if (valid && prs >= 0 && prs / NR == rs / NR)
+            gap = max(0, min(rs % NR, P.inner_rows) - (prs % NR + 1));
+          const int add = valid ? gap + 1 : 0;
+          int incl = add;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += v;
-        }
-        const int pos = ns + incl - add;
-        if (valid) {
-          for (int q = 0; q < gap && pos + q < kMaxRows; ++q) {
-            SC[pos + q] = -1;
-            SR[pos + q] = (uint16_t)(rs - rs % NR + prs % NR + 1 + q);
+          for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
           }
-          if (pos + gap < kMaxRows) {
-            SC[pos + gap] = c;
-            SR[pos + gap] = (uint16_t)rs;
-            // Phase III: clusters held by a station outside the inner region
-            // are not extrapolation candidates of any track
-            if (P.ext_rows > 0 && rs % NR >= P.inner_rows) F.ft_fixed[c] = 1;
+          const int at = nsj + incl - add;
+          if (valid) {
+            for (int e = 0; e < gap && at + e < kMaxRows; ++e) {
+              const int re = rs - rs % NR + prs % NR + 1 + e;
+              SC[at + e] = -1;
+              SR[at + e] = (uint16_t)re;
+              SM[at + e] = make_float4(0.0f, 0.0f, 0.0f,
+                                       __uint_as_float((unsigned)(re / NR) << 8 |
+                                                       (unsigned)(re % NR)));
+            }
+            if (at + gap < kMaxRows) {
+              SC[at + gap] = c;
+              SR[at + gap] = (uint16_t)rs;
+              SM[at + gap] = fit_meas<kMap>(M, P, rs, ps.x, ps.y,
+                                            track_z(ps.z, rs / NR, zside, zshj, P), z0j);
+              // Phase III: clusters held by a station outside the inner region
+              // are not extrapolation candidates of any track
+              if (P.ext_rows > 0 && rs % NR >= P.inner_rows) F.ft_fixed[c] = 1;
+            }
           }
+          const int nvalid = min(32, nj - j0);
+          nsj += __shfl_sync(0xffffffffu, incl, 31);
+          pj = __shfl_sync(0xffffffffu, rs, nvalid - 1);
         }
-        const int nvalid = min(32, nk - j0);
-        ns += __shfl_sync(0xffffffffu, incl, 31);
-        prev = __shfl_sync(0xffffffffu, rs, nvalid - 1);
+        if (lane == j) {
+          ns = nsj;
+          prev = pj;
+        }
       }
+      sg = nxt;
     }
-    if (lane == 0) {
+    if (mine) {
       F.ft_side0[f] = side0;
       F.ft_zsh[f] = zsh;
       F.ft_nst[f] = min(ns, kMaxRows);
       F.ft_key[f] = F.st_key[head];
       F.ft_last[f] = last;
-      F.ft_z0[f] = zoff(F.st_ie + (long)head * kStateF);
+      F.ft_z0[f] = z0;
       F.ft_next[f] = 0;
       F.ft_nout[f] = 0;
     }
@@ -1150,21 +1270,6 @@ __device__ __forceinline__ bool ext_step(Lin& L, int& sec, int r, const float* r
     sec = nsec;
   }
   return !(fabsf(L.t.p[0]) > L.t.x * P.tan_half + P.edge_margin);
-}
-
-// Tracks merged across the central electrode: the measured z of a cluster of
-// sector sec in the frame of the track's first side (zside: the side whose
-// clusters take the shift zsh, -1 for a track on one side), and the window
-// centre cz of that frame in the measured z of sector sec.
-__device__ __forceinline__ int shift_side(const FrameDev& F, int f) {
-  return F.ft_zsh[f] != 0.0f ? 1 - F.ft_side0[f] : -1;
-}
-__device__ __forceinline__ float track_z(float z, int sec, int zside, float zsh, const KParams& P) {
-  return zside >= 0 && ((sec / P.n_phi) & 1) == zside ? z + zsh : z;
-}
-// The shift that applies to the clusters of sector sec (0: none).
-__device__ __forceinline__ float row_shift(int sec, int zside, float zsh, const KParams& P) {
-  return zside >= 0 && ((sec / P.n_phi) & 1) == zside ? zsh : 0.0f;
 }
 
 __device__ __forceinline__ void inner_candidates(FrameDev& F, const KParams& P, const MapDev& M,
@@ -1284,14 +1389,14 @@ __device__ __forceinline__ void ext_candidates(FrameDev& F, const KParams& P, co
   F.ft_assigned[slot] = -1;
 }
 
-// Iteration 1 (inward, storing the predictions) and the Phase III
+// Iteration 1 (inward, storing the predictions) and (kExt) the Phase III
 // extrapolation below the track, as a per-lane state machine: every loop
 // iteration is one station (or extrapolated row) of the lane's current track,
 // and a lane whose track ends takes the next one from the work queue.  The
-// end state of iteration 1 goes to ft_end2 for k_fit2.
-template <bool kMap, int kPart>
-__global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
-    k_fit1(FrameDev F, KParams P, MapDev M) {
+// next station's record is requested one step ahead.  The end state of
+// iteration 1 goes to ft_end2 for k_fit2.
+template <bool kMap, bool kExt>
+__global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1303,45 +1408,39 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
   int phase = kFitIdle;
   int f = 0, ns = 0, k = 0;
   bool lp = false;  // FP64 updates (low-pT looper)
-  float z0 = 0.0f;
-  int zside = -1;   // central-electrode merging: side whose z takes zsh
-  float zsh = 0.0f;
   int xsec = 0;     // sector of the extrapolation
-  const int* SC = nullptr;
-  const uint16_t* SR = nullptr;
+  const float4* SM = nullptr;
+  float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float* store = nullptr;
   Lin L;
   for (;;) {
     if (phase == kFitIdle) {
-      const int q = fit_next_part<kPart>(F.cnt, kQFit12, kQFit12N, nL, nf);
+      const int q = fit_next(F.cnt, kQFit12, kQFit12N, nL, nf);
       if (q >= nf) break;
       f = F.ft_order[q];
-      lp = fit_looper<kPart>(F, f);
+      lp = F.ft_looper[f] != 0;
       ns = F.ft_nst[f];
       F.ft_ok[f] = 0;
       if (ns == 0) continue;  // not reached: every chain holds clusters
-      z0 = F.ft_z0[f];
-      zsh = F.ft_zsh[f];
-      zside = shift_side(F, f);
-      SC = F.ft_st_cl + (long)f * kMaxRows;
-      SR = F.ft_st_rs + (long)f * kMaxRows;
+      SM = F.ft_meas + (long)f * kMaxRows;
       store = F.ft_store + (long)f * kMaxRows * 5;
+      nxt = SM[ns - 1];
       Trk<float> s0;
       get_state(F.st_oe + (long)F.ft_last[f] * kStateF, s0);
-      lin_start(L, s0, SR[ns - 1] / NR, P);
+      lin_start(L, s0, st_sector(nxt), P);
       k = ns - 1;
       phase = kFitIn;
       continue;
     }
-    if (phase == kFitExt) {
+    if (kExt && phase == kFitExt) {
       // Phase III: one row of the inward extrapolation below the innermost
-      // station (k counts the rows done)
-      const int r = SR[0] % NR - 1 - k;
+      // station (k counts the rows done; nxt: the innermost station)
+      const int r = st_row(nxt) - 1 - k;
       bool go = k < P.ext_rows && r >= 0;
       if (go) go = ext_step(L, xsec, r, rx, P);
       if (go) {
-        ext_candidates(F, P, M, f, kMaxInner + k, xsec * NR + r, L, z0,
-                       row_shift(xsec, zside, zsh, P));
+        ext_candidates(F, P, M, f, kMaxInner + k, xsec * NR + r, L, F.ft_z0[f],
+                       row_shift(xsec, shift_side(F, f), F.ft_zsh[f], P));
         F.ft_ext_sec[(long)f * 2 * P.ext_rows + k] = (uint16_t)xsec;
         ++k;
       } else {
@@ -1351,27 +1450,18 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
       }
       continue;
     }
-    // ---- one station.  The cluster does not depend on the state: it is
-    // requested before the station change so that its latency overlaps the
-    // arithmetic.
-    const int rs = SR[k];
-    const int c = SC[k];
-    const int sec = rs / NR, row = rs % NR;
-    float cy = 0.0f, cz = 0.0f;
-    if (c >= 0) {
-      const float2 pc = F.syz[c];
-      cy = pc.x;
-      cz = track_z(pc.y, sec, zside, zsh, P);
-    }
+    // ---- one station
+    const float4 m = nxt;
+    if (k > 0) nxt = SM[k - 1];
     bool ok = true;
-    if (k != ns - 1) ok = lin_goto(L, sec, rx[row], P);
+    if (k != ns - 1) ok = lin_goto(L, st_sector(m), rx[st_row(m)], P);
     bool have = false;
     float my = 0.0f, mz = 0.0f;
     if (ok) {
       float* st = store + k * 5;
       st[0] = L.t.p[0]; st[1] = L.t.p[1]; st[2] = L.t.c[0]; st[3] = L.t.c[1]; st[4] = L.t.c[2];
-      if (c >= 0) {
-        ok = corrected(M, P, sec, L.t.x, cy, cz, z0, L.r, my, mz);
+      if (st_have(m)) {
+        ok = meas_at<kMap>(m, P, L.r, my, mz);
         have = ok;
       }
     }
@@ -1383,9 +1473,9 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     if (--k < 0) {
       // the end of iteration 1 starts iteration 2
       put_state(F.ft_end2 + (long)f * kStateF, L.t, L.sector);
-      if (P.ext_rows > 0) {
+      if (kExt) {
         k = 0;
-        xsec = SR[0] / NR;
+        xsec = st_sector(nxt);
         phase = kFitExt;
       } else {
         F.ft_ok[f] = 1;
@@ -1397,13 +1487,13 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
 
 // Iteration 2 (outward) as the same kind of state machine: interpolation with
 // the stored predictions, flags of outliers, inner-row candidates (Sec. 3,
-// Phases I and II), then the Phase III extrapolation above the outermost
-// station.  Starts from the end of iteration 1, ends in ft_end2.
+// Phases I and II), then (kExt) the Phase III extrapolation above the
+// outermost station.  Starts from the end of iteration 1, ends in ft_end2.  A
+// flagged station's record loses its cluster (iteration 3 skips it).
 enum : int { kFit2Idle = 0, kFit2St, kFit2Out };
 
-template <bool kMap, int kPart>
-__global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
-    k_fit2(FrameDev F, KParams P, MapDev M) {
+template <bool kMap, bool kExt>
+__global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1415,46 +1505,43 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
   int phase = kFit2Idle;
   int f = 0, ns = 0, k = 0;
   bool lp = false;  // FP64 updates (low-pT looper)
-  float z0 = 0.0f;
-  int zside = -1;   // central-electrode merging: side whose z takes zsh
-  float zsh = 0.0f;
   int xsec = 0;     // sector of the extrapolation
-  const int* SC = nullptr;
-  const uint16_t* SR = nullptr;
+  float4* SM = nullptr;
+  float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const float* store = nullptr;
+  float sn[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // the next station's prediction
   uint8_t* flag = nullptr;
   Lin L;
   for (;;) {
     if (phase == kFit2Idle) {
-      const int q = fit_next_part<kPart>(F.cnt, kQFit2, kQFit2N, nL, nf);
+      const int q = fit_next(F.cnt, kQFit2, kQFit2N, nL, nf);
       if (q >= nf) break;
       f = F.ft_order[q];
       if (!F.ft_ok[f]) continue;
-      lp = fit_looper<kPart>(F, f);
+      lp = F.ft_looper[f] != 0;
       ns = F.ft_nst[f];
-      z0 = F.ft_z0[f];
-      zsh = F.ft_zsh[f];
-      zside = shift_side(F, f);
-      SC = F.ft_st_cl + (long)f * kMaxRows;
-      SR = F.ft_st_rs + (long)f * kMaxRows;
+      SM = F.ft_meas + (long)f * kMaxRows;
       store = F.ft_store + (long)f * kMaxRows * 5;
       flag = F.ft_flag + (long)f * kMaxRows;
+      nxt = SM[0];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) sn[i] = store[i];
       Trk<float> s1;
       get_state(F.ft_end2 + (long)f * kStateF, s1);
-      lin_start(L, s1, SR[0] / NR, P);
+      lin_start(L, s1, st_sector(nxt), P);
       k = 0;
       phase = kFit2St;
       continue;
     }
-    if (phase == kFit2Out) {
+    if (kExt && phase == kFit2Out) {
       // Phase III: one row of the outward extrapolation above the outermost
-      // station (k counts the rows done)
-      const int r = SR[ns - 1] % NR + 1 + k;
+      // station (k counts the rows done; nxt: the outermost station)
+      const int r = st_row(nxt) + 1 + k;
       bool go = k < P.ext_rows && r < NR;
       if (go) go = ext_step(L, xsec, r, rx, P);
       if (go) {
-        ext_candidates(F, P, M, f, kMaxInner + P.ext_rows + k, xsec * NR + r, L, z0,
-                       row_shift(xsec, zside, zsh, P));
+        ext_candidates(F, P, M, f, kMaxInner + P.ext_rows + k, xsec * NR + r, L, F.ft_z0[f],
+                       row_shift(xsec, shift_side(F, f), F.ft_zsh[f], P));
         F.ft_ext_sec[(long)f * 2 * P.ext_rows + P.ext_rows + k] = (uint16_t)xsec;
         ++k;
       } else {
@@ -1463,34 +1550,34 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
       }
       continue;
     }
-    // ---- one station.  The cluster and the stored prediction do not depend
-    // on the state: they are requested before the station change.
-    const int rs = SR[k];
-    const int c = SC[k];
-    const int sec = rs / NR, row = rs % NR;
-    float cy = 0.0f, cz = 0.0f;
-    if (c >= 0) {
-      const float2 pc = F.syz[c];
-      cy = pc.x;
-      cz = track_z(pc.y, sec, zside, zsh, P);
-    }
+    // ---- one station
+    const float4 m = nxt;
     float sv[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) sv[i] = store[k * 5 + i];
+    for (int i = 0; i < 5; ++i) sv[i] = sn[i];
+    if (k + 1 < ns) {
+      nxt = SM[k + 1];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) sn[i] = store[(k + 1) * 5 + i];
+    }
     bool ok = true;
-    if (k != 0) ok = lin_goto(L, sec, rx[row], P);
-    const bool inner = row < P.inner_rows;
+    if (k != 0) ok = lin_goto(L, st_sector(m), rx[st_row(m)], P);
+    const bool inner = st_row(m) < P.inner_rows;
     bool have = false;
     float my = 0.0f, mz = 0.0f;
     if (ok) {
       const float a[5] = {L.t.p[0], L.t.p[1], L.t.c[0], L.t.c[1], L.t.c[2]};
       const Interp I = interpolate(a, sv);
-      flag[k] = 0;
-      if (c >= 0 && !inner) {
-        ok = corrected(M, P, sec, L.t.x, cy, cz, z0, L.r, my, mz);
+      int fl = 0;
+      if (st_have(m)) {
+        ok = meas_at<kMap>(m, P, L.r, my, mz);
         have = ok;
-        if (ok) flag[k] = chi2_interp(I, my, mz, P) > P.int_chi2 ? 1 : 0;
+        if (ok && !inner && chi2_interp(I, my, mz, P) > P.int_chi2) {
+          fl = 1;
+          SM[k].w = __uint_as_float(__float_as_uint(m.w) & ~kStHave);
+        }
       }
+      flag[k] = (uint8_t)fl;
       if (ok && inner) {
         // Phase II candidates of this inner station: the search runs later in
         // k_inner_cand, over all (track, inner station) pairs at once
@@ -1499,10 +1586,6 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
         ip[5] = L.t.x;
 #pragma unroll
         for (int i = 0; i < 5; ++i) ip[6 + i] = L.r[i];
-        if (c >= 0) {
-          ok = corrected(M, P, sec, L.t.x, cy, cz, z0, L.r, my, mz);
-          have = ok;
-        }
       }
     }
     if (have) update_as(L.t, residual(L.t, my, mz, P), lp);
@@ -1514,8 +1597,8 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     if (++k == ns) {
       put_state(F.ft_end2 + (long)f * kStateF, L.t, L.sector);
       k = 0;
-      xsec = SR[ns - 1] / NR;
-      phase = P.ext_rows > 0 ? kFit2Out : kFit2Idle;
+      xsec = st_sector(nxt);
+      phase = kExt ? kFit2Out : kFit2Idle;
     }
   }
 }
@@ -1607,7 +1690,11 @@ __global__ void k_amb_resolve(FrameDev F, KParams P, int round) {
   }
 }
 
-__global__ void k_amb_mark(FrameDev F, KParams P, int round) {
+// The last round (kLast) also brings the inner stations' measurements in line
+// with the clusters they were given, for iteration 3.
+template <bool kLast, bool kMap>
+__global__ void k_amb_mark(FrameDev F, KParams P, MapDev M, int round) {
+  if (!kMap) M.on = 0;
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   if (F.cnt->err) return;
   const long tot = (long)nf * amb_per(P);
@@ -1616,6 +1703,22 @@ __global__ void k_amb_mark(FrameDev F, KParams P, int round) {
     int f;
     const long sk = amb_slot(F, P, w, f);
     if (sk < 0) continue;
+    if (kLast) {
+      const int k = (int)(w % amb_per(P));
+      if (k < P.inner_rows) {
+        const int c = F.ft_assigned[sk];
+        float4* m = F.ft_meas + (long)f * kMaxRows + k;
+        if (c < 0) {
+          m->w = __uint_as_float(__float_as_uint(m->w) & ~kStHave);
+        } else if (c != F.ft_st_cl[(long)f * kMaxRows + k]) {
+          const int rs = F.ft_st_rs[(long)f * kMaxRows + k];
+          const float2 pc = F.syz[c];
+          *m = fit_meas<kMap>(M, P, rs, F.row_x[rs % P.n_rows], pc.x,
+                              track_z(pc.y, rs / P.n_rows, shift_side(F, f), F.ft_zsh[f], P),
+                              F.ft_z0[f]);
+        }
+      }
+    }
     if (F.ft_ncand[sk] <= round) continue;
     const int c = F.ft_cand[sk * kMaxCand + round];
     if (F.ft_newly[sk]) F.taken[c] = 1;
@@ -1623,8 +1726,10 @@ __global__ void k_amb_mark(FrameDev F, KParams P, int round) {
   }
 }
 
-// Iteration 3: inward with the surviving and re-attached clusters, simple cut.
-template <bool kMap, int kPart>
+// Iteration 3: inward with the surviving and re-attached clusters (as the
+// station records hold them after iteration 2 and the second ambiguity
+// solving), simple cut.
+template <bool kMap, bool kExt, int kPart>
 __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     k_fit3(FrameDev F, KParams P, MapDev M) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
@@ -1643,8 +1748,7 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     if (!F.ft_ok[f]) continue;
     const int ns = F.ft_nst[f];
     const int* SC = F.ft_st_cl + (long)f * kMaxRows;
-    const uint16_t* SR = F.ft_st_rs + (long)f * kMaxRows;
-    const uint8_t* flag = F.ft_flag + (long)f * kMaxRows;
+    const float4* SM = F.ft_meas + (long)f * kMaxRows;
     int* used = F.ft_used + (long)f * kMaxRows;
     const float z0 = F.ft_z0[f];
     const float zsh = F.ft_zsh[f];
@@ -1652,8 +1756,9 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     Trk<float> s2;
     const float* e2 = F.ft_end2 + (long)f * kStateF;
     get_state(e2, s2);
+    float4 nxt = SM[ns - 1];
     Lin L;
-    lin_start(L, s2, SR[ns - 1] / NR, P);
+    lin_start(L, s2, st_sector(nxt), P);
     float chi2 = 0.0f;
     int n = 0;
     Trk<float> out = L.t;
@@ -1663,10 +1768,9 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
     // against a forward extrapolation of the iteration-2 end state (its own
     // covariance), so that it joins the track without moving the fit of the
     // stations; in the list the outward clusters precede the stations
-    const int nout = P.ext_rows > 0 ? F.ft_nout[f] : 0;
-    if (nout > 0) {
-      const int rsl = SR[ns - 1];
-      const int secl = rsl / NR, rl = rsl % NR;
+    const int nout = kExt ? F.ft_nout[f] : 0;
+    if (kExt && nout > 0) {
+      const int secl = st_sector(nxt), rl = st_row(nxt);
       Lin E;
       E.t = s2;
 #pragma unroll
@@ -1698,34 +1802,35 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
       }
     }
     // the stations inward, then the rows extrapolated below the innermost one
-    const int next = P.ext_rows > 0 ? F.ft_next[f] : 0;
-    const int rs0 = SR[0];
+    const int next = kExt ? F.ft_next[f] : 0;
     for (int k = ns - 1; k >= -next; --k) {
-      // the station's cluster is requested before the station change (it
-      // does not depend on the state); inner stations hold at most
-      // inner_rows <= kMaxInner entries, as rows increase along a track
+      // the station's record is requested one step ahead, its cluster's index
+      // before the station change; inner stations hold at most inner_rows <=
+      // kMaxInner entries, as rows increase along a track
       int sec, row, c;
-      if (k >= 0) {
-        const int rs = SR[k];
-        sec = rs / NR;
-        row = rs % NR;
-        const bool inner = row < P.inner_rows;
-        c = inner ? F.ft_assigned[(long)f * F.nslot + k] : (flag[k] ? -1 : SC[k]);
-      } else {
+      float4 m = nxt;
+      if (!kExt || k >= 0) {
+        if (k > 0) nxt = SM[k - 1];
+        sec = st_sector(m);
+        row = st_row(m);
+        c = -1;
+        if (st_have(m)) c = row < P.inner_rows ? F.ft_assigned[(long)f * F.nslot + k] : SC[k];
+      } else {  // nxt: the innermost station
         sec = F.ft_ext_sec[(long)f * 2 * P.ext_rows - 1 - k];
-        row = rs0 % NR + k;
+        row = st_row(nxt) + k;
         c = F.ft_assigned[(long)f * F.nslot + kMaxInner - 1 - k];
-      }
-      float cy = 0.0f, cz = 0.0f;
-      if (c >= 0) {
-        const float2 pc = F.syz[c];
-        cy = pc.x;
-        cz = track_z(pc.y, sec, zside, zsh, P);
+        if (c >= 0) {
+          const float2 pc = F.syz[c];
+          m = fit_meas<kMap>(M, P, sec * NR + row, rx[row], pc.x,
+                             track_z(pc.y, sec, zside, zsh, P), z0);
+        } else {
+          m.w = 0.0f;
+        }
       }
       if (k != ns - 1 && !lin_goto(L, sec, rx[row], P)) break;
-      if (c < 0) continue;
+      if (!st_have(m)) continue;
       float my, mz;
-      if (!corrected(M, P, sec, L.t.x, cy, cz, z0, L.r, my, mz)) continue;
+      if (!meas_at<kMap>(m, P, L.r, my, mz)) continue;
       const Resid R = residual(L.t, my, mz, P);
       if (R.chi2 > P.final_chi2) continue;
       chi2 = chi2 + R.chi2;
@@ -2306,23 +2411,29 @@ int stage_merge(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   return k + 10;
 }
 
-int stage_fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
-  k_fit_stations<<<sms * 8, kBlock, 0, s>>>(F, P);
+// The fit kernels' variants: with a correction map or without, with the Phase
+// III rows or without (the common form carries neither's code nor registers).
+template <bool kMap>
+int fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const unsigned g = persistent_grid(F.lc, kLFit12, sms);
   const int b = F.lc.block[kLFit12];
+  k_fit_stations<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
   // iterations 1 and 2 keep loopers and other tracks in one launch (split in
   // two parts, as iteration 3 is, they measured slower: 22.4 -> 25.1 ms per
   // batch, the two kinds of track no longer sharing the warps)
-  if (F.map.on) {
-    k_fit1<true, 0><<<g, b, 0, s>>>(F, P, F.map);
-    k_fit2<true, 0><<<g, b, 0, s>>>(F, P, F.map);
-    k_inner_cand<true><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
+  if (P.ext_rows > 0) {
+    k_fit1<kMap, true><<<g, b, 0, s>>>(F, P, F.map);
+    k_fit2<kMap, true><<<g, b, 0, s>>>(F, P, F.map);
   } else {
-    k_fit1<false, 0><<<g, b, 0, s>>>(F, P, F.map);
-    k_fit2<false, 0><<<g, b, 0, s>>>(F, P, F.map);
-    k_inner_cand<false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
+    k_fit1<kMap, false><<<g, b, 0, s>>>(F, P, F.map);
+    k_fit2<kMap, false><<<g, b, 0, s>>>(F, P, F.map);
   }
+  k_inner_cand<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
   return 4;  // the station lists, iterations 1 and 2, the candidate search
+}
+
+int stage_fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+  return F.map.on ? fit12<true>(F, P, sms, s) : fit12<false>(F, P, sms, s);
 }
 
 int stage_ambiguity2(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
@@ -2330,22 +2441,32 @@ int stage_ambiguity2(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   for (int r = 0; r < P.cand_k; ++r) {
     k_amb_bid<<<sms * 8, kBlock, 0, s>>>(F, P, r);
     k_amb_resolve<<<sms * 8, kBlock, 0, s>>>(F, P, r);
-    k_amb_mark<<<sms * 8, kBlock, 0, s>>>(F, P, r);
+    if (r + 1 < P.cand_k) k_amb_mark<false, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
+    else if (F.map.on) k_amb_mark<true, true><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
+    else k_amb_mark<true, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
     k += 3;
   }
   return k;
 }
 
-int stage_fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+template <bool kMap, bool kExt>
+int fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const unsigned g = persistent_grid(F.lc, kLFit3, sms);
   const int b = F.lc.block[kLFit3];
-  if (F.map.on) {
-    k_fit3<true, 0><<<g, b, 0, s>>>(F, P, F.map);
+  if constexpr (kMap && kExt) {
+    k_fit3<kMap, kExt, 0><<<g, b, 0, s>>>(F, P, F.map);
     return 1;
+  } else {
+    k_fit3<kMap, kExt, 1><<<g, b, 0, s>>>(F, P, F.map);
+    k_fit3<kMap, kExt, 2><<<g, b, 0, s>>>(F, P, F.map);
+    return 2;
   }
-  k_fit3<false, 1><<<g, b, 0, s>>>(F, P, F.map);
-  k_fit3<false, 2><<<g, b, 0, s>>>(F, P, F.map);
-  return 2;
+}
+
+int stage_fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+  if (P.ext_rows > 0)
+    return F.map.on ? fit3<true, true>(F, P, sms, s) : fit3<false, true>(F, P, sms, s);
+  return F.map.on ? fit3<true, false>(F, P, sms, s) : fit3<false, false>(F, P, sms, s);
 }
 
 int stage_output(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {

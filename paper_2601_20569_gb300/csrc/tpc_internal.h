@@ -86,6 +86,10 @@ enum : int {
   kErrCapEdge = 256, // segments of the edge following beyond the tracklet capacity
 };
 
+// Station word of a fit measurement: row in bits 0..7, batch sector in bits
+// 8..23 (sectors x rows is at most 65535), bit 31: the station holds a cluster.
+constexpr unsigned kStHave = 0x80000000u;
+
 // Largest number of clusters one search bin may hold.  Bins are sized for a
 // few clusters each; a frame that piles more than this into one bin (many
 // clusters at one point of a row) is rejected as invalid input, which keeps
@@ -225,8 +229,10 @@ struct FrameDev {
 
   // a7 sector tracks (capacity cap_tl)
   int* st_tl;              // tracklet index of each accepted tracklet
-  int* st_off;             // first entry of the track's kept-cluster positions
-  float4* st_pos;          // [cap_pos] (x, y, z, -) of kept clusters, outermost first per track
+  int* st_off;             // first entry of the track's kept-cluster positions (-1: none,
+                           // a segment found by the edge following)
+  float4* st_pos;          // [cap_pos] (x, y, z, sector*n_rows + row bits) of kept clusters,
+                           // outermost first per track
   long cap_pos;
   int* st_order;           // order in which the sector refit takes the tracks
   int* st_obucket;         // scheduling bucket
@@ -274,6 +280,8 @@ struct FrameDev {
   float* ft_z0;
   int* ft_st_cl;           // [cap_ft][kMaxRows] sorted cluster or -1
   uint16_t* ft_st_rs;      // [cap_ft][kMaxRows] sector*n_rows + row
+  float4* ft_meas;         // [cap_ft][kMaxRows] the fit's measurement at each station: (x
+                           // displacement, y, z of the corrected cluster, station word)
   float* ft_store;         // [cap_ft][kMaxRows][5] iteration-1 predictions
   uint8_t* ft_flag;        // [cap_ft][kMaxRows]
   float* ft_end2;          // [cap_ft][kStateF] end of iteration 2 (+ sector)

@@ -1458,6 +1458,7 @@ __global__ void k_edge_write(FrameDev F, KParams P) {
     F.tl_rlo[ti] = 1;  // no tracklet hits (the seeding history of the cluster removal)
     F.tl_rhi[ti] = 0;
     F.st_tl[i] = ti;
+    F.st_off[i] = -1;
     F.st_key[i] = F.st_key[j] + (inner ? (1 << 29) : (1 << 30));
     F.st_sector[i] = sec;
     const int r_a = F.srow[H[0]] % P.n_rows, r_b = F.srow[H[nh - 1]] % P.n_rows;
