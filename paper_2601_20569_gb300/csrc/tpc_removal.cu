@@ -194,26 +194,29 @@ __device__ __forceinline__ void cr_tube(const FrameDev& F, const KParams& P,
 }
 
 // Tubes of every output track and the seeding history of the physics ones.
+// A track's tube cross-sections do not depend on one another: one warp per
+// track, a lane per cluster (its own cross-section and those of the gap rows up
+// to the next cluster), then the lanes over the rows of each seeding tracklet.
+// (One thread per track, walking its clusters in turn, was bound by that serial
+// chain of window scans: 1.06 ms for the 4,600 tracks of an event.)
 __global__ void k_cr_tubes(FrameDev F, KParams P, RemovalParams R) {
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   const int NR = P.n_rows;
-  for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  for (int f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); f < nf; f += nw) {
     const int t = F.ft_outidx[f];
     if (t < 0) continue;
     const bool protect = F.cr_cls[t] == 0;
     const int n = F.ft_n[f];
     if (n <= 0) continue;
     const int* used = F.ft_used + (long)f * kMaxRows;
-    int crr = F.srow[used[0]];
-    float2 pc = F.syz[used[0]];
-    for (int i = 0; i < n; ++i) {
-      // the next cluster is requested before this one's tube is scanned
-      const int d = i + 1 < n ? used[i + 1] : -1;
-      const int drr = d >= 0 ? F.srow[d] : -1;
-      const float2 pd = d >= 0 ? F.syz[d] : make_float2(0.0f, 0.0f);
+    for (int i = lane; i < n; i += 32) {
+      const int c = used[i], d = i + 1 < n ? used[i + 1] : -1;
+      const int crr = F.srow[c], drr = d >= 0 ? F.srow[d] : -1;
+      const float2 pc = F.syz[c], pd = d >= 0 ? F.syz[d] : make_float2(0.0f, 0.0f);
       cr_tube(F, P, R, crr, pc.x, pc.y, protect);
-      if (d < 0) break;
-      if (drr / NR == crr / NR) {
+      if (d >= 0 && drr / NR == crr / NR) {
         const bool cl = crr < drr;  // interpolate from the lower-row cluster
         const int rl = (cl ? crr : drr) % NR, rh = (cl ? drr : crr) % NR;
         const float2 lo = cl ? pc : pd, hi = cl ? pd : pc;
@@ -224,14 +227,13 @@ __global__ void k_cr_tubes(FrameDev F, KParams P, RemovalParams R) {
                   protect);
         }
       }
-      crr = drr;
-      pc = pd;
     }
     if (!protect) continue;
     for (int sg = F.ft_head[f]; sg >= 0; sg = F.st_next[sg]) {
       const int ti = F.st_tl[sg];
       const int* H = F.tl_hits + (long)ti * kMaxRows;
-      for (int r = F.tl_rlo[ti]; r <= F.tl_rhi[ti]; ++r)
+      const int rhi = F.tl_rhi[ti];
+      for (int r = F.tl_rlo[ti] + lane; r <= rhi; r += 32)
         if (H[r] >= 0) atomicOr(&F.cr_flags[H[r]], 2u);
     }
   }
