@@ -299,6 +299,8 @@ __global__ void __launch_bounds__(256) k_sector_refit(FrameDev F, KParams P) {
 }
 
 // z range of each sector (from the row statistics of the grid build).
+constexpr float kMergeBinCm = 8.0f;
+
 __global__ void k_sector_zrange(FrameDev F, KParams P) {
   const int s = blockIdx.x;
   __shared__ unsigned lo, hi;
@@ -316,7 +318,8 @@ __global__ void k_sector_zrange(FrameDev F, KParams P) {
     float zl = 0.0f, zh = 1.0f;
     if (hi >= lo && hi != 0u) { zl = o2f(lo); zh = o2f(hi); }
     F.sec_zlo[s] = zl;
-    F.sec_zinv[s] = zh > zl ? (float)kMergeZ / (zh - zl) : 0.0f;
+    // (bins of at least kMergeBinCm: the search windows are 10-30 cm long)
+    F.sec_zinv[s] = zh > zl ? fminf((float)kMergeZ / (zh - zl), 1.0f / kMergeBinCm) : 0.0f;
   }
 }
 
@@ -486,6 +489,30 @@ __device__ __forceinline__ bool merge_pos(const MergeA& m, float xb, const KPara
   return true;
 }
 
+// z window of the candidates of an outer end in the frame of MergeA m, for
+// inner ends on rows with x in [x0, x1].  The full test needs B's z within
+// merge_dz of A's z at B's x.  sin(phi) is linear in x, so over the run |sin(phi)|
+// stays below its larger end value (and below fit_max_snp, beyond which the
+// test fails), and the arc from A to B lies between dx and dx / cos(phi) of that
+// value; the arc times tan(lambda) bounds the z step.  0.1 % and 0.02 cm + 1e-5
+// |z| cover the rounding of both evaluations.  Against the window the index
+// was searched with before (both signs, the steepest angle the cuts allow) it
+// is several times shorter, and so are the ranges and candidates to visit.
+__device__ __forceinline__ void merge_window(const MergeA& m, float x0, float x1, const KParams& P,
+                                             float& zlo, float& zhi) {
+  const float d0 = x0 - m.x, d1 = x1 - m.x;
+  const float s = fminf(fmaxf(fabsf(m.s0), fmaxf(fabsf(m.s0 + m.kap * d0),
+                                                 fabsf(m.s0 + m.kap * d1))),
+                        P.fit_max_snp);
+  const float rc = 1.001f * rsqrtf(1.0f - s * s);
+  const float a0 = d0 < 0.0f ? d0 * rc : d0 * 0.999f;  // shortest (most negative) arc
+  const float a1 = d1 > 0.0f ? d1 * rc : d1 * 0.999f;  // longest
+  const float e0 = m.tgl * a0, e1 = m.tgl * a1;
+  const float mg = P.merge_dz + 0.02f + 1e-5f * (fabsf(m.z) + fabsf(e0) + fabsf(e1));
+  zlo = m.z + fminf(e0, e1) - mg;
+  zhi = m.z + fmaxf(e0, e1) + mg;
+}
+
 // Best merge partner of every outer end A, searched by a group of G lanes
 // (G = 1: one thread per end).  The (sector, z bin) ranges of A's candidates
 // in the index are dealt out to the lanes, their sizes summed by a group scan,
@@ -501,21 +528,24 @@ __global__ void __launch_bounds__(256, 4) k_merge_best(FrameDev F, KParams P) {
   const int gl = lane & (G - 1);
   const unsigned gmask = G == 32 ? 0xFFFFFFFFu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int half = P.n_phi;
+  // up to kFetch ends per queue fetch: lane gl < fetch of the group looks at
+  // end base + gl; the ends with no row to search (those that reach the last
+  // rows) are answered at once, the others searched one after the other by the
+  // whole group.  (A few ends per fetch, so that the atomics stay few; one
+  // where the ends are too few to give every group several fetches, as a
+  // group's ends are a serial chain.)
+  constexpr int kFetch = G < 8 ? G : 8;
+  const int groups = (int)(gridDim.x * blockDim.x) / G;
+  const int fetch = max(1, min(kFetch, ns / (4 * groups)));
   for (;;) {
-    // kFetch ends per queue fetch: lane gl < kFetch of the group looks at
-    // end base + gl; the ends with no row to search (those that reach the
-    // last rows) are answered at once, the others searched one after the
-    // other by the whole group.  (A few ends per fetch: the atomics stay
-    // few, and the last fetches of the grid stay short.)
-    constexpr int kFetch = G < 8 ? G : 8;
     int base = 0;
-    if (gl == 0) base = queue_next_n(&F.cnt->queue[kQMerge], kFetch);
+    if (gl == 0) base = queue_next_n(&F.cnt->queue[kQMerge], fetch);
     base = __shfl_sync(gmask, base, 0, G);
     if (base >= ns) break;
     const int am = base + gl;
     bool live = false;
     // (an outer end linked by the edge following is not searched)
-    if (gl < kFetch && am < ns && F.st_ok[am] && F.st_next[am] < 0) {
+    if (gl < fetch && am < ns && F.st_ok[am] && F.st_next[am] < 0) {
       const int rmx = F.st_rmax[am];
       live = rmx + 1 <= min(rmx + P.merge_max_gap, P.n_rows - 1);
       if (!live) {
@@ -528,92 +558,108 @@ __global__ void __launch_bounds__(256, 4) k_merge_best(FrameDev F, KParams P) {
       const int keyA = F.st_key[a];
       unsigned long long best = ~0ull;
       int bb = -1;
+      // the pair test needs 1 <= rmin(B) - rmax(A) <= merge_max_gap: only
+      // those rows of the index are visited
       const int r0 = F.st_rmax[a] + 1;
       const int r1 = min(F.st_rmax[a] + P.merge_max_gap, P.n_rows - 1);
-      {
-        // the pair test needs 1 <= rmin(B) - rmax(A) <= merge_max_gap: only
-        // those rows of the index are visited
-        const int sa = F.st_sector[a];
-        const int side = sa / half, ph = sa % half;
-        const float* oe = F.st_oe + (long)a * kStateF;
-        const float zwin = P.merge_dz + fabsf(oe[3]) * P.merge_zspan;
-        const float m = 0.01f;
-        int sq[3], zq[3], nq[3];
-        int nr = 0;
+      const float x0 = F.row_x[r0], x1 = F.row_x[r1];
+      const int sa = F.st_sector[a];
+      const int side = sa / half, ph = sa % half;
+      const float* oe = F.st_oe + (long)a * kStateF;
+      const float zwin = P.merge_dz + fabsf(oe[3]) * P.merge_zspan;
+      const float oz = oe[1];
+      // A's state and z bins in the three sectors: lanes 0-2 of the group hold
+      // one sector each and hand it to the lanes by shuffles (with fewer lanes
+      // every lane computes the three); no bins where A cannot be turned into
+      // the sector, as the test fails there
+      MergeA ma{};
+      int sq[3], zq[3], nq[3];
+      int nr = 0;
+      int my_s = 0, my_z = 0, my_n = 0;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          sq[q] = side * half + (ph + (q == 0 ? 0 : q == 1 ? 1 : half - 1)) % half;
-          zq[q] = merge_zbin(F, sq[q], oe[1] - zwin - m);
-          nq[q] = merge_zbin(F, sq[q], oe[1] + zwin + m) - zq[q] + 1;
-          nr += nq[q];
+      for (int q = 0; q < 3; ++q) {
+        if (G < 4 || gl == q) {
+          ma = merge_a(oe, q, P);
+          my_s = side * half + (ph + (q == 0 ? 0 : q == 1 ? 1 : half - 1)) % half;
+          float zlo, zhi;
+          merge_window(ma, x0, x1, P, zlo, zhi);
+          zlo = fmaxf(zlo, oz - zwin - 0.01f);
+          zhi = fminf(zhi, oz + zwin + 0.01f);
+          my_z = merge_zbin(F, my_s, zlo);
+          my_n = ma.ok && zlo <= zhi ? merge_zbin(F, my_s, zhi) - my_z + 1 : 0;
         }
-        // A's state in the three sectors: lanes 0-2 of the group hold one
-        // each and hand it to the lanes by shuffles (one lane computes it
-        // where it needs it)
-        MergeA ma{};
-        if (G >= 4 && gl < 3) ma = merge_a(oe, gl, P);
-        const float oz = oe[1];
-        for (int j0 = 0; j0 < nr; j0 += G) {
-          int lo = 0, cnt = 0, qj = 0;
-          int j = j0 + gl;
-          if (j < nr) {
-            const int q = j < nq[0] ? 0 : j < nq[0] + nq[1] ? 1 : 2;
-            j -= q == 0 ? 0 : q == 1 ? nq[0] : nq[0] + nq[1];
-            const int base = (sq[q] * kMergeZ + zq[q] + j) * P.n_rows;
-            lo = F.ie_first[base + r0];
-            cnt = F.ie_first[base + r1 + 1] - lo;
-            qj = q;
-          }
-          int inc = cnt;  // inclusive scan of the range sizes over the group
+        if (G < 4) {
+          sq[q] = my_s;
+          zq[q] = my_z;
+          nq[q] = my_n;
+        } else {
+          sq[q] = __shfl_sync(gmask, my_s, q, G);
+          zq[q] = __shfl_sync(gmask, my_z, q, G);
+          nq[q] = __shfl_sync(gmask, my_n, q, G);
+        }
+        nr += nq[q];
+      }
+      for (int j0 = 0; j0 < nr; j0 += G) {
+        int lo = 0, cnt = 0, qj = 0;
+        int j = j0 + gl;
+        if (j < nr) {
+          const int q = j < nq[0] ? 0 : j < nq[0] + nq[1] ? 1 : 2;
+          j -= q == 0 ? 0 : q == 1 ? nq[0] : nq[0] + nq[1];
+          const int base = ((q == 0 ? sq[0] : q == 1 ? sq[1] : sq[2]) * kMergeZ +
+                            (q == 0 ? zq[0] : q == 1 ? zq[1] : zq[2]) + j) * P.n_rows;
+          lo = F.ie_first[base + r0];
+          cnt = F.ie_first[base + r1 + 1] - lo;
+          qj = q;
+        }
+        int inc = cnt;  // inclusive scan of the range sizes over the group
 #pragma unroll
-          for (int o = 1; o < G; o <<= 1) {
-            const int v = __shfl_up_sync(gmask, inc, o, G);
-            if (gl >= o) inc += v;
-          }
-          const int total = __shfl_sync(gmask, inc, G - 1, G);
-          for (int c0 = 0; c0 < total; c0 += G) {
-            const int c = c0 + gl;
-            int L = 0;  // the range holding candidate c: first lane with inc > c
+        for (int o = 1; o < G; o <<= 1) {
+          const int v = __shfl_up_sync(gmask, inc, o, G);
+          if (gl >= o) inc += v;
+        }
+        const int total = __shfl_sync(gmask, inc, G - 1, G);
+        for (int c0 = 0; c0 < total; c0 += G) {
+          const int c = c0 + gl;
+          int L = 0;  // the range holding candidate c: first lane with inc > c
 #pragma unroll
-            for (int st = G / 2; st >= 1; st >>= 1) {
-              const int v = __shfl_sync(gmask, inc, L + st - 1, G);
-              if (v <= c) L += st;
-            }
-            const int excl = __shfl_sync(gmask, inc - cnt, L, G);
-            const int lo_l = __shfl_sync(gmask, lo, L, G);
-            const int q_l = __shfl_sync(gmask, qj, L, G);
-            MergeA mq;
-            if (G >= 4) {
-              mq.y = __shfl_sync(gmask, ma.y, q_l, G);
-              mq.z = __shfl_sync(gmask, ma.z, q_l, G);
-              mq.s0 = __shfl_sync(gmask, ma.s0, q_l, G);
-              mq.c0 = __shfl_sync(gmask, ma.c0, q_l, G);
-              mq.kap = __shfl_sync(gmask, ma.kap, q_l, G);
-              mq.tgl = __shfl_sync(gmask, ma.tgl, q_l, G);
-              mq.x = __shfl_sync(gmask, ma.x, q_l, G);
-              mq.ok = __shfl_sync(gmask, ma.ok, q_l, G);
-            }
-            if (c >= total) continue;
-            // the indexed inner end: (y, z, x, track)
-            const float4 rec = F.ie_rec[lo_l + (c - excl)];
-            if (!(fabsf(rec.y - oz) <= zwin)) continue;  // the full test's z window
-            if (G < 4) mq = merge_a(oe, q_l, P);
-            float yb, zb;
-            if (merge_pos(mq, rec.z, P, yb, zb) &&
-                (fabsf(rec.x - yb) > P.merge_dy + 0.01f + 1e-5f * fabsf(rec.x) ||
-                 fabsf(rec.y - zb) > P.merge_dz + 0.01f + 1e-5f * fabsf(rec.y)))
-              continue;
-            const int b = __float_as_int(rec.w);
-            if (b == a || !F.st_ok[b]) continue;
-            float chi2;
-            if (!merge_test(F, P, a, b, chi2)) continue;
-            const unsigned long long kb = pack_chi_key(chi2, F.st_key[b]);
-            if (kb < best) {
-              best = kb;
-              bb = b;
-            }
-            atomicMin(&F.st_bestA[b], pack_chi_key(chi2, keyA));
+          for (int st = G / 2; st >= 1; st >>= 1) {
+            const int v = __shfl_sync(gmask, inc, L + st - 1, G);
+            if (v <= c) L += st;
           }
+          const int excl = __shfl_sync(gmask, inc - cnt, L, G);
+          const int lo_l = __shfl_sync(gmask, lo, L, G);
+          const int q_l = __shfl_sync(gmask, qj, L, G);
+          MergeA mq;
+          if (G >= 4) {
+            mq.y = __shfl_sync(gmask, ma.y, q_l, G);
+            mq.z = __shfl_sync(gmask, ma.z, q_l, G);
+            mq.s0 = __shfl_sync(gmask, ma.s0, q_l, G);
+            mq.c0 = __shfl_sync(gmask, ma.c0, q_l, G);
+            mq.kap = __shfl_sync(gmask, ma.kap, q_l, G);
+            mq.tgl = __shfl_sync(gmask, ma.tgl, q_l, G);
+            mq.x = __shfl_sync(gmask, ma.x, q_l, G);
+            mq.ok = __shfl_sync(gmask, ma.ok, q_l, G);
+          }
+          if (c >= total) continue;
+          // the indexed inner end: (y, z, x, track)
+          const float4 rec = F.ie_rec[lo_l + (c - excl)];
+          if (!(fabsf(rec.y - oz) <= zwin)) continue;  // the full test's z window
+          if (G < 4) mq = merge_a(oe, q_l, P);
+          float yb, zb;
+          if (merge_pos(mq, rec.z, P, yb, zb) &&
+              (fabsf(rec.x - yb) > P.merge_dy + 0.01f + 1e-5f * fabsf(rec.x) ||
+               fabsf(rec.y - zb) > P.merge_dz + 0.01f + 1e-5f * fabsf(rec.y)))
+            continue;
+          const int b = __float_as_int(rec.w);
+          if (b == a || !F.st_ok[b]) continue;
+          float chi2;
+          if (!merge_test(F, P, a, b, chi2)) continue;
+          const unsigned long long kb = pack_chi_key(chi2, F.st_key[b]);
+          if (kb < best) {
+            best = kb;
+            bb = b;
+          }
+          atomicMin(&F.st_bestA[b], pack_chi_key(chi2, keyA));
         }
       }
 #pragma unroll
