@@ -777,7 +777,9 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
     bool ok = true;
     ok &= dalloc(ctx, &R.ref, T * 10);
     ok &= dalloc(ctx, &R.flag, NR);
-    ok &= dalloc(ctx, &R.zref, NR);
+    ok &= dalloc(ctx, &R.raw, NR);
+    ok &= dalloc(ctx, &R.meas, NR);
+    ok &= dalloc(ctx, &R.queue, kRefitQueues);
     ok &= dalloc(ctx, &R.acc, NR);
     ok &= dalloc(ctx, &R.z0, T);
     ok &= dalloc(ctx, &R.ckpt, T * 3 * kCkptSeg * kCkptF);
@@ -790,7 +792,6 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
     ok &= dalloc(ctx, &R.out_par, T * 5);
     ok &= dalloc(ctx, &R.out_cov, T * 15);
     ok &= dalloc(ctx, &R.out_x, T);
-    ok &= dalloc(ctx, &R.dD, NR * 3);
     ok &= dalloc(ctx, &ctx->steps3, T);
     if (!ok) return fail(ctx, TPC_ERR_OOM, "refit buffers");
     R.cap = T;
@@ -813,6 +814,7 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
   R.row_x = F.row_x;
   R.freeze = freeze ? 1 : 0;
   R.map = make_mapdev(mp);
+  CK(cudaMemsetAsync(R.queue, 0, sizeof(int) * kRefitQueues, s));
   const int k = ctx->opt.mode == 0 ? strict::refit_forward(R, ctx->P, ctx->steps3, ctx->sms, s)
                                    : fast::refit_forward(R, ctx->P, ctx->steps3, ctx->sms, s);
   ctx->launches_last = k;
@@ -857,6 +859,11 @@ tpc_status tpc_refit_backward(tpc_ctx* ctx, const float* dl_dchi2, float* dl_dma
                 ncoef);
   R.ncoef = (int)ncoef;
   R.gblocks = ctx->sms;
+  R.smem_max = smem_max;
+  if (!R.rec) {
+    const long tracks = R.cap < (long)kAdjChunk ? R.cap : (long)kAdjChunk;
+    if (!dalloc(ctx, &R.rec, tracks * 3 * kMaxRows * kRecV)) return fail(ctx, TPC_ERR_OOM, "adjoint records");
+  }
   if ((long)R.gblocks * ncoef > ctx->gpart_cap) {
     if (!dalloc(ctx, &R.gpart, (long)R.gblocks * ncoef)) return fail(ctx, TPC_ERR_OOM, "gradient partials");
     ctx->gpart_cap = (long)R.gblocks * ncoef;

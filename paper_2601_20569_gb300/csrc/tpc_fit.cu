@@ -47,6 +47,18 @@ struct SplinePt {
   float wp[4], wr[4], wz[4];
 };
 
+// x^2 + y^2 of a map point.  Strict mode rounds every operation; fast mode fuses
+// one product into the sum.  The refit states which one (kXFirst), so that its
+// values do not hang on the order in which the compiler meets the products.
+template <bool kXFirst>
+__device__ __forceinline__ float square_sum(float x, float y) {
+#ifdef TPC_FAST_ARITH
+  if (kXFirst) return __fmaf_rn(x, x, __fmul_rn(y, y));
+#endif
+  return x * x + y * y;
+}
+
+template <bool kXFirst = false>
 __device__ __forceinline__ SplinePt spline_point(const MapDev& M, const KParams& P, int sector,
                                                  float x, float y, float zdrift) {
   SplinePt sp;
@@ -55,7 +67,7 @@ __device__ __forceinline__ SplinePt spline_point(const MapDev& M, const KParams&
   const float tp = u * M.phi_scale - 0.5f;
   sp.ip = (int)floorf(tp);
   const float fp = tp - (float)sp.ip;
-  const float r = sqrtf(x * x + y * y);
+  const float r = sqrtf(square_sum<kXFirst>(x, y));
   float fr, fz;
   spline_span((r - M.rmin) * M.r_scale, M.nr, sp.ir, fr);
   float zc = zdrift;
@@ -72,11 +84,12 @@ __device__ __forceinline__ int phi_index(int ip, int e, int nphi) {
   return ((ip - 1 + e) % nphi + nphi) % nphi;
 }
 
+template <bool kXFirst = false>
 __device__ __forceinline__ void map_eval(const MapDev& M, const KParams& P, int sector, float x,
                                          float y, float zdrift, float* D) {
   D[0] = D[1] = D[2] = 0.0f;
   if (!M.on) return;
-  const SplinePt sp = spline_point(M, P, sector, x, y, zdrift);
+  const SplinePt sp = spline_point<kXFirst>(M, P, sector, x, y, zdrift);
   int pidx[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) pidx[e] = phi_index(sp.ip, e, M.nphi);
@@ -1077,9 +1090,12 @@ __device__ __forceinline__ Interp interpolate(const float* a, const float* b) {
 
 __device__ __forceinline__ float chi2_interp(const Interp& I, float my, float mz,
                                              const KParams& P) {
+  // (explicitly rounded: fused with the products they come from or not, as the
+  // compiler finds them in one basic block or in two, these would let the cut's
+  // decision depend on the kernel that evaluates it)
   float w00, w01, w11;
-  inv2(I.c00 + P.sy2, I.c01, I.c11 + P.sz2, w00, w01, w11);
-  const float r0 = my - I.y, r1 = mz - I.z;
+  inv2(__fadd_rn(I.c00, P.sy2), I.c01, __fadd_rn(I.c11, P.sz2), w00, w01, w11);
+  const float r0 = __fsub_rn(my, I.y), r1 = __fsub_rn(mz, I.z);
   return r0 * (w00 * r0 + w01 * r1) + r1 * (w01 * r0 + w11 * r1);
 }
 
@@ -2088,127 +2104,236 @@ __device__ __forceinline__ void lin_start2(Lin& L, const Trk<float>& s, const fl
 
 // Forward refit (see the oracle's definition): extended-Kalman start pass on
 // uncorrected clusters, then iterations 1-3 with checkpoints of the filter
-// (state, covariance, reference) every kCkptStride stations.
-__global__ void __launch_bounds__(128) k_refit(RefitDev R, KParams P, int* steps3) {
+// (state, covariance, reference) every kCkptStride stations.  First, one warp
+// per track, the lanes over its clusters: each reference's position in the
+// frame of the track's innermost side and its correction, which depend on no
+// filter state and would otherwise be evaluated in every pass on the serial
+// chain of the track's steps.  Then four kernels, one per pass, each a
+// per-lane state machine (a step per loop iteration, refilled from a work
+// queue), each leaving the next one's start in that pass's first checkpoint.
+// (As one kernel of four loops per track the lanes of a warp did not reconverge:
+// 4.9 ms for the 3,900 tracks of an event in strict mode.)
+// R.ok counts the passes done: a pass takes a track only if the one before it
+// succeeded.
+__global__ void __launch_bounds__(256, 2) k_refit_prep(RefitDev R, KParams P, int* steps3) {
   const MapDev M = R.map;
-  const int half = P.n_phi;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < R.n_tracks;
-       t += gridDim.x * blockDim.x) {
-    R.ok[t] = 0;
-    R.nused[t] = 0;
-    R.chi2[t] = 0.0f;
-    steps3[t] = 0;
+  const int lane = threadIdx.x & 31;
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < R.n_tracks; t += nw) {
     const int o0 = R.offset[t], ns = R.offset[t + 1] - o0;
-    if (ns < 1 || ns > kMaxRows) continue;
-    const int* ids = R.ids + o0;
-    float ip[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) ip[i] = R.in_par[(long)t * 5 + i];
+    const float* ip = R.in_par + (long)t * 5;
     const float inx = R.in_x[t];
     const float z0 = ip[1] - ip[3] * sqrtf(inx * inx + ip[0] * ip[0]);
-    R.z0[t] = z0;
-    float* zr = R.zref + o0;  // each cluster's z in the innermost side's frame
-    {
-      float zsh;
-      int zside;
-      refit_shift(R, P, t, zsh, zside);
-      for (int k = 0; k < ns; ++k) zr[k] = track_z(R.z[ids[k]], R.sector[ids[k]], zside, zsh, P);
+    if (lane == 0) {
+      R.ok[t] = 0;
+      R.nused[t] = 0;
+      R.chi2[t] = 0.0f;
+      steps3[t] = 0;
+      R.z0[t] = z0;
     }
-    Trk<float> t0;
+    if (ns < 1 || ns > kMaxRows) continue;
+    float zsh;
+    int zside;
+    refit_shift(R, P, t, zsh, zside);
+    for (int k = lane; k < ns; k += 32) {
+      const int c = R.ids[o0 + k];
+      const int s = R.sector[c], row = R.row[c];
+      const float y = R.y[c], z = track_z(R.z[c], s, zside, zsh, P);
+      float4 m = make_float4(0.0f, y, z, __int_as_float(s << 8 | row));
+      if (M.on) {
+        float D[3];
+        map_eval<true>(M, P, s, R.row_x[row], y, z - z0, D);
+        m.x = D[0];
+        m.y = y + D[1];
+        m.z = z + D[2];
+      }
+      R.raw[o0 + k] = make_float2(y, z);
+      R.meas[o0 + k] = m;
+    }
+  }
+}
+
+__device__ __forceinline__ float* refit_ckpt(const RefitDev& R, int t, int it, int seg) {
+  return R.ckpt + (((long)t * 3 + it) * kCkptSeg + seg) * kCkptF;
+}
+
+__global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P) {
+  __shared__ float rx[kMaxRows];
+  for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = R.row_x[r];
+  __syncthreads();
+  const int half = P.n_phi;
+  bool busy = false;
+  int t = 0, k = 0, ns = 0, sec = 0;
+  const float2* raw = nullptr;
+  const float4* meas = nullptr;
+  float2 nyz = make_float2(0.0f, 0.0f);
+  int nw = 0;
+  Trk<float> t0;
+  for (;;) {
+    if (!busy) {
+      t = queue_next(&R.queue[0]);
+      if (t >= R.n_tracks) break;
+      const int o0 = R.offset[t];
+      ns = R.offset[t + 1] - o0;
+      if (ns < 1 || ns > kMaxRows) continue;
+      raw = R.raw + o0;
+      meas = R.meas + o0;
+      nyz = raw[0];
+      nw = __float_as_int(meas[0].w);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) t0.p[i] = ip[i];
-    t0.x = inx;
-    reset_cov(t0.c, P);
-    int sec = R.in_sector[t];
+      for (int i = 0; i < 5; ++i) t0.p[i] = R.in_par[(long)t * 5 + i];
+      t0.x = R.in_x[t];
+      reset_cov(t0.c, P);
+      sec = R.in_sector[t];
+      k = 0;
+      busy = true;
+      continue;
+    }
+    const float2 yz = nyz;
+    const int s = nw >> 8, row = nw & 0xFF;
+    if (k + 1 < ns) {
+      nyz = raw[k + 1];
+      nw = __float_as_int(meas[k + 1].w);
+    }
     bool ok = true;
-    for (int k = 0; k < ns && ok; ++k) {
-      const int c = ids[k];
-      const int s = R.sector[c];
-      if (s != sec) {
-        const int ds = ((s % half) - (sec % half) + half) % half;
-        // ds == 0: the same azimuthal sector across the central electrode
-        if ((ds != 0 && ds != 1 && ds != half - 1) ||
-            (ds != 0 && !rotate(t0, ds == 1 ? 1 : -1, P, P.fit_max_snp))) {
-          ok = false;
-          break;
-        }
-        sec = s;
-      }
-      if (!propagate(t0, R.row_x[R.row[c]], P, P.fit_max_snp)) { ok = false; break; }
-      update(t0, residual(t0, R.y[c], zr[k], P));
+    if (s != sec) {
+      const int ds = ((s % half) - (sec % half) + half) % half;
+      // ds == 0: the same azimuthal sector across the central electrode
+      if ((ds != 0 && ds != 1 && ds != half - 1) ||
+          (ds != 0 && !rotate(t0, ds == 1 ? 1 : -1, P, P.fit_max_snp)))
+        ok = false;
+      sec = s;
     }
-    if (!ok) continue;
-    float* store = R.store + (long)t * kMaxRows * 5;
-    float* ck = R.ckpt + (long)t * 3 * kCkptSeg * kCkptF;
-    float* ref = R.ref + (long)t * 10;
-    uint8_t* flag = R.flag + o0;
-    uint8_t* acc = R.acc + o0;
+    if (ok) ok = propagate(t0, rx[row], P, P.fit_max_snp);
+    if (!ok) {
+      busy = false;
+      continue;
+    }
+    update(t0, residual(t0, yz.x, yz.y, P));
+    if (++k < ns) continue;
     Lin L;
-    lin_start(L, t0, R.sector[ids[ns - 1]], P);
-    for (int j = 0; j < ns && ok; ++j) {  // iteration 1: inward
-      const int k = ns - 1 - j, c = ids[k];
-      if (j % kCkptStride == 0) save_ckpt(ck + (0 * kCkptSeg + j / kCkptStride) * kCkptF, L);
-      if (j != 0 && !lin_goto(L, R.sector[c], R.row_x[R.row[c]], P)) { ok = false; break; }
-      float* sv = store + k * 5;
-      sv[0] = L.t.p[0]; sv[1] = L.t.p[1]; sv[2] = L.t.c[0]; sv[3] = L.t.c[1]; sv[4] = L.t.c[2];
-      float my, mz;
-      if (!corrected(M, P, R.sector[c], L.t.x, R.y[c], zr[k], z0, L.r, my, mz)) {
-        ok = false;
-        break;
+    lin_start(L, t0, s, P);
+    save_ckpt(refit_ckpt(R, t, 0, 0), L);
+    R.ok[t] = 1;
+    busy = false;
+  }
+}
+
+// Iteration IT of the refit (0: inward, 1: outward with the interpolation
+// flags, 2: inward with the cuts).
+template <int IT, bool kMap>
+__global__ void __launch_bounds__(128, 4) k_refit_iter(RefitDev R, KParams P, int* steps3) {
+  __shared__ float rx[kMaxRows];
+  for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = R.row_x[r];
+  __syncthreads();
+  bool busy = false;
+  int t = 0, j = 0, ns = 0, o0 = 0, n = 0, out_sec = 0;
+  const float4* meas = nullptr;
+  float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float* store = nullptr;
+  float sn[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // the next station's prediction
+  float chi2 = 0.0f;
+  Lin L;
+  Trk<float> out;  // the state after the last cluster used
+  for (;;) {
+    if (!busy) {
+      t = queue_next(&R.queue[1 + IT]);
+      if (t >= R.n_tracks) break;
+      if (R.ok[t] != IT + 1) continue;
+      o0 = R.offset[t];
+      ns = R.offset[t + 1] - o0;
+      meas = R.meas + o0;
+      store = R.store + (long)t * kMaxRows * 5;
+      nxt = meas[IT == 1 ? 0 : ns - 1];
+      if (IT == 1) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) sn[i] = store[i];
       }
-      fit_update(L.t, residual(L.t, my, mz, P), P);
-    }
-    if (!ok) continue;
-    {
-      const Trk<float> s1 = L.t;
-      if (!R.freeze)
-        for (int i = 0; i < 5; ++i) ref[i] = s1.p[i];
-      lin_start2(L, s1, ref, R.sector[ids[0]], P);
-    }
-    for (int j = 0; j < ns && ok; ++j) {  // iteration 2: outward
-      const int k = j, c = ids[k];
-      if (j % kCkptStride == 0) save_ckpt(ck + (1 * kCkptSeg + j / kCkptStride) * kCkptF, L);
-      if (j != 0 && !lin_goto(L, R.sector[c], R.row_x[R.row[c]], P)) { ok = false; break; }
-      const float a[5] = {L.t.p[0], L.t.p[1], L.t.c[0], L.t.c[1], L.t.c[2]};
-      const Interp I = interpolate(a, store + k * 5);
-      float my, mz;
-      if (!corrected(M, P, R.sector[c], L.t.x, R.y[c], zr[k], z0, L.r, my, mz)) {
-        ok = false;
-        break;
+      load_ckpt(refit_ckpt(R, t, IT, 0), L);
+      if (IT == 2) {
+        chi2 = 0.0f;
+        n = 0;
+        out = L.t;
+        out_sec = L.sector;
       }
-      if (!R.freeze) flag[k] = chi2_interp(I, my, mz, P) > P.int_chi2 ? 1 : 0;
-      fit_update(L.t, residual(L.t, my, mz, P), P);
+      j = 0;
+      busy = true;
+      continue;
     }
-    if (!ok) continue;
-    {
-      const Trk<float> s2 = L.t;
-      if (!R.freeze)
-        for (int i = 0; i < 5; ++i) ref[5 + i] = s2.p[i];
-      lin_start2(L, s2, ref + 5, R.sector[ids[ns - 1]], P);
+    const int k = IT == 1 ? j : ns - 1 - j;
+    const float4 m = nxt;
+    const int w = __float_as_int(m.w);
+    float sv[5];
+    if (IT == 1) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) sv[i] = sn[i];
     }
-    float chi2 = 0.0f;
-    int n = 0;
-    Trk<float> out = L.t;
-    int out_sec = L.sector;
-    int j = 0;
-    for (; j < ns; ++j) {  // iteration 3: inward
-      const int k = ns - 1 - j, c = ids[k];
-      if (j % kCkptStride == 0) save_ckpt(ck + (2 * kCkptSeg + j / kCkptStride) * kCkptF, L);
-      if (j != 0 && !lin_goto(L, R.sector[c], R.row_x[R.row[c]], P)) break;
-      if (flag[k]) continue;
-      float my, mz;
-      if (!corrected(M, P, R.sector[c], L.t.x, R.y[c], zr[k], z0, L.r, my, mz))
+    bool skip = false, keep = false;
+    if (IT == 2) {
+      skip = R.flag[o0 + k] != 0;
+      if (R.freeze) keep = R.acc[o0 + k] != 0;
+    }
+    if (j + 1 < ns) {
+      nxt = meas[IT == 1 ? k + 1 : k - 1];
+      if (IT == 1) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) sn[i] = store[(k + 1) * 5 + i];
+      }
+    }
+    if (j > 0 && j % kCkptStride == 0) save_ckpt(refit_ckpt(R, t, IT, j / kCkptStride), L);
+    bool ok = true;
+    if (j != 0) ok = lin_goto(L, w >> 8, rx[w & 0xFF], P);
+    float my = 0.0f, mz = 0.0f;
+    Interp I;
+    if (IT < 2) {
+      if (ok) {
+        if (IT == 0) {
+          float* st = store + k * 5;
+          st[0] = L.t.p[0]; st[1] = L.t.p[1]; st[2] = L.t.c[0]; st[3] = L.t.c[1];
+          st[4] = L.t.c[2];
+        }
+        if (IT == 1) {
+          const float a[5] = {L.t.p[0], L.t.p[1], L.t.c[0], L.t.c[1], L.t.c[2]};
+          I = interpolate(a, sv);
+        }
+        ok = meas_at<kMap>(m, P, L.r, my, mz);
+      }
+      if (!ok) {
+        R.ok[t] = 0;
+        busy = false;
         continue;
-      const Resid Rs = residual(L.t, my, mz, P);
-      const bool accept = R.freeze ? acc[k] != 0 : !(Rs.chi2 > P.final_chi2);
-      if (!R.freeze) acc[k] = accept ? 1 : 0;
-      if (!accept) continue;
-      chi2 = chi2 + Rs.chi2;
-      fit_update(L.t, Rs, P);
-      ++n;
-      out = L.t;
-      out_sec = L.sector;
+      }
+      if (IT == 1 && !R.freeze) {
+        R.flag[o0 + k] = chi2_interp(I, my, mz, P) > P.int_chi2 ? 1 : 0;
+      }
+      fit_update(L.t, residual(L.t, my, mz, P), P);
+      if (++j < ns) continue;
+      // the end of this pass starts the next, about the reference kept for it
+      float* ref = R.ref + (long)t * 10 + 5 * IT;
+      if (!R.freeze) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) ref[i] = L.t.p[i];
+      }
+      const Trk<float> s = L.t;
+      lin_start2(L, s, ref, w >> 8, P);
+      save_ckpt(refit_ckpt(R, t, IT + 1, 0), L);
+      R.ok[t] = IT + 2;
+      busy = false;
+      continue;
     }
+    if (ok && !skip && meas_at<kMap>(m, P, L.r, my, mz)) {
+      const Resid Rs = residual(L.t, my, mz, P);
+      const bool accept = R.freeze ? keep : !(Rs.chi2 > P.final_chi2);
+      if (!R.freeze) R.acc[o0 + k] = accept ? 1 : 0;
+      if (accept) {
+        chi2 = chi2 + Rs.chi2;
+        fit_update(L.t, Rs, P);
+        ++n;
+        out = L.t;
+        out_sec = L.sector;
+      }
+    }
+    if (ok && ++j < ns) continue;
     steps3[t] = j;
     R.ok[t] = n > 0 ? 1 : 0;
     R.nused[t] = n;
@@ -2216,179 +2341,315 @@ __global__ void __launch_bounds__(128) k_refit(RefitDev R, KParams P, int* steps
     R.ndf[t] = 2 * n - 5;
     R.out_sector[t] = out_sec;
     R.out_x[t] = out.x;
-    for (int i = 0; i < 5; ++i) R.out_par[(long)t * 5 + i] = out.p[i];
-    for (int i = 0; i < 15; ++i) R.out_cov[(long)t * 15 + i] = out.c[i];
-  }
-}
-
-// One recomputed forward step of the refit, kept for the reverse sweep.
-struct StepRec {
-  float j00, j10, j20, j22;
-  StepJ F;
-  float k0[5], k1[5];
-  float w00, w01, w11, r0, r1;
-  float gy, gz;  // d(measurement)/d(Dx)
-  int bits;      // 1 rotated, 2 propagated, 4 updated, 8 counted in chi2
-};
-
-// Replays forward step j of iteration `it` (0: first inward, 1: outward,
-// 2: last inward) from the current filter state, with identical arithmetic,
-// recording the Jacobians, gain and residual.  Returns false when the
-// forward pass stopped at this step.
-__device__ __forceinline__ bool replay_step(const RefitDev& R, const KParams& P, int t, int it,
-                                            int j, int ns, const int* ids, const float* zr,
-                                            float z0, Lin& L, StepRec& S) {
-  const int k = it == 1 ? j : ns - 1 - j;
-  const int c = ids[k];
-  S.bits = 0;
-  if (j != 0) {
-    bool rot = false;
-    float jr[4];
-    if (!lin_goto(L, R.sector[c], R.row_x[R.row[c]], P, jr, &rot, &S.F)) return false;
-    S.bits |= 2;
-    if (rot) {
-      S.bits |= 1;
-      S.j00 = jr[0]; S.j10 = jr[1]; S.j20 = jr[2]; S.j22 = jr[3];
-    }
-  }
-  if (it == 2 && R.flag[R.offset[t] + k]) return true;
-  // measurement with its derivative by the x displacement
-  float D[3];
-  const float zc = zr[k];
-  map_eval(R.map, P, R.sector[c], L.t.x, R.y[c], zc - z0, D);
-  float my = R.y[c] + D[1], mz = zc + D[2];
-  float snp1 = L.r[2];
-  if (D[0] != 0.0f) {
-    StepJ st;
-    if (!helix_step(L.r, D[0], P, st, P.fit_max_snp)) return it == 2;  // it 2: skipped cluster
-    my = my - (st.p0 - L.r[0]);
-    mz = mz - (st.p1 - L.r[1]);
-    snp1 = st.p2;
-  }
-  const float csp1 = sqrtf(1.0f - snp1 * snp1);
-  S.gy = -snp1 / csp1;
-  S.gz = -L.r[3] / csp1;
-  const Resid Rs = residual(L.t, my, mz, P);
-  if (it == 2) {
-    if (!R.acc[R.offset[t] + k]) return true;
-    S.bits |= 8;
-  }
-  const float h0[5] = {L.t.c[0], L.t.c[1], L.t.c[3], L.t.c[6], L.t.c[10]};
-  const float h1[5] = {L.t.c[1], L.t.c[2], L.t.c[4], L.t.c[7], L.t.c[11]};
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    S.k0[i] = h0[i] * Rs.w00 + h1[i] * Rs.w01;
-    S.k1[i] = h0[i] * Rs.w01 + h1[i] * Rs.w11;
+    for (int i = 0; i < 5; ++i) R.out_par[(long)t * 5 + i] = out.p[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) R.out_cov[(long)t * 15 + i] = out.c[i];
+    busy = false;
   }
-  S.w00 = Rs.w00; S.w01 = Rs.w01; S.w11 = Rs.w11; S.r0 = Rs.r0; S.r1 = Rs.r1;
-  S.bits |= 4;
-  fit_update(L.t, Rs, P);
-  return true;
 }
 
 // Adjoint of the refit: d(sum_t w_t chi2_t)/d(map) with references and
-// decisions held fixed.  One thread per track: reverse sweep over iterations
-// 3, 2, 1, each segment of kCkptStride stations recomputed forward from its
-// checkpoint; per-cluster gradients of the (dx, dy, dz) correction are then
-// scattered through the 64 spline weights into an FP64 accumulator of the
-// block (cross-track reduction in FP64), written per block and summed in a
-// fixed order by k_grad_reduce.
-__global__ void __launch_bounds__(256) k_refit_adjoint(RefitDev R, KParams P,
-                                                       const int* steps3) {
-  extern __shared__ double gacc[];
-  for (int i = threadIdx.x; i < R.ncoef; i += blockDim.x) gacc[i] = 0.0;
-  __syncthreads();
-  const MapDev M = R.map;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < R.n_tracks;
-       t += gridDim.x * blockDim.x) {
-    if (!R.ok[t]) continue;
-    const float w = R.dl_dchi2[t];
-    const int o0 = R.offset[t], ns = R.offset[t + 1] - o0;
-    const int* ids = R.ids + o0;
-    const float z0 = R.z0[t];
-    const float* zr = R.zref + o0;  // cluster z in the innermost side's frame (k_refit)
-    float* dD = R.dD + (long)o0 * 3;
-    for (int i = 0; i < 3 * ns; ++i) dD[i] = 0.0f;
-    const float* ck = R.ckpt + (long)t * 3 * kCkptSeg * kCkptF;
-    float lam[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    for (int it = 2; it >= 0; --it) {
-      const int nsteps = it == 2 ? steps3[t] : ns;
-      const int nseg = (nsteps + kCkptStride - 1) / kCkptStride;
-      for (int sg = nseg - 1; sg >= 0; --sg) {
-        const int j0 = sg * kCkptStride, j1 = min(nsteps, j0 + kCkptStride);
-        StepRec rec[kCkptStride];
-        Lin L;
-        load_ckpt(ck + (it * kCkptSeg + sg) * kCkptF, L);
-        for (int j = j0; j < j1; ++j)
-          replay_step(R, P, t, it, j, ns, ids, zr, z0, L, rec[j - j0]);
-        for (int j = j1 - 1; j >= j0; --j) {
-          const StepRec& S = rec[j - j0];
-          const int k = it == 1 ? j : ns - 1 - j;
-          if (S.bits & 4) {
-            float g0 = 0.0f, g1 = 0.0f;
-            if (S.bits & 8) {
-              g0 = 2.0f * w * (S.w00 * S.r0 + S.w01 * S.r1);
-              g1 = 2.0f * w * (S.w01 * S.r0 + S.w11 * S.r1);
-            }
-            float a0 = g0, a1 = g1;
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-              a0 += S.k0[i] * lam[i];
-              a1 += S.k1[i] * lam[i];
-            }
-            dD[k * 3 + 0] += S.gy * a0 + S.gz * a1;
-            dD[k * 3 + 1] += a0;
-            dD[k * 3 + 2] += a1;
-            lam[0] -= a0;
-            lam[1] -= a1;
-          }
-          if (S.bits & 2) {
-            const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
-            lam[2] = l2 + S.F.f02 * l0 + S.F.f12 * l1;
-            lam[3] = lam[3] + S.F.f13 * l1;
-            lam[4] = lam[4] + S.F.f04 * l0 + S.F.f14 * l1 + S.F.f24 * l2;
-          }
-          if (S.bits & 1) {
-            const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
-            lam[0] = S.j00 * l0 + S.j10 * l1 + S.j20 * l2;
-            lam[2] = S.j22 * l2;
-          }
+// decisions held fixed, in three kernels per chunk of tracks:
+//  k_refit_replay   one thread per (track, iteration, segment of kCkptStride
+//                   stations): the segment's filter steps recomputed from its
+//                   checkpoint, with identical arithmetic, each leaving what
+//                   the reverse sweep needs of it in a 96-byte record.  The
+//                   segments do not depend on one another, so 30 times as many
+//                   threads as tracks share this (most of the arithmetic);
+//  k_refit_reverse  one thread per track over iterations 3, 2, 1 in reverse:
+//                   five adjoint words and some thirty operations per step,
+//                   leaving the gradient by the step's corrected cluster;
+//  k_refit_scatter  those gradients through the 64 spline weights into FP64
+//                   accumulators (the cross-track reduction in FP64), summed
+//                   over the blocks in a fixed order by k_grad_reduce.
+// (As one kernel with a thread per track, the steps of a segment in local
+// memory and 192 FP64 shared-memory atomics per cluster, its 138 KB of
+// accumulators left 8 warps per SM: 17 ms for the 7,500 tracks of a distorted
+// 1.2e6-cluster frame.)
+//
+// Step record: F (f02, f04, f12, f13, f14, f24), W r of a step counted in
+// chi2 (else 0), d(measurement)/d(x displacement), gain columns k0 and k1, the
+// rotation's (j00, j10, j20, j22) (else the identity's); zeros where a step has
+// no propagation or no update.  The reverse sweep replaces the first float4 by
+// the gradient by the step's (x displacement, y, z).
+__device__ __forceinline__ float4* adj_rec(const RefitDev& R, int q) {  // track q of the chunk
+  return R.rec + (long)q * 3 * kMaxRows * kRecV;
+}
+
+__global__ void __launch_bounds__(128, 4) k_refit_replay(RefitDev R, KParams P,
+                                                         const int* steps3, int t0, int tn) {
+  const long wk = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (wk >= (long)tn * 3 * kCkptSeg) return;
+  // (a warp's lanes: 32 neighbouring tracks in one segment and iteration)
+  const int t = t0 + (int)(wk % tn);
+  const int it = (int)(wk / tn) % 3, sg = (int)(wk / tn) / 3;
+  if (!R.ok[t]) return;
+  const int o0 = R.offset[t], ns = R.offset[t + 1] - o0;
+  const int nsteps = it == 2 ? steps3[t] : ns;
+  const int j0 = sg * kCkptStride, j1 = min(nsteps, j0 + kCkptStride);
+  if (j0 >= nsteps) return;
+  float4* rec = adj_rec(R, t - t0) + (long)it * ns * kRecV;
+  Lin L;
+  load_ckpt(refit_ckpt(R, t, it, sg), L);
+  for (int j = j0; j < j1; ++j) {
+    const int k = it == 1 ? j : ns - 1 - j;
+    const float4 m = R.meas[o0 + k];
+    const int w = __float_as_int(m.w);
+    StepJ S;
+    S.f02 = S.f04 = S.f12 = S.f13 = S.f14 = S.f24 = 0.0f;
+    float jr[4] = {1.0f, 0.0f, 0.0f, 1.0f};
+    float k0[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, k1[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float q0 = 0.0f, q1 = 0.0f, gy = 0.0f, gz = 0.0f;
+    bool go = true;
+    if (j != 0) go = lin_goto(L, w >> 8, R.row_x[w & 0xFF], P, jr, nullptr, &S);
+    if (go && !(it == 2 && (R.flag[o0 + k] || !R.acc[o0 + k]))) {
+      // the measurement with its derivative by the x displacement
+      float my = m.y, mz = m.z, snp1 = L.r[2];
+      if (m.x != 0.0f) {
+        StepJ st;
+        go = helix_step(L.r, m.x, P, st, P.fit_max_snp);
+        if (go) {
+          my = my - (st.p0 - L.r[0]);
+          mz = mz - (st.p1 - L.r[1]);
+          snp1 = st.p2;
         }
       }
-    }
-    // scatter d(loss)/d(correction) through the spline weights
-    if (M.on) {
-      for (int k = 0; k < ns; ++k) {
-        const int c = ids[k];
-        const SplinePt sp =
-            spline_point(M, P, R.sector[c], R.row_x[R.row[c]], R.y[c], zr[k] - z0);
-        int pidx[4];
+      if (go) {  // (iteration 3 skips a cluster that the reference cannot reach)
+        const float csp1 = sqrtf(1.0f - snp1 * snp1);
+        gy = -snp1 / csp1;
+        gz = -L.r[3] / csp1;
+        const Resid Rs = residual(L.t, my, mz, P);
+        const float h0[5] = {L.t.c[0], L.t.c[1], L.t.c[3], L.t.c[6], L.t.c[10]};
+        const float h1[5] = {L.t.c[1], L.t.c[2], L.t.c[4], L.t.c[7], L.t.c[11]};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) pidx[e] = phi_index(sp.ip, e, M.nphi);
-        for (int comp = 0; comp < 3; ++comp) {
-          const double g = (double)dD[k * 3 + comp];
-          if (g == 0.0) continue;
-          for (int a = 0; a < 4; ++a)
-            for (int b = 0; b < 4; ++b) {
-              const float wzr = sp.wz[a] * sp.wr[b];
-              const long base = (((long)comp * M.nz + (sp.iz + a)) * M.nr + (sp.ir + b)) * M.nphi;
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                atomicAdd(&gacc[base + pidx[e]], (double)(wzr * sp.wp[e]) * g);
-            }
+        for (int i = 0; i < 5; ++i) {
+          k0[i] = h0[i] * Rs.w00 + h1[i] * Rs.w01;
+          k1[i] = h0[i] * Rs.w01 + h1[i] * Rs.w11;
         }
+        if (it == 2) {
+          q0 = Rs.w00 * Rs.r0 + Rs.w01 * Rs.r1;
+          q1 = Rs.w01 * Rs.r0 + Rs.w11 * Rs.r1;
+        }
+        fit_update(L.t, Rs, P);
+      }
+    }
+    float4* r = rec + (long)j * kRecV;
+    r[0] = make_float4(S.f02, S.f04, S.f12, S.f13);
+    r[1] = make_float4(S.f14, S.f24, q0, q1);
+    r[2] = make_float4(gy, gz, k0[0], k0[1]);
+    r[3] = make_float4(k0[2], k0[3], k0[4], k1[0]);
+    r[4] = make_float4(k1[1], k1[2], k1[3], k1[4]);
+    r[5] = make_float4(jr[0], jr[1], jr[2], jr[3]);
+  }
+}
+
+// The records of kRevStage steps are copied to shared memory one stage ahead
+// (16-byte asynchronous copies, each thread its own track's records, laid out
+// so that a warp's reads hit distinct banks): the sweep is a serial chain of
+// steps, and each step's loads would otherwise stand in it.
+constexpr int kRevStage = 8;
+constexpr int kRevBlock = 64;
+
+__device__ __forceinline__ void copy_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(smem)),
+               "l"(gmem)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(kRevBlock) k_refit_reverse(RefitDev R, const int* steps3, int t0,
+                                                             int tn) {
+  extern __shared__ float4 rev_sh[];  // [2][kRevStage * kRecV][kRevBlock]
+  const int q = blockIdx.x * kRevBlock + threadIdx.x;
+  if (q >= tn || !R.ok[t0 + q]) return;
+  const int t = t0 + q;
+  const int ns = R.offset[t + 1] - R.offset[t];
+  const int tot = 2 * ns + steps3[t];
+  const float w2 = 2.0f * R.dl_dchi2[t];
+  float4* rec = adj_rec(R, q);
+  float4* const sh = rev_sh + threadIdx.x;
+  auto fetch = [&](int s) {  // stage s: steps tot - 1 - s kRevStage downwards
+    float4* d = sh + (s & 1) * (kRevStage * kRecV * kRevBlock);
+    for (int e = 0; e < kRevStage; ++e) {
+      const int i = tot - 1 - s * kRevStage - e;
+      if (i < 0) break;
+#pragma unroll
+      for (int v = 0; v < kRecV; ++v)
+        copy_async16(d + (e * kRecV + v) * kRevBlock, rec + (long)i * kRecV + v);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float lam[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  const int nst = (tot + kRevStage - 1) / kRevStage;
+  fetch(0);
+  for (int s = 0; s < nst; ++s) {
+    fetch(s + 1);  // (empty past the last stage)
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    const float4* d = sh + (s & 1) * (kRevStage * kRecV * kRevBlock);
+    for (int e = 0; e < kRevStage; ++e) {
+      const int i = tot - 1 - s * kRevStage - e;
+      if (i < 0) break;
+      const float4 v0 = d[(e * kRecV + 0) * kRevBlock], v1 = d[(e * kRecV + 1) * kRevBlock];
+      const float4 v2 = d[(e * kRecV + 2) * kRevBlock], v3 = d[(e * kRecV + 3) * kRevBlock];
+      const float4 v4 = d[(e * kRecV + 4) * kRevBlock], v5 = d[(e * kRecV + 5) * kRevBlock];
+      const float k0[5] = {v2.z, v2.w, v3.x, v3.y, v3.z};
+      const float k1[5] = {v3.w, v4.x, v4.y, v4.z, v4.w};
+      float a0 = w2 * v1.z, a1 = w2 * v1.w;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        a0 += k0[j] * lam[j];
+        a1 += k1[j] * lam[j];
+      }
+      // (a step without an update has k = g = 0 here and no gradient)
+      rec[(long)i * kRecV] = make_float4(v2.x * a0 + v2.y * a1, a0, a1, 0.0f);
+      lam[0] -= a0;
+      lam[1] -= a1;
+      {
+        const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
+        lam[2] = l2 + v0.x * l0 + v0.z * l1;
+        lam[3] = lam[3] + v0.w * l1;
+        lam[4] = lam[4] + v0.y * l0 + v1.x * l1 + v1.y * l2;
+      }
+      {
+        const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
+        lam[0] = v5.x * l0 + v5.y * l1 + v5.z * l2;
+        lam[2] = v5.w * l2;
       }
     }
   }
-  __syncthreads();
-  double* part = R.gpart + (long)blockIdx.x * R.ncoef;
-  for (int i = threadIdx.x; i < R.ncoef; i += blockDim.x) part[i] = gacc[i];
 }
 
-__global__ void k_grad_reduce(RefitDev R) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R.ncoef; i += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < R.gblocks; ++b) s += R.gpart[(long)b * R.ncoef + i];
+// Scatter of the gradients through the spline weights, one warp per track.  Its
+// lanes first lay out 32 clusters' weights, cell and gradient in shared memory;
+// then the warp takes the clusters in track order, each lane holding two of the
+// cell's 64 control points for the three components.  A track stays about ten
+// clusters in one cell, so the lanes sum in registers and add to the FP64
+// accumulators only where the cell changes.  Those sums are kept as float pairs
+// (TwoProduct / TwoSum, 2^-46 relative): this GPU's FP64 rate is 1/60 of its
+// FP32 rate, and 192 FP64 operations per cluster would cost more than the whole
+// sweep.  kShared: the block's accumulators lie in shared memory; a map too large
+// for that has them in the block's partial sums in global memory.
+constexpr int kScatWarps = 16;
+constexpr int kScatF = 16;  // floats per staged cluster: wz[4], wr[4], wp[4], g[3], cell
+
+template <bool kShared>
+__global__ void __launch_bounds__(32 * kScatWarps) k_refit_scatter(RefitDev R, KParams P,
+                                                                   const int* steps3, int t0,
+                                                                   int tn) {
+  extern __shared__ double scat_sh[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* part = R.gpart + (long)blockIdx.x * R.ncoef;
+  double* gacc = kShared ? scat_sh : part;
+  float* st = (float*)(scat_sh + (kShared ? R.ncoef : 0)) + (long)warp * 32 * kScatF;
+  if (kShared || t0 == 0)
+    for (int i = threadIdx.x; i < R.ncoef; i += blockDim.x) gacc[i] = t0 == 0 ? 0.0 : part[i];
+  __syncthreads();
+  const MapDev M = R.map;
+  const int la = lane >> 3, lb = (lane >> 1) & 3, lh = 2 * (lane & 1);  // z, r, first phi point
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  const int ncomp = M.nz * M.nr * M.nphi;
+  for (int q = blockIdx.x * (blockDim.x >> 5) + warp; q < tn; q += nw) {
+    const int t = t0 + q;
+    if (!R.ok[t]) continue;
+    const int o0 = R.offset[t], ns = R.offset[t + 1] - o0;
+    const int n3 = steps3[t];
+    const float z0 = R.z0[t];
+    const float4* rec = adj_rec(R, q);
+    float hi[6], lo[6];  // [component][point]
+    int cell = -1;
+    auto flush = [&]() {
+      if (cell < 0) return;
+      const int nphi = M.nphi, ip = cell % nphi;
+      const int zr = cell / nphi;  // (z, r) cell corner
+      const int row = ((zr / M.nr + la) * M.nr + (zr % M.nr + lb)) * nphi;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int at = row + phi_index(ip, lh + e, nphi);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          atomicAdd(&gacc[c * ncomp + at], (double)hi[2 * c + e] + (double)lo[2 * c + e]);
+      }
+    };
+    for (int k0 = 0; k0 < ns; k0 += 32) {
+      const int k = k0 + lane;
+      if (k < ns) {
+        const float2 yz = R.raw[o0 + k];
+        const int w = __float_as_int(R.meas[o0 + k].w);
+        const SplinePt sp = spline_point<true>(M, P, w >> 8, R.row_x[w & 0xFF], yz.x, yz.y - z0);
+        // the three iterations' gradients, in the order of the reverse sweep
+        float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+#pragma unroll
+        for (int it = 2; it >= 0; --it) {
+          const int j = it == 1 ? k : ns - 1 - k;
+          if (it == 2 && j >= n3) continue;
+          const float4 g = rec[((long)it * ns + j) * kRecV];
+          gx += g.x;
+          gy += g.y;
+          gz += g.z;
+        }
+        float* d = st + lane * kScatF;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          d[i] = sp.wz[i];
+          d[4 + i] = sp.wr[i];
+          d[8 + i] = sp.wp[i];
+        }
+        d[12] = gx;
+        d[13] = gy;
+        d[14] = gz;
+        // (phi_index wraps its argument, so the cell's phi can be wrapped here)
+        const int ipw = ((sp.ip % M.nphi) + M.nphi) % M.nphi;
+        d[15] = __int_as_float((sp.iz * M.nr + sp.ir) * M.nphi + ipw);
+      }
+      __syncwarp();
+      const int m = min(32, ns - k0);
+      for (int i = 0; i < m; ++i) {
+        const float* d = st + i * kScatF;
+        const int c = __float_as_int(d[15]);
+        if (c != cell) {
+          flush();
+          cell = c;
+#pragma unroll
+          for (int e = 0; e < 6; ++e) hi[e] = lo[e] = 0.0f;
+        }
+        const float wzr = d[la] * d[4 + lb];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float w = wzr * d[8 + lh + e];
+#pragma unroll
+          for (int g = 0; g < 3; ++g) {
+            float p, pe, s, se;
+            two_prod(w, d[12 + g], p, pe);
+            two_sum(hi[2 * g + e], p, s, se);
+            lo[2 * g + e] = df_add(lo[2 * g + e], df_add(se, pe));
+            hi[2 * g + e] = s;
+          }
+        }
+      }
+      __syncwarp();
+    }
+    flush();
+  }
+  if (kShared) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < R.ncoef; i += blockDim.x) part[i] = gacc[i];
+  }
+}
+
+// Sum of the blocks' partial gradients in a fixed order: eight threads per
+// coefficient, each over every eighth block, then the eight sums in turn.
+__global__ void __launch_bounds__(256) k_grad_reduce(RefitDev R) {
+  __shared__ double sh[8][32];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + x;
+  double s = 0.0;
+  if (i < R.ncoef)
+    for (int b = y; b < R.gblocks; b += 8) s += R.gpart[(long)b * R.ncoef + i];
+  sh[y][x] = s;
+  __syncthreads();
+  if (y == 0 && i < R.ncoef) {
+    for (int k = 1; k < 8; ++k) s += sh[k][x];
     R.dl_dmap[i] = (float)s;
   }
 }
@@ -2396,17 +2657,61 @@ __global__ void k_grad_reduce(RefitDev R) {
 }  // namespace
 
 int refit_forward(RefitDev& R, const KParams& P, int* steps3, int sms, cudaStream_t s) {
-  if (R.n_tracks > 0) k_refit<<<sms * 16, 128, 0, s>>>(R, P, steps3);
-  return R.n_tracks > 0 ? 1 : 0;
+  if (R.n_tracks <= 0) return 0;
+  // (no more blocks than there are tracks for)
+  const unsigned g = (unsigned)min((long)sms * 4, (long)blocks_for(R.n_tracks, 32));
+  k_refit_prep<<<(unsigned)min((long)sms * 16, (long)blocks_for(R.n_tracks, 8)), 256, 0, s>>>(
+      R, P, steps3);
+  k_refit_start<<<g, 128, 0, s>>>(R, P);
+  if (R.map.on) {
+    k_refit_iter<0, true><<<g, 128, 0, s>>>(R, P, steps3);
+    k_refit_iter<1, true><<<g, 128, 0, s>>>(R, P, steps3);
+    k_refit_iter<2, true><<<g, 128, 0, s>>>(R, P, steps3);
+  } else {
+    k_refit_iter<0, false><<<g, 128, 0, s>>>(R, P, steps3);
+    k_refit_iter<1, false><<<g, 128, 0, s>>>(R, P, steps3);
+    k_refit_iter<2, false><<<g, 128, 0, s>>>(R, P, steps3);
+  }
+  return 5;
 }
 
 int refit_backward(RefitDev& R, const KParams& P, const int* steps3, int sms, cudaStream_t s) {
   (void)sms;
-  const size_t smem = sizeof(double) * (size_t)R.ncoef;
-  cudaFuncSetAttribute(k_refit_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_refit_adjoint<<<R.gblocks, 256, smem, s>>>(R, P, steps3);
-  k_grad_reduce<<<(R.ncoef + 255) / 256, 256, 0, s>>>(R);
-  return 2;
+  const size_t rev = sizeof(float4) * 2 * kRevStage * kRecV * kRevBlock;
+  const size_t acc = sizeof(double) * (size_t)R.ncoef;
+  const size_t stage = sizeof(float) * 32 * kScatF;  // per warp
+  // accumulators in shared memory beside the staging of at least four warps
+  // (the 18 x 16 x 20 map's 138 KB leave room for all sixteen)
+  int warps = kScatWarps;
+  bool shared = true;
+  while (warps > 4 && acc + warps * stage > (size_t)R.smem_max) --warps;
+  if (acc + warps * stage > (size_t)R.smem_max) {
+    shared = false;
+    warps = kScatWarps;
+  }
+  const size_t scat = (shared ? acc : 0) + warps * stage;
+  cudaFuncSetAttribute(k_refit_reverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rev);
+  cudaFuncSetAttribute(k_refit_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       shared ? (int)scat : 0);
+  int k = 0;
+  long t0 = 0;
+  do {
+    const int tn = (int)min(R.n_tracks - t0, (long)kAdjChunk);
+    if (tn > 0) {
+      k_refit_replay<<<blocks_for((long)tn * 3 * kCkptSeg, 128), 128, 0, s>>>(R, P, steps3,
+                                                                              (int)t0, tn);
+      k_refit_reverse<<<blocks_for(tn, kRevBlock), kRevBlock, rev, s>>>(R, steps3, (int)t0, tn);
+      k += 2;
+    }
+    if (shared)
+      k_refit_scatter<true><<<R.gblocks, 32 * warps, scat, s>>>(R, P, steps3, (int)t0, tn);
+    else
+      k_refit_scatter<false><<<R.gblocks, 32 * warps, scat, s>>>(R, P, steps3, (int)t0, tn);
+    ++k;
+    t0 += kAdjChunk;
+  } while (t0 < R.n_tracks);
+  k_grad_reduce<<<blocks_for(R.ncoef, 32), 256, 0, s>>>(R);
+  return k + 1;
 }
 
 int stage_sector_refit(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {

@@ -331,6 +331,12 @@ constexpr int kCkptStride = 16;                        // stations per checkpoin
 constexpr int kCkptSeg = (kMaxRows + kCkptStride - 1) / kCkptStride;
 constexpr int kCkptF = 27;                             // p[5], c[15], ref[5], x, sector
 
+constexpr int kRefitQueues = 4;   // start pass, iterations 1-3
+constexpr int kRecV = 6;          // float4 per step record of the adjoint
+// Tracks per chunk of the adjoint, which bounds its step records: 3 kMaxRows
+// steps of 96 bytes each at most, 1.5 GB.
+constexpr int kAdjChunk = 32768;
+
 // Refit of given tracks (fixed clusters) and its adjoint.
 struct RefitDev {
   long n_tracks;
@@ -349,10 +355,14 @@ struct RefitDev {
   const float* in_zsh;     // [n_tracks] z shift of the far side (central electrode), or NULL
   const float* row_x;
   int freeze;
+  // per cluster reference (k_refit_prep)
+  float2* raw;             // [cap_refs] cluster y, and z in the frame of the track's innermost side
+  float4* meas;            // [cap_refs] (x displacement, y, z of the corrected cluster, station
+                           // word: row in bits 0..7, sector above)
+  int* queue;              // [kRefitQueues] work-queue heads of the filter passes
   // state kept for freezing and for the adjoint
   float* ref;              // [cap][10]
   uint8_t* flag;           // [cap_refs]
-  float* zref;             // [cap_refs] cluster z in the frame of the track's innermost side
   uint8_t* acc;            // [cap_refs]
   float* z0;               // [cap]
   float* ckpt;             // [cap][3][kCkptSeg][kCkptF]
@@ -368,11 +378,13 @@ struct RefitDev {
   float* out_x;
   // adjoint
   const float* dl_dchi2;   // [n_tracks]
-  float* dD;               // [cap_refs][3]
+  float4* rec;             // [min(cap, kAdjChunk)][3 kMaxRows][kRecV] adjoint: step
+                           // records of one chunk of tracks
   double* gpart;           // [blocks][ncoef]
   float* dl_dmap;          // [ncoef]
   int ncoef;
   int gblocks;
+  int smem_max;            // shared memory a block may have [bytes]
   MapDev map;
 };
 
