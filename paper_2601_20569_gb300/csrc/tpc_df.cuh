@@ -129,4 +129,78 @@ TPC_DF void df_update(float* p, float* c, float r0, float r1, float w00, float w
   }
 }
 
+// The same update for callers that need the FP64 update's results bit for bit:
+// every result is checked against the interval its exact value can lie in, and
+// the function returns false (the caller then runs the FP64 update) where the
+// interval holds a rounding boundary.
+//
+// Error of a result v -+ (k0 x + k1 y) before its final rounding, with
+// A0 = |h0 w00| + |h1 w01|, A1 = |h0 w01| + |h1 w11| (the gains' terms),
+// B = A0 |x| + A1 |y| and u = 2^-24:
+//   gain pairs (df_dot2): low part off by at most 3 u^2 A, so 3 u^2 B in the result;
+//   products (kl x into ue): at most 3 u^2 B;  t = ue + we: at most 3 u^2 B;
+//   e1 + e2: at most 2 u^2 (|v| + B);  the last sum into the low word:
+//   u^2 (2 |v| + 5 B).
+// Together below 16 u^2 (|v| + B) = 2^-44 (|v| + B).  The FP64 update's own
+// roundings (2^-53 relative per operation) add less than 2^-50 (|v| + B), the
+// low word +- E rounds by at most 2^-45 (|v| + B), the float evaluation of the
+// bound is right to 2^-20 of itself: E = 2^-42 (|v| + B) covers the sum twice
+// over.  2^-110 covers products whose error terms underflow, for operands below
+// the limit set on the bound (10^9).  Rounding to float is monotonic, so when
+// both ends of the interval round alike, so do the exact value, the FP64
+// update's and this one's.  A result that is zero term by term is evaluated
+// term by term, where float and double agree in sign.
+template <bool kSub>
+TPC_DF bool df_axpy2_checked(float v, float kh, float kl, float x, float gh, float gl, float y,
+                             float bound, bool zero, float& out) {
+  float u, ue, w, we, s1, e1, s2, e2;
+  two_prod(kh, x, u, ue);
+  ue = df_fma(kl, x, ue);
+  two_prod(gh, y, w, we);
+  we = df_fma(gl, y, we);
+  two_sum(v, kSub ? -u : u, s1, e1);
+  two_sum(s1, kSub ? -w : w, s2, e2);
+  const float t = df_add(ue, we);
+  const float lo = df_add(df_add(e1, e2), kSub ? -t : t);
+  const float E = df_fma(bound, 2.2737367544323206e-13f, 7.7037197775489434e-34f);
+  out = df_add(s2, lo);
+  const bool same = df_add(s2, df_sub(lo, E)) == df_add(s2, df_add(lo, E)) && bound < 1e9f;
+  if (zero) {
+    const float z = df_add(u, w);
+    out = kSub ? df_sub(v, z) : df_add(v, z);
+  }
+  return same || zero;
+}
+
+TPC_DF bool df_update_checked(const float* p, const float* c, float r0, float r1, float w00,
+                              float w01, float w11, float* po, float* co) {
+  const float h0[5] = {c[0], c[1], c[3], c[6], c[10]};
+  const float h1[5] = {c[1], c[2], c[4], c[7], c[11]};
+  bool ok = true;
+  int idx = 0;
+  TPC_DF_UNROLL
+  for (int i = 0; i < 5; ++i) {
+    float k0h, k0l, k1h, k1l;
+    df_dot2(h0[i], w00, h1[i], w01, k0h, k0l);
+    df_dot2(h0[i], w01, h1[i], w11, k1h, k1l);
+    const float a0 = df_fma(fabsf(h0[i]), fabsf(w00), fabsf(df_mul(h1[i], w01)));
+    const float a1 = df_fma(fabsf(h0[i]), fabsf(w01), fabsf(df_mul(h1[i], w11)));
+    const bool hz = h0[i] == 0.0f && h1[i] == 0.0f;
+    {
+      const float b = df_fma(a0, fabsf(r0), df_fma(a1, fabsf(r1), fabsf(p[i])));
+      ok &= df_axpy2_checked<false>(p[i], k0h, k0l, r0, k1h, k1l, r1, b,
+                                    p[i] == 0.0f && (hz || (r0 == 0.0f && r1 == 0.0f)), po[i]);
+    }
+    TPC_DF_UNROLL
+    for (int j = 0; j <= i; ++j) {
+      const float b = df_fma(a0, fabsf(h0[j]), df_fma(a1, fabsf(h1[j]), fabsf(c[idx])));
+      ok &= df_axpy2_checked<true>(c[idx], k0h, k0l, h0[j], k1h, k1l, h1[j], b,
+                                   c[idx] == 0.0f && (hz || (h0[j] == 0.0f && h1[j] == 0.0f)),
+                                   co[idx]);
+      ++idx;
+    }
+  }
+  return ok;
+}
+
 }  // namespace tpc

@@ -262,20 +262,21 @@ __device__ __forceinline__ void update(Trk<float>& t, const Resid& R) {
 }
 
 // The same update with the gain and covariance arithmetic in FP64, rounded
-// back to FP32 (the final fit's update of low-pT loopers).  Fast mode runs it
-// in double-float arithmetic on the FP32 pipe instead (tpc_df.cuh: on GB300
-// the FP64 unit is about 1/60 of the FP32 rate; the rounded results are those
-// of the FP64 update unless one lies within about 2^-46 of a rounding
-// boundary).
-__device__ __forceinline__ void update_fp64(Trk<float>& t, const Resid& R) {
-#ifdef TPC_FAST_ARITH
-  df_update(t.p, t.c, R.r0, R.r1, R.w00, R.w01, R.w11);
-#else
-  const double w00 = widen(R.w00), w01 = widen(R.w01), w11 = widen(R.w11), r0 = widen(R.r0),
-               r1 = widen(R.r1);
-  const double h0[5] = {widen(t.c[0]), widen(t.c[1]), widen(t.c[3]), widen(t.c[6]),
-                        widen(t.c[10])};
-  const double h1[5] = {h0[1], widen(t.c[2]), widen(t.c[4]), widen(t.c[7]), widen(t.c[11])};
+// back to FP32 (the final fit's update of low-pT loopers).  On GB300 the FP64
+// unit is about 1/60 of the FP32 rate (80 FP64 operations hold a warp for some
+// 5,000 cycles), so both modes run it in double-float arithmetic on the FP32
+// pipe (tpc_df.cuh).  Fast mode takes those results, which are those of the FP64
+// update unless one lies within about 2^-46 of a rounding boundary.  Strict mode
+// checks each result against such a boundary and runs the FP64 update where one
+// is near (about one update in 10^4), so its results are the FP64 update's, as
+// the oracle defines them.
+#ifndef TPC_FAST_ARITH
+static __device__ __noinline__ void update_fp64_exact(float* p, float* c, float fr0, float fr1, float fw00,
+                                               float fw01, float fw11) {
+  const double w00 = widen(fw00), w01 = widen(fw01), w11 = widen(fw11), r0 = widen(fr0),
+               r1 = widen(fr1);
+  const double h0[5] = {widen(c[0]), widen(c[1]), widen(c[3]), widen(c[6]), widen(c[10])};
+  const double h1[5] = {h0[1], widen(c[2]), widen(c[4]), widen(c[7]), widen(c[11])};
   double k0[5], k1[5];
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
@@ -283,16 +284,40 @@ __device__ __forceinline__ void update_fp64(Trk<float>& t, const Resid& R) {
     k1[i] = h0[i] * w01 + h1[i] * w11;
   }
 #pragma unroll
-  for (int i = 0; i < 5; ++i) t.p[i] = narrow(widen(t.p[i]) + (k0[i] * r0 + k1[i] * r1));
+  for (int i = 0; i < 5; ++i) p[i] = narrow(widen(p[i]) + (k0[i] * r0 + k1[i] * r1));
   int idx = 0;
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
 #pragma unroll
     for (int j = 0; j <= i; ++j) {
-      t.c[idx] = narrow(widen(t.c[idx]) - (k0[i] * h0[j] + k1[i] * h1[j]));
+      c[idx] = narrow(widen(c[idx]) - (k0[i] * h0[j] + k1[i] * h1[j]));
       ++idx;
     }
   }
+}
+#endif
+
+__device__ __forceinline__ void update_fp64(Trk<float>& t, const Resid& R) {
+#ifdef TPC_FAST_ARITH
+  df_update(t.p, t.c, R.r0, R.r1, R.w00, R.w01, R.w11);
+#else
+  float p[5], c[15];
+  if (!df_update_checked(t.p, t.c, R.r0, R.r1, R.w00, R.w01, R.w11, p, c)) {
+    float pe[5], ce[15];  // (a copy, so that the call keeps nothing else in memory)
+#pragma unroll
+    for (int i = 0; i < 5; ++i) pe[i] = t.p[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) ce[i] = t.c[i];
+    update_fp64_exact(pe, ce, R.r0, R.r1, R.w00, R.w01, R.w11);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) p[i] = pe[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) c[i] = ce[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) t.p[i] = p[i];
+#pragma unroll
+  for (int i = 0; i < 15; ++i) t.c[i] = c[i];
 #endif
 }
 
