@@ -347,12 +347,92 @@ __device__ __forceinline__ void links_one(const FrameDev& F, const KParams& P, l
   }
 }
 
+// The same search over whole z strips.  A row's clusters are sorted strip by
+// strip, so the strips the window reaches are one contiguous run: two bin
+// offsets instead of two per strip, and one loop that the lanes of a warp run
+// together (neighbouring sorted clusters have neighbouring runs of nearly the
+// same length).  The clusters inside the window are kept as bit masks over the
+// runs, and the pairs of the two masks tested in a loop of their own, ids read
+// on exact ties only.  It visits a superset of the clusters links_one visits,
+// tests them alike, and the best pair is a minimum under a total order: the
+// same links.  Testing all y bins of the strips pays while they are few (a row
+// of a 2.8 ms frame has five or six): rows with more than kRunMaxY, and runs of
+// more than 32 clusters, take links_one (returns false).
+constexpr int kRunMaxY = 9;
+
+template <bool kLeft>
+__device__ __forceinline__ bool links_run(const FrameDev& F, const KParams& P, long k, int& bu,
+                                          int& bd) {
+  const int rr = F.srow[k];
+  const int r = rr % P.n_rows;
+  bu = -1;
+  bd = -1;
+  if (r < 1 || r > P.n_rows - 2 || (kLeft && F.sused[k])) return true;
+  const float2 pc = F.syz[k];
+  const float yc = pc.x, zc = pc.y;
+  const RowGrid gd = F.rows[rr - 1], gu = F.rows[rr + 1];
+  if (gd.ncl == 0 || gu.ncl == 0) return true;
+  const float m = 0.01f;
+  const float zlo = zc - P.link_wz - m, zhi = zc + P.link_wz + m;
+  if (!(zlo <= zhi)) return true;
+  const int* bf = F.bin_first;
+  const int d0 = bf[gd.bin0 + bin_of(zlo, gd.z0, gd.invDz, gd.nZ) * gd.nY];
+  const int nd = bf[gd.bin0 + (bin_of(zhi, gd.z0, gd.invDz, gd.nZ) + 1) * gd.nY] - d0;
+  const int u0 = bf[gu.bin0 + bin_of(zlo, gu.z0, gu.invDz, gu.nZ) * gu.nY];
+  const int nu = bf[gu.bin0 + (bin_of(zhi, gu.z0, gu.invDz, gu.nZ) + 1) * gu.nY] - u0;
+  if (gd.nY > kRunMaxY || gu.nY > kRunMaxY || nd > 32 || nu > 32) return false;
+  unsigned md = 0u, mu = 0u;
+  for (int c = 0; c < nd; ++c) {
+    const float2 p = F.syz[d0 + c];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
+        !(kLeft && F.sused[d0 + c]))
+      md |= 1u << c;
+  }
+  if (md == 0u) return true;
+  for (int c = 0; c < nu; ++c) {
+    const float2 p = F.syz[u0 + c];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
+        !(kLeft && F.sused[u0 + c]))
+      mu |= 1u << c;
+  }
+  const float xd = F.row_x[r - 1], xc = F.row_x[r], xu = F.row_x[r + 1];
+  const float f = (xc - xd) / (xu - xd);
+  float best = 0.0f;
+  unsigned dm = md;
+  while (mu) {  // all pairs: the lower mask once per upper cluster
+    const int u = u0 + __ffs(mu) - 1, d = d0 + __ffs(dm) - 1;
+    const float2 pu = F.syz[u], pd = F.syz[d];
+    const float yp = pd.x + (pu.x - pd.x) * f;
+    const float zp = pd.y + (pu.y - pd.y) * f;
+    const float ey = yp - yc, ez = zp - zc;
+    const float d2 = ey * ey + ez * ez;
+    if (d2 < P.link_chi2) {
+      bool take = bu < 0 || d2 < best;
+      if (!take && d2 == best) {
+        const int uid = F.sid[u], buid = F.sid[bu];
+        take = uid < buid || (uid == buid && F.sid[d] < F.sid[bd]);
+      }
+      if (take) {
+        best = d2;
+        bu = u;
+        bd = d;
+      }
+    }
+    dm &= dm - 1u;
+    if (dm == 0u) {
+      dm = md;
+      mu &= mu - 1u;
+    }
+  }
+  return true;
+}
+
 template <bool kLeft>
 __global__ void k_links(FrameDev F, KParams P) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= F.n || F.cnt->err) return;
   int bu, bd;
-  links_one<kLeft>(F, P, k, bu, bd);
+  if (!links_run<kLeft>(F, P, k, bu, bd)) links_one<kLeft>(F, P, k, bu, bd);
   F.lup[k] = bu;
   F.ldn[k] = bd;
 }
@@ -728,9 +808,9 @@ __device__ __forceinline__ int pick(const FrameDev& F, const KParams& P, const T
   const float hz = sqrtf(P.follow_chi2 * (t.c[2] + P.sz2)) * 1.001f + 0.01f;
   const float ylo = t.p[0] - hy, yhi = t.p[0] + hy;
   const float zlo = t.p[1] - hz, zhi = t.p[1] + hz;
-  int best = -1, bid = 0;
+  int best = -1;
   float bchi = 0.0f;
-  for_window(F.bin_first, g, ylo, yhi, zlo, zhi, [&](int k) {
+  for_window_flat(F.bin_first, g, ylo, yhi, zlo, zhi, [&](int k) {
     if (kLeft && F.sused[k]) return;
     if (kKept && F.st_kept[k]) return;
     const float2 pk = F.syz[k];
@@ -739,11 +819,10 @@ __device__ __forceinline__ int pick(const FrameDev& F, const KParams& P, const T
     if (fabsf(zk - t.p[1]) > hz) return;
     const float chi2 = chi2_of(t, yk, zk, P);
     if (!(chi2 < P.follow_chi2)) return;
-    const int id = F.sid[k];
-    if (best < 0 || chi2 < bchi || (chi2 == bchi && id < bid)) {
+    // (the input ids are read on exact ties only)
+    if (best < 0 || chi2 < bchi || (chi2 == bchi && F.sid[k] < F.sid[best])) {
       best = k;
       bchi = chi2;
-      bid = id;
       by = yk;
       bz = zk;
     }

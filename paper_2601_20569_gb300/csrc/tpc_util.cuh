@@ -40,6 +40,58 @@ __device__ __forceinline__ void for_window(const int* __restrict__ bin_first, co
   }
 }
 
+// The clusters of up to kStrips z strips of a search window as one run of
+// candidates.  A window of a few cm covers one or two strips holding about one
+// cluster each (bins of some 5 cm with half a cluster), so what a search waits
+// for is its chain of dependent loads, and what it diverges over is the nesting
+// of strips and clusters: the strips' ranges are requested together, and the
+// lanes of a warp run one loop over their candidates, not one per strip.
+constexpr int kStrips = 3;
+
+struct StripRun {
+  int l0, l1, l2;  // the strips' first clusters
+  int n0, n1, n;   // candidates of the first, the first two, all strips
+  __device__ __forceinline__ int at(int c) const {
+    return c < n0 ? l0 + c : c < n1 ? l1 + (c - n0) : l2 + (c - n1);
+  }
+};
+
+// Strips iz .. min(iz + kStrips - 1, iz1), y bins iy0 .. iy1.
+__device__ __forceinline__ StripRun strip_run(const int* __restrict__ bin_first, const RowGrid& g,
+                                              int iy0, int iy1, int iz, int iz1) {
+  const int* b = bin_first + g.bin0 + iz * g.nY;
+  int h1 = 0, h2 = 0;
+  StripRun r;
+  r.l1 = r.l2 = 0;
+  r.l0 = b[iy0];
+  const int h0 = b[iy1 + 1];
+  if (iz + 1 <= iz1) {
+    r.l1 = b[g.nY + iy0];
+    h1 = b[g.nY + iy1 + 1];
+  }
+  if (iz + 2 <= iz1) {
+    r.l2 = b[2 * g.nY + iy0];
+    h2 = b[2 * g.nY + iy1 + 1];
+  }
+  r.n0 = h0 - r.l0;
+  r.n1 = r.n0 + (h1 - r.l1);
+  r.n = r.n1 + (h2 - r.l2);
+  return r;
+}
+
+// for_window over such runs (the same clusters in the same order).
+template <typename Fn>
+__device__ __forceinline__ void for_window_flat(const int* __restrict__ bin_first, const RowGrid& g,
+                                           float ylo, float yhi, float zlo, float zhi, Fn&& fn) {
+  if (g.ncl == 0 || !(ylo <= yhi) || !(zlo <= zhi)) return;
+  const int iy0 = bin_of(ylo, g.y0, g.invDy, g.nY), iy1 = bin_of(yhi, g.y0, g.invDy, g.nY);
+  const int iz0 = bin_of(zlo, g.z0, g.invDz, g.nZ), iz1 = bin_of(zhi, g.z0, g.invDz, g.nZ);
+  for (int iz = iz0; iz <= iz1; iz += kStrips) {
+    const StripRun r = strip_run(bin_first, g, iy0, iy1, iz, iz1);
+    for (int c = 0; c < r.n; ++c) fn(r.at(c));
+  }
+}
+
 __device__ __forceinline__ int block_exscan(int v, int* sh_warp, int* total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int x = v;
