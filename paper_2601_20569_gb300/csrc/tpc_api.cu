@@ -311,6 +311,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   const long T = F.cap_tl;
   const long nmb = nrr * kMergeZ;
   ok &= dalloc(ctx, &F.st_tl, T);
+  F.tl_order = F.st_tl;  // (the sector-track list comes after the constructor)
   ok &= dalloc(ctx, &F.st_off, T);
   F.cap_pos = n + n / 4 + 4096;
   ok &= dalloc(ctx, &F.st_pos, F.cap_pos);

@@ -1305,6 +1305,20 @@ __global__ void __launch_bounds__(kBlock, 3) k_fit_stations(FrameDev F, KParams 
   }
 }
 
+// The fit tracks' order, stretch by stretch by stations (loopers stay first).
+__global__ void __launch_bounds__(kBlock) k_fit_order(FrameDev F) {
+  const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
+  if (F.cnt->err) return;
+  constexpr int kHalf = kOrdBuckets / 2;
+  for (int c0 = blockIdx.x * kOrdChunk; c0 < nf; c0 += gridDim.x * kOrdChunk)
+    order_chunk(
+        min(kOrdChunk, nf - c0), [&](int q) { return F.ft_order[c0 + q]; },
+        [&](int f) {
+          return (F.ft_looper[f] ? kHalf - 1 : -1) + min(kHalf - 1, F.ft_nst[f] * kHalf / kMaxRows);
+        },
+        F.ft_order + c0);
+}
+
 // Iterations 1 and 2 of the final fit (k_fit1, k_fit2) run as per-lane state
 // machines: every loop iteration is one station (station change, then the
 // iteration's own work, then the update) of the lane's current track, and a
@@ -1475,10 +1489,17 @@ __global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M
   float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float* store = nullptr;
   Lin L;
+  bool done = false, all_done;
   for (;;) {
+    const bool fetch = refill(phase != kFitIdle, done, all_done);
+    if (all_done) break;
     if (phase == kFitIdle) {
+      if (!fetch) continue;
       const int q = fit_next(F.cnt, kQFit12, kQFit12N, nL, nf);
-      if (q >= nf) break;
+      if (q >= nf) {
+        done = true;
+        continue;
+      }
       f = F.ft_order[q];
       lp = F.ft_looper[f] != 0;
       ns = F.ft_nst[f];
@@ -1574,10 +1595,17 @@ __global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M
   float sn[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // the next station's prediction
   uint8_t* flag = nullptr;
   Lin L;
+  bool done = false, all_done;
   for (;;) {
+    const bool fetch = refill(phase != kFit2Idle, done, all_done);
+    if (all_done) break;
     if (phase == kFit2Idle) {
+      if (!fetch) continue;
       const int q = fit_next(F.cnt, kQFit2, kQFit2N, nL, nf);
-      if (q >= nf) break;
+      if (q >= nf) {
+        done = true;
+        continue;
+      }
       f = F.ft_order[q];
       if (!F.ft_ok[f]) continue;
       lp = F.ft_looper[f] != 0;
@@ -2769,6 +2797,7 @@ int fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const unsigned g = persistent_grid(F.lc, kLFit12, sms);
   const int b = F.lc.block[kLFit12];
   k_fit_stations<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
+  k_fit_order<<<sms * 4, kBlock, 0, s>>>(F);
   // iterations 1 and 2 keep loopers and other tracks in one launch (split in
   // two parts, as iteration 3 is, they measured slower: 22.4 -> 25.1 ms per
   // batch, the two kinds of track no longer sharing the warps)
@@ -2780,7 +2809,7 @@ int fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
     k_fit2<kMap, false><<<g, b, 0, s>>>(F, P, F.map);
   }
   k_inner_cand<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
-  return 4;  // the station lists, iterations 1 and 2, the candidate search
+  return 5;  // the station lists, the order, iterations 1 and 2, the candidate search
 }
 
 int stage_fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {

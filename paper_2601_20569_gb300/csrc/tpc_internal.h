@@ -201,6 +201,7 @@ struct FrameDev {
   int* tl_rhi;
   int* tl_hits;            // [cap_tl*kMaxRows] row-indexed sorted cluster or -1
   int* tl_len;             // [cap_tl] CA chain length from the start hit
+  int* tl_order;           // [cap_tl] order in which a kernel takes the tracklets
   float* tl_seed;          // [cap_tl][kSeedF] seed state, start (sector, row), valid flag
   // a6
   unsigned long long* owner_key;  // [n] sorted index space
@@ -273,6 +274,7 @@ struct FrameDev {
   int* ft_last;            // last sector track of the chain
   int* ft_order;           // [cap_ft] order in which the fit kernels take the tracks:
                            // FP64-update loopers first, then the rest, each in list order
+                           // but for the order by length within a stretch of kOrdChunk
   int* ft_looper;          // [cap_ft] 1: |q/pT| of the chain's inner end above looper_qpt
   int* ft_key;
   int* ft_ok;

@@ -152,6 +152,58 @@ __device__ __forceinline__ int queue_next(int* q) {
   return base + __popc(mask & ((1u << lane) - 1u));
 }
 
+// Refill of the per-lane state machines (all lanes of the warp call it once per
+// loop iteration): lanes without an item wait until kRefill of them do, or until
+// no lane has one, and fetch together.  Loading an item costs as much as a step
+// or two, and run for one or two lanes at a time it would cost that in every
+// iteration.  (Two full frames, k_tl_chain / k_tl_refit / k_fit1: 0.82 / 1.07 /
+// 1.34 ms at 1, 0.51 / 0.81 / 1.05 at 8, 0.58 / 0.96 / 0.99 at 24.)
+constexpr int kRefill = 8;
+__device__ __forceinline__ bool refill(bool busy, bool done, bool& all_done) {
+  const unsigned b = __ballot_sync(0xffffffffu, busy);
+  const unsigned w = __ballot_sync(0xffffffffu, !busy && !done);
+  all_done = (b | w) == 0u;
+  return !busy && !done && (b == 0u || __popc(w) >= kRefill);
+}
+
+// Order of kOrdChunk consecutive items by length, longest first: order[base +
+// rank] = item for the chunk's items item(0..n-1), with len(i) < kOrdBuckets
+// (the longest in bucket 0; -1: nothing to do, last).  The lanes of a warp then
+// run items of one length side by side, start and end together, and still take
+// them from one stretch of the list, which keeps their cluster accesses close.
+// (By length over the whole list the lanes fill as well, but two full frames'
+// k_tl_chain and k_fit1 took 0.73 and 1.64 ms instead of 0.51 and 1.05.)
+constexpr int kOrdChunk = 4096;
+template <typename Item, typename Len>
+__device__ __forceinline__ void order_chunk(int n, Item&& item, Len&& len, int* order) {
+  constexpr int kPer = kOrdChunk / kBlock;
+  __shared__ int cnt[kOrdBuckets], sh[32];
+  static_assert(kOrdBuckets <= kBlock && kOrdChunk % kBlock == 0, "chunk shape");
+  if (threadIdx.x < kOrdBuckets) cnt[threadIdx.x] = 0;
+  __syncthreads();
+  int it[kPer], b[kPer], slot[kPer];
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const int q = j * kBlock + threadIdx.x;
+    b[j] = -1;
+    if (q < n) {
+      it[j] = item(q);
+      b[j] = kOrdBuckets - 1 - min(kOrdBuckets - 1, len(it[j]) + 1);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (b[j] >= 0) slot[j] = atomicAdd(&cnt[b[j]], 1);
+  __syncthreads();
+  const int ex = block_exscan(threadIdx.x < kOrdBuckets ? cnt[threadIdx.x] : 0, sh, nullptr);
+  if (threadIdx.x < kOrdBuckets) cnt[threadIdx.x] = ex;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (b[j] >= 0) order[cnt[b[j]] + slot[j]] = it[j];
+  __syncthreads();
+}
+
 // Scheduling order from per-item buckets: order[start of bucket b + slot] = i
 // for the first min(*n, cap) items.  Every block scans the kOrdBuckets counts
 // in shared memory.  The order only decides which item a thread takes next;
