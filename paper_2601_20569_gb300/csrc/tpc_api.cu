@@ -301,7 +301,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.tl_nkept, F.cap_tl);
   ok &= dalloc(ctx, &F.tl_kept, F.cap_tl * kMaxRows);
   ok &= dalloc(ctx, &F.sec_owner, n);
-  ok &= dalloc(ctx, &F.sused, n);
+  ok &= dalloc(ctx, &F.sused, n + 3);  // (cleared in words)
   ok &= dalloc(ctx, &F.cr_flags, n);
   ok &= dalloc(ctx, &F.cr_out, n);
   ok &= dalloc(ctx, &F.cr_bin_cnt, kCrBins + 1);
@@ -378,14 +378,13 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.ft_cand, FT * NS * kMaxCand);
   ok &= dalloc(ctx, &F.ft_cchi, FT * NS * kMaxCand);
   ok &= dalloc(ctx, &F.ft_assigned, FT * NS);
-  ok &= dalloc(ctx, &F.ft_newly, FT * NS);
   ok &= dalloc(ctx, &F.ft_next, FT);
   ok &= dalloc(ctx, &F.ft_nout, FT);
   ok &= dalloc(ctx, &F.ft_ext_sec, FT * (opt->ext_rows > 0 ? 2 * opt->ext_rows : 1));
   ok &= dalloc(ctx, &F.ft_ipol, FT * kMaxInner * kIpolF);
-  ok &= dalloc(ctx, &F.ft_fixed, n);
+  ok &= dalloc(ctx, &F.ft_fixed, n + 3);  // (cleared in words)
   ok &= dalloc(ctx, &F.bid, n);
-  ok &= dalloc(ctx, &F.taken, n);
+  ok &= dalloc(ctx, &F.taken, n + 3);  // (cleared in words)
   ok &= dalloc(ctx, &F.ft_n, FT);
   ok &= dalloc(ctx, &F.ft_chi2, FT);
   ok &= dalloc(ctx, &F.ft_out, FT * kStateF);
@@ -416,6 +415,14 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   if (!ok) {
     tpc_destroy(ctx);
     return TPC_ERR_OOM;
+  }
+  // kept by the chain itself from call to call: zero bin counts (k_row_scan),
+  // empty bids (k_amb_resolve)
+  if (cudaMemset(F.bin_cnt, 0, sizeof(int) * (F.cap_bins + 1)) != cudaSuccess ||
+      cudaMemset(F.bid, 0xFF, sizeof(unsigned long long) * n) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess) {
+    tpc_destroy(ctx);
+    return TPC_ERR_CUDA;
   }
   if (cudaMemcpy((void*)F.row_x, geo->row_x, sizeof(float) * geo->n_rows,
                  cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -448,27 +455,8 @@ namespace {
 // per-call parameters Pc; returns the number of kernels.  No host sync.
 tpc_status enqueue_chain(tpc_ctx* ctx, FrameDev& F, const KParams& Pc, cudaStream_t s,
                          bool events, long* launches) {
-  const long nrr = (long)Pc.n_sectors * ctx->n_rows;
-  const long n = F.n;
-  CK(cudaMemsetAsync(F.cnt, 0, sizeof(Counters), s));
-  CK(cudaMemsetAsync(F.row_cnt, 0, sizeof(int) * nrr, s));
-  CK(cudaMemsetAsync(F.row_zmin, 0xFF, sizeof(unsigned) * nrr, s));
-  CK(cudaMemsetAsync(F.row_zmax, 0, sizeof(unsigned) * nrr, s));
-  CK(cudaMemsetAsync(F.bin_cnt, 0, sizeof(int) * (F.cap_bins + 1), s));
-  if (n > 0) {
-    CK(cudaMemsetAsync(F.owner_key, 0, sizeof(unsigned long long) * n, s));
-    CK(cudaMemsetAsync(F.sec_owner, 0xFF, sizeof(int) * n, s));
-    CK(cudaMemsetAsync(F.bid, 0xFF, sizeof(unsigned long long) * n, s));
-    CK(cudaMemsetAsync(F.taken, 0, n, s));
-    CK(cudaMemsetAsync(F.attach, 0xFF, sizeof(int) * n, s));
-    CK(cudaMemsetAsync(F.attach_key, 0x7F, sizeof(int) * n, s));
-    if (Pc.ext_rows > 0) CK(cudaMemsetAsync(F.ft_fixed, 0, n, s));
-    if (Pc.seed_iters > 1) CK(cudaMemsetAsync(F.sused, 0, n, s));
-  }
-  CK(cudaMemsetAsync(F.ie_cnt, 0, sizeof(int) * (nrr * kMergeZ + 1), s));
-  CK(cudaMemsetAsync(F.st_ord_cnt, 0, sizeof(int) * kOrdBuckets, s));
-  CK(cudaMemsetAsync(F.out_offset, 0, sizeof(int), s));
-  long k = 0;
+  long k = ctx->opt.mode == 0 ? strict::call_init(F, Pc, ctx->sms, s)
+                              : fast::call_init(F, Pc, ctx->sms, s);
   if (events) CK(cudaEventRecord(ctx->ev[0], s));
   for (int i = 0; i < kNumStages; ++i) {
     const StageFn fn = ctx->opt.mode == 0 ? kStages[i].strict_fn : kStages[i].fast_fn;

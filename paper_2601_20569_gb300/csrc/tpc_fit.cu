@@ -192,23 +192,24 @@ __global__ void k_st_gather(FrameDev F, KParams P) {
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < NR; r += blockDim.x) rx[r] = F.row_x[r];
   __syncthreads();
-  // One warp per 32 consecutive tracks: lane j loads track j's tracklet,
-  // length and output place (all lanes at once), then the warp takes the
-  // tracks one by one, its lanes reading the whole kept list (up to kMaxRows
+  // One warp per 32 consecutive tracks (fewer where that would leave warps
+  // without work): lane j loads track j's tracklet, length and output place
+  // (all lanes at once), then the warp takes the tracks one by one, its lanes reading the whole kept list (up to kMaxRows
   // entries, all loads issued before the positions they address) and
   // writing the positions 32 at a time.
   constexpr int kChunks = (kMaxRows + 31) / 32;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
-  for (int j0 = 32 * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); j0 < ns;
-       j0 += 32 * nw) {
+  const int per = warp_share(ns, nw);
+  for (int j0 = per * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); j0 < ns;
+       j0 += per * nw) {
     int ti = 0, nk = 0, off = 0;
-    if (j0 + lane < ns) {
+    if (lane < per && j0 + lane < ns) {
       ti = F.st_tl[j0 + lane];
       nk = F.tl_nkept[ti];
       off = F.st_off[j0 + lane];
     }
-    for (int j = 0; j < 32; ++j) {
+    for (int j = 0; j < per; ++j) {
       const int tj = __shfl_sync(0xffffffffu, ti, j);
       const int nj = __shfl_sync(0xffffffffu, nk, j);
       const int oj = __shfl_sync(0xffffffffu, off, j);
@@ -851,6 +852,10 @@ __global__ void k_head_count(FrameDev F) {
 __global__ void k_head_write(FrameDev F, KParams P) {
   __shared__ int sh[32];
   const int ns = F.cnt->n_tracks;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && F.cnt->n_merged > F.cap_ft) {
+    atomicOr(&F.cnt->err, kErrCapTracks);
+    atomicMax(&F.cnt->need_tracks, F.cnt->n_merged);
+  }
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int f = F.cnt->err ? 0 : is_head(F, i, ns);
   int tot;
@@ -891,13 +896,6 @@ __global__ void k_looper_write(FrameDev F) {
   const int lr = F.scan_tmp[blockIdx.x] + block_exscan(fl, sh, &tot);  // loopers before f
   if (F.cnt->err || f >= nf) return;
   F.ft_order[fl ? lr : F.cnt->n_loopers + (f - lr)] = f;
-}
-
-__global__ void k_head_check(FrameDev F) {
-  if (F.cnt->n_merged > F.cap_ft) {
-    atomicOr(&F.cnt->err, kErrCapTracks);
-    atomicMax(&F.cnt->need_tracks, F.cnt->n_merged);
-  }
 }
 
 // Next fit track for the calling lane from the two queues of a fit kernel:
@@ -1191,8 +1189,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_fit_stations(FrameDev F, KParams 
   const int NR = P.n_rows;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
-  // tracks per warp: 32, fewer where that would leave warps without work
-  const int per = max(1, min(32, (nf + nw - 1) / nw));
+  const int per = warp_share(nf, nw);
   for (int f0 = per * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); f0 < nf;
        f0 += per * nw) {
     const int f = f0 + lane;
@@ -1760,30 +1757,14 @@ __global__ void k_amb_bid(FrameDev F, KParams P, int round) {
   }
 }
 
-__global__ void k_amb_resolve(FrameDev F, KParams P, int round) {
-  const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
-  if (F.cnt->err) return;
-  const long tot = (long)nf * amb_per(P);
-  for (long w = (long)blockIdx.x * blockDim.x + threadIdx.x; w < tot;
-       w += (long)gridDim.x * blockDim.x) {
-    int f;
-    const long sk = amb_slot(F, P, w, f);
-    if (sk < 0) continue;
-    F.ft_newly[sk] = 0;
-    if (F.ft_assigned[sk] >= 0 || F.ft_ncand[sk] <= round) continue;
-    const int c = F.ft_cand[sk * kMaxCand + round];
-    if (F.taken[c]) continue;
-    if (F.bid[c] == pack_chi_key(F.ft_cchi[sk * kMaxCand + round], F.ft_key[f])) {
-      F.ft_assigned[sk] = c;
-      F.ft_newly[sk] = 1;
-    }
-  }
-}
-
-// The last round (kLast) also brings the inner stations' measurements in line
-// with the clusters they were given, for iteration 3.
+// The round's winners: the slot whose own (chi2, track key) is the cluster's
+// lowest bid takes it, marks it taken and empties the bid again.  Keys are
+// unique per track and a track lists a cluster once, so every bid has one winner,
+// and a slot that reads the bid or the mark after its winner changed them loses,
+// as it would before.  The last round (kLast) also brings the inner stations'
+// measurements in line with the clusters they were given, for iteration 3.
 template <bool kLast, bool kMap>
-__global__ void k_amb_mark(FrameDev F, KParams P, MapDev M, int round) {
+__global__ void k_amb_resolve(FrameDev F, KParams P, MapDev M, int round) {
   if (!kMap) M.on = 0;
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   if (F.cnt->err) return;
@@ -1793,26 +1774,29 @@ __global__ void k_amb_mark(FrameDev F, KParams P, MapDev M, int round) {
     int f;
     const long sk = amb_slot(F, P, w, f);
     if (sk < 0) continue;
-    if (kLast) {
-      const int k = (int)(w % amb_per(P));
-      if (k < P.inner_rows) {
-        const int c = F.ft_assigned[sk];
-        float4* m = F.ft_meas + (long)f * kMaxRows + k;
-        if (c < 0) {
-          m->w = __uint_as_float(__float_as_uint(m->w) & ~kStHave);
-        } else if (c != F.ft_st_cl[(long)f * kMaxRows + k]) {
-          const int rs = F.ft_st_rs[(long)f * kMaxRows + k];
-          const float2 pc = F.syz[c];
-          *m = fit_meas<kMap>(M, P, rs, F.row_x[rs % P.n_rows], pc.x,
-                              track_z(pc.y, rs / P.n_rows, shift_side(F, f), F.ft_zsh[f], P),
-                              F.ft_z0[f]);
-        }
+    int got = F.ft_assigned[sk];
+    if (got < 0 && F.ft_ncand[sk] > round) {
+      const int c = F.ft_cand[sk * kMaxCand + round];
+      if (!F.taken[c] &&
+          F.bid[c] == pack_chi_key(F.ft_cchi[sk * kMaxCand + round], F.ft_key[f])) {
+        F.ft_assigned[sk] = got = c;
+        F.taken[c] = 1;
+        F.bid[c] = ~0ull;
       }
     }
-    if (F.ft_ncand[sk] <= round) continue;
-    const int c = F.ft_cand[sk * kMaxCand + round];
-    if (F.ft_newly[sk]) F.taken[c] = 1;
-    F.bid[c] = ~0ull;
+    const int k = (int)(w % amb_per(P));
+    if (kLast && k < P.inner_rows) {
+      float4* m = F.ft_meas + (long)f * kMaxRows + k;
+      if (got < 0) {
+        m->w = __uint_as_float(__float_as_uint(m->w) & ~kStHave);
+      } else if (got != F.ft_st_cl[(long)f * kMaxRows + k]) {
+        const int rs = F.ft_st_rs[(long)f * kMaxRows + k];
+        const float2 pc = F.syz[got];
+        *m = fit_meas<kMap>(M, P, rs, F.row_x[rs % P.n_rows], pc.x,
+                            track_z(pc.y, rs / P.n_rows, shift_side(F, f), F.ft_zsh[f], P),
+                            F.ft_z0[f]);
+      }
+    }
   }
 }
 
@@ -1993,12 +1977,11 @@ __global__ void k_out_write(FrameDev F, KParams P) {
   int tt, tr;
   const int et = block_exscan(fl, sh, &tt);
   const int er = block_exscan(v, sh, &tr);
-  int off = 0, key = 0, fits = 0;
   if (!fl) {
     if (f < nf) F.ft_outidx[f] = -1;
   } else {
     const int t = F.scan_tmp[2 * blockIdx.x] + et;
-    off = F.scan_tmp[2 * blockIdx.x + 1] + er;
+    const int off = F.scan_tmp[2 * blockIdx.x + 1] + er;
     F.ft_outidx[f] = t;
     const float* o = F.ft_out + (long)f * kStateF;
     for (int i = 0; i < 5; ++i) F.out_par[(long)t * 5 + i] = o[i];
@@ -2009,57 +1992,73 @@ __global__ void k_out_write(FrameDev F, KParams P) {
     F.out_chi2[t] = F.ft_chi2[f];
     F.out_ndf[t] = 2 * v - 5;
     F.out_ncl[t] = v;
-    key = F.ft_key[f];
-    F.out_key[t] = key;
+    F.out_key[t] = F.ft_key[f];
     F.out_offset[t] = off;
-    fits = (long)off + v <= F.cap_refs;
-    if (!fits) atomicOr(&F.cnt->err, kErrCapRefs);
+    if ((long)off + v > F.cap_refs) atomicOr(&F.cnt->err, kErrCapRefs);
   }
-  // Cluster lists: the warp takes its lanes' tracks one by one, its lanes
-  // over the track's clusters (the used list read innermost first, all loads
-  // issued before the ids they address), writing the input ids 32 at a time
-  // and lowering their attachment keys.
+}
+
+// Cluster lists: a warp takes its lanes' tracks one by one, its lanes over the
+// track's clusters (the used list read innermost first, all loads issued before
+// the ids they address), writing the input ids 32 at a time and lowering their
+// attachment keys.
+__global__ void k_out_lists(FrameDev F) {
+  const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
+  if (F.cnt->err) return;
   constexpr int kChunks = (kMaxRows + 31) / 32;
   const int lane = threadIdx.x & 31;
-  for (unsigned todo = __ballot_sync(0xffffffffu, fl != 0); todo; todo &= todo - 1) {
-    const int j = __ffs(todo) - 1;
-    const int fj = f - lane + j;
-    const int nj = __shfl_sync(0xffffffffu, v, j);
-    const int oj = __shfl_sync(0xffffffffu, off, j);
-    const int kj = __shfl_sync(0xffffffffu, key, j);
-    const int fitj = __shfl_sync(0xffffffffu, fits, j);
-    const int* used = F.ft_used + (long)fj * kMaxRows;
-    int u[kChunks], id[kChunks];
-#pragma unroll
-    for (int c = 0; c < kChunks; ++c) {
-      const int q = lane + 32 * c;
-      u[c] = q < nj ? used[nj - 1 - q] : -1;
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  const int per = warp_share(nf, nw);
+  for (int f0 = per * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); f0 < nf;
+       f0 += per * nw) {
+    const int f = f0 + lane;
+    int t = -1, v = 0, off = 0, key = 0;
+    if (lane < per && f < nf) t = F.ft_outidx[f];
+    if (t >= 0) {
+      v = F.ft_n[f];
+      key = F.ft_key[f];
+      off = F.out_offset[t];
     }
+    for (unsigned todo = __ballot_sync(0xffffffffu, t >= 0); todo; todo &= todo - 1) {
+      const int j = __ffs(todo) - 1;
+      const int nj = __shfl_sync(0xffffffffu, v, j);
+      const int oj = __shfl_sync(0xffffffffu, off, j);
+      const int kj = __shfl_sync(0xffffffffu, key, j);
+      const bool fits = (long)oj + nj <= F.cap_refs;
+      const int* used = F.ft_used + (long)(f0 + j) * kMaxRows;
+      int u[kChunks], id[kChunks];
 #pragma unroll
-    for (int c = 0; c < kChunks; ++c) id[c] = u[c] >= 0 ? F.sid[u[c]] : -1;
+      for (int c = 0; c < kChunks; ++c) {
+        const int q = lane + 32 * c;
+        u[c] = q < nj ? used[nj - 1 - q] : -1;
+      }
 #pragma unroll
-    for (int c = 0; c < kChunks; ++c) {
-      if (id[c] < 0) continue;
-      if (fitj) F.out_ids[oj + lane + 32 * c] = id[c];
-      atomicMin(&F.attach_key[id[c]], kj);
+      for (int c = 0; c < kChunks; ++c) id[c] = u[c] >= 0 ? F.sid[u[c]] : -1;
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) {
+        if (id[c] < 0) continue;
+        if (fits) F.out_ids[oj + lane + 32 * c] = id[c];
+        atomicMin(&F.attach_key[id[c]], kj);
+      }
     }
   }
 }
 
 // Attachment: every cluster goes to the track with the smallest key among
-// those that use it.  One warp per 32 consecutive fit tracks, taken one by
-// one with the lanes over the track's clusters.
+// those that use it.  A warp takes up to 32 consecutive fit tracks one by one,
+// the lanes over the track's clusters.
 __global__ void k_out_attach(FrameDev F, KParams P) {
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   if (F.cnt->err) return;
   constexpr int kChunks = (kMaxRows + 31) / 32;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
-  for (int f0 = 32 * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); f0 < nf;
-       f0 += 32 * nw) {
+  const int per = warp_share(nf, nw);
+  for (int f0 = per * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); f0 < nf;
+       f0 += per * nw) {
     const int f = f0 + lane;
     int t = -1, n = 0, key = 0, off = 0;
-    if (f < nf) {
+    if (lane < per && f < nf) {
       t = F.ft_outidx[f];
       if (t >= 0) {
         n = F.ft_n[f];
@@ -2782,12 +2781,11 @@ int stage_merge(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   k_head_count<<<nb_tl, kBlock, 0, s>>>(F);
   k_scan_partials<<<1, 1024, 0, s>>>(F.scan_tmp, nb_tl, &F.cnt->n_merged);
   k_head_write<<<nb_tl, kBlock, 0, s>>>(F, P);
-  k_head_check<<<1, 1, 0, s>>>(F);
   const int nb_ft = (int)blocks_for(F.cap_ft, kBlock);
   k_looper_count<<<nb_ft, kBlock, 0, s>>>(F);
   k_scan_partials<<<1, 1024, 0, s>>>(F.scan_tmp, nb_ft, &F.cnt->n_loopers);
   k_looper_write<<<nb_ft, kBlock, 0, s>>>(F);
-  return k + 10;
+  return k + 9;
 }
 
 // The fit kernels' variants: with a correction map or without, with the Phase
@@ -2820,11 +2818,10 @@ int stage_ambiguity2(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   int k = 0;
   for (int r = 0; r < P.cand_k; ++r) {
     k_amb_bid<<<sms * 8, kBlock, 0, s>>>(F, P, r);
-    k_amb_resolve<<<sms * 8, kBlock, 0, s>>>(F, P, r);
-    if (r + 1 < P.cand_k) k_amb_mark<false, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
-    else if (F.map.on) k_amb_mark<true, true><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
-    else k_amb_mark<true, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
-    k += 3;
+    if (r + 1 < P.cand_k) k_amb_resolve<false, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
+    else if (F.map.on) k_amb_resolve<true, true><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
+    else k_amb_resolve<true, false><<<sms * 8, kBlock, 0, s>>>(F, P, F.map, r);
+    k += 2;
   }
   return k;
 }
@@ -2854,8 +2851,9 @@ int stage_output(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   k_out_count<<<nb, kBlock, 0, s>>>(F, P);
   k_out_scan<<<1, 1024, 0, s>>>(F, nb);
   k_out_write<<<nb, kBlock, 0, s>>>(F, P);
+  k_out_lists<<<sms * 8, kBlock, 0, s>>>(F);
   k_out_attach<<<sms * 8, kBlock, 0, s>>>(F, P);
-  return 4;
+  return 5;
 }
 
 }  // namespace TPC_NS

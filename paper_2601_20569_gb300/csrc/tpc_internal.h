@@ -295,7 +295,6 @@ struct FrameDev {
   int* ft_cand;            // [cap_ft][nslot][kMaxCand]
   float* ft_cchi;          // [cap_ft][nslot][kMaxCand]
   int* ft_assigned;        // [cap_ft][nslot]
-  uint8_t* ft_newly;       // [cap_ft][nslot]
   int* ft_next;            // [cap_ft] rows extrapolated below the innermost station
   int* ft_nout;            // [cap_ft] rows extrapolated above the outermost station
   uint16_t* ft_ext_sec;    // [cap_ft][2 ext_rows] sector of each extrapolated row (inward,

@@ -88,6 +88,24 @@ cudaError_t scratch_address(void** out) {
   return cudaSuccess;
 }
 
+// Row radii, passed by value (a copy from the caller's pageable array would wait
+// for the host).
+struct RowX {
+  float x[kMaxRows];
+};
+
+__global__ void k_links_init(FrameDev F, RowX row_x, int n_rows, long nrr) {
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nrr) {
+    F.row_cnt[i] = 0;
+    F.row_zmin[i] = 0xFFFFFFFFu;
+    F.row_zmax[i] = 0u;
+  }
+  if (blockIdx.x > 0) return;
+  for (int k = threadIdx.x; k < n_rows; k += blockDim.x) ((float*)F.row_x)[k] = row_x.x[k];
+  for (int k = threadIdx.x; k < (int)(sizeof(Counters) / 4); k += blockDim.x) ((int*)F.cnt)[k] = 0;
+}
+
 // Sorted-order links -> caller's input-id order.  Writes nothing when the grid
 // build or the neighbour finding recorded an error: those kernels then leave
 // the sorted arrays partly unwritten, holding an earlier call's ids, which may
@@ -167,15 +185,11 @@ extern "C" tpc_status tpc_links_noalloc(const tpc_geometry* geo, const tpc_optio
   F.srec = (int4*)(b + kOffSrec);
   F.row_first = (int*)(b + kOffRowFirst);
 
-  // clear what the grid build accumulates into; copy the geometry
-  if (cudaMemsetAsync(F.cnt, 0, sizeof(Counters), s) != cudaSuccess ||
-      cudaMemsetAsync(F.row_cnt, 0, sizeof(int) * nrr, s) != cudaSuccess ||
-      cudaMemsetAsync(F.row_zmin, 0xFF, sizeof(unsigned) * nrr, s) != cudaSuccess ||
-      cudaMemsetAsync(F.row_zmax, 0, sizeof(unsigned) * nrr, s) != cudaSuccess ||
-      cudaMemsetAsync(F.bin_cnt, 0, sizeof(int) * (kNoAllocBins + 1), s) != cudaSuccess ||
-      cudaMemcpyAsync((void*)F.row_x, geo->row_x, sizeof(float) * geo->n_rows,
-                      cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return TPC_ERR_CUDA;
+  // clear what the grid build accumulates into and set the geometry in one
+  // launch (the bin counts are zero from the start and left so by every call)
+  RowX row_x;
+  std::memcpy(row_x.x, geo->row_x, sizeof(float) * geo->n_rows);
+  k_links_init<<<(unsigned)((nrr + 255) / 256), 256, 0, s>>>(F, row_x, geo->n_rows, nrr);
   int sms = 1;
   int dev = 0;
   cudaGetDevice(&dev);

@@ -58,17 +58,22 @@ __global__ void k_row_stats(FrameDev F, KParams P) {
 }
 
 // The same statistics with each block's share of them gathered in shared
-// memory first.  A block takes kRowStatsChunk consecutive input clusters,
+// memory first.  A block takes `chunk` consecutive input clusters,
 // which lie (all but a block at a frame boundary) in one frame, and keeps
 // count, z minimum and z maximum of that frame's W rows in shared memory;
 // clusters of another frame go to global memory directly.  Then one global
 // update per row the block has seen.  The statistics are a sum, a minimum and
 // a maximum, so the result does not depend on the order of the updates.
+// Chunks are as long as leaves every SM one, within these bounds (a chunk's
+// shared-memory rows are cleared and flushed once, which costs as much as a few
+// thousand clusters; with 32,768 clusters each the 57 chunks of a central event
+// took 87 us).
 constexpr int kRowStatsChunk = 256 * 128;
+constexpr int kRowStatsMin = 256 * 16;
 constexpr int kRowStatsMaxRows = 6144;  // W * 12 bytes of shared memory per block
 bool g_row_stats_shared = false;        // the kernel's shared-memory size is allowed
 
-__global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int W) {
+__global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int W, int chunk) {
   extern __shared__ unsigned rs_sh[];
   unsigned* cnt = rs_sh;
   unsigned* zlo = rs_sh + W;
@@ -78,8 +83,8 @@ __global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int
     zlo[w] = 0xFFFFFFFFu;
     zhi[w] = 0u;
   }
-  const long c0 = (long)blockIdx.x * kRowStatsChunk;
-  const long c1 = min((long)F.n, c0 + kRowStatsChunk);
+  const long c0 = (long)blockIdx.x * chunk;
+  const long c1 = min((long)F.n, c0 + chunk);
   int f0 = 0;  // frame of the chunk's first cluster
   if (F.nsrc > 0) {
     int lo = 0, hi = F.nsrc - 1;
@@ -124,68 +129,63 @@ __global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int
   }
 }
 
-// One block: bin layout of every (sector,row) and the row/bin offsets.
-__global__ void k_row_grid(FrameDev F, KParams P) {
+// One block: bin layout of every (sector,row) and the row/bin offsets.  A thread
+// lays out consecutive rows, one block scan over the threads' sums gives the
+// offsets (a scan per 1024 rows, with its barriers, took 13 us for a frame).
+__global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
   __shared__ int sh[32];
-  __shared__ int carry_bins, carry_cl;
   const int nrr = P.n_sectors * P.n_rows;
-  if (threadIdx.x == 0) carry_bins = carry_cl = 0;
-  __syncthreads();
-  for (int base = 0; base < nrr; base += blockDim.x) {
-    const int rr = base + threadIdx.x;
+  const int per = (nrr + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int lo = min(nrr, (int)threadIdx.x * per), hi = min(nrr, lo + per);
+  int nb = 0, nc = 0;  // bins and clusters of the thread's rows
+  for (int rr = lo; rr < hi; ++rr) {
     RowGrid g{};
-    int nb = 0, cnt = 0;
-    if (rr < nrr) {
-      const int r = rr % P.n_rows;
-      cnt = F.row_cnt[rr];
-      const float x = F.row_x[r];
-      const float ymax = x * P.tan_half + 0.5f;
-      int nZ = 1;
-      float zlo = 0.0f, zr = 0.0f;
-      if (cnt > 0) {
-        zlo = o2f(F.row_zmin[rr]);
-        zr = o2f(F.row_zmax[rr]) - zlo;
-      }
-      // about square bins holding grid_occ clusters each (0.5), at least grid_dy
-      // wide in y: the search windows (a few cm in y and in z) then cover few
-      // bins and few clusters outside the window
-      const float side = sqrtf(2.0f * ymax * fmaxf(zr, 1.0f) * P.grid_occ / (float)max(cnt, 1));
-      int nY = (int)(2.0f * ymax / fmaxf(side, P.grid_dy));
-      nY = clampi(nY, 1, 64);
-      g.nY = nY;
-      g.y0 = -ymax;
-      g.invDy = (float)nY / (2.0f * ymax);
-      if (cnt > 0) {
-        const float want = ceilf((float)cnt / ((float)nY * P.grid_occ));
-        const float zmax_bins = floorf(zr) + 1.0f;  // bins of at least ~1 cm
-        nZ = (int)fminf(fminf(want, zmax_bins), (float)((1 << 20) / nY));
-        nZ = max(nZ, 1);
-      }
-      g.nZ = nZ;
-      g.z0 = zlo;
-      g.invDz = zr > 0.0f ? (float)nZ / zr : 0.0f;
-      g.ncl = cnt;
-      nb = nY * nZ;
+    const int r = rr % P.n_rows;
+    const int cnt = F.row_cnt[rr];
+    const float x = F.row_x[r];
+    const float ymax = x * P.tan_half + 0.5f;
+    int nZ = 1;
+    float zlo = 0.0f, zr = 0.0f;
+    if (cnt > 0) {
+      zlo = o2f(F.row_zmin[rr]);
+      zr = o2f(F.row_zmax[rr]) - zlo;
     }
-    int tot_b, tot_c;
-    const int ob = block_exscan(nb, sh, &tot_b);
-    const int oc = block_exscan(cnt, sh, &tot_c);
-    if (rr < nrr) {
-      g.bin0 = carry_bins + ob;
-      F.rows[rr] = g;
-      F.row_first[rr] = carry_cl + oc;
+    // about square bins holding grid_occ clusters each (0.5), at least grid_dy
+    // wide in y: the search windows (a few cm in y and in z) then cover few
+    // bins and few clusters outside the window
+    const float side = sqrtf(2.0f * ymax * fmaxf(zr, 1.0f) * P.grid_occ / (float)max(cnt, 1));
+    int nY = (int)(2.0f * ymax / fmaxf(side, P.grid_dy));
+    nY = clampi(nY, 1, 64);
+    g.nY = nY;
+    g.y0 = -ymax;
+    g.invDy = (float)nY / (2.0f * ymax);
+    if (cnt > 0) {
+      const float want = ceilf((float)cnt / ((float)nY * P.grid_occ));
+      const float zmax_bins = floorf(zr) + 1.0f;  // bins of at least ~1 cm
+      nZ = (int)fminf(fminf(want, zmax_bins), (float)((1 << 20) / nY));
+      nZ = max(nZ, 1);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      carry_bins += tot_b;
-      carry_cl += tot_c;
-    }
-    __syncthreads();
+    g.nZ = nZ;
+    g.z0 = zlo;
+    g.invDz = zr > 0.0f ? (float)nZ / zr : 0.0f;
+    g.ncl = cnt;
+    g.bin0 = nb;
+    F.rows[rr] = g;
+    F.row_first[rr] = nc;
+    nb += nY * nZ;
+    nc += cnt;
+  }
+  int tot_b, tot_c;
+  const int ob = block_exscan(nb, sh, &tot_b);
+  const int oc = block_exscan(nc, sh, &tot_c);
+  for (int rr = lo; rr < hi; ++rr) {
+    F.rows[rr].bin0 += ob;
+    F.row_first[rr] += oc;
   }
   if (threadIdx.x == 0) {
-    F.row_first[nrr] = carry_cl;
-    F.cnt->n_bins = carry_bins;
-    if (carry_bins > F.cap_bins) atomicOr(&F.cnt->err, kErrCapBins);
+    F.row_first[nrr] = tot_c;
+    F.cnt->n_bins = tot_b;
+    if (tot_b > F.cap_bins) atomicOr(&F.cnt->err, kErrCapBins);
   }
 }
 
@@ -214,33 +214,32 @@ __global__ void k_scatter(FrameDev F) {
 
 // First sorted cluster of every bin: one block per row scans the row's bin
 // counts from the row's first cluster (the rows' bins and clusters are both
-// laid out row after row), so the scan covers the bins in use only.
+// laid out row after row), so the scan covers the bins in use only.  It leaves
+// the counts at zero for the next call (they are zero from the start, and only
+// bins in use are counted), and writes the (sector, row) of the row's sorted
+// clusters, which are contiguous, in order (rather than the scatter adding
+// another scattered store per cluster).
 __global__ void k_row_scan(FrameDev F) {
   __shared__ int sh[32];
   if (F.cnt->err) return;  // the same for the whole block
   const int rr = blockIdx.x;
   const RowGrid g = F.rows[rr];
   const int nb = g.nY * g.nZ;
-  int base = F.row_first[rr];
+  const int first = F.row_first[rr];
+  int base = first;
   for (int j0 = 0; j0 < nb; j0 += blockDim.x) {
     const int j = j0 + threadIdx.x;
     const int c = j < nb ? F.bin_cnt[g.bin0 + j] : 0;
     int tot;
     const int ex = block_exscan(c, sh, &tot);
-    if (j < nb) F.bin_first[g.bin0 + j] = base + ex;
+    if (j < nb) {
+      F.bin_first[g.bin0 + j] = base + ex;
+      F.bin_cnt[g.bin0 + j] = 0;
+    }
     base += tot;
   }
   if (rr == gridDim.x - 1 && threadIdx.x == 0) F.bin_first[g.bin0 + nb] = base;
-}
-
-// (sector, row) of every sorted cluster: a row's clusters are contiguous in
-// the sorted order, so one block per row writes its range in order (rather
-// than the scatter adding another scattered store per cluster).
-__global__ void k_row_fill(FrameDev F) {
-  if (F.cnt->err) return;
-  const int rr = blockIdx.x;
-  const int lo = F.row_first[rr], hi = F.row_first[rr + 1];
-  for (int k = lo + threadIdx.x; k < hi; k += blockDim.x) F.srow[k] = (uint16_t)rr;
+  for (int k = first + threadIdx.x; k < first + g.ncl; k += blockDim.x) F.srow[k] = (uint16_t)rr;
 }
 
 // Order the clusters of each bin by input id (deterministic layout) and
@@ -768,7 +767,15 @@ __global__ void k_start_count(FrameDev F) {
 __global__ void k_start_write(FrameDev F) {
   __shared__ int sh[32];
   __shared__ int off;
-  if (F.cnt->err) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int ns = F.cnt->tl_base + F.cnt->n_new;
+    F.cnt->n_starts = ns;
+    if (ns > F.cap_tl) {
+      atomicOr(&F.cnt->err, kErrCapTracklets);
+      atomicMax(&F.cnt->need_tracklets, ns);
+    }
+  }
+  if (F.cnt->err) return;  // (differing between blocks only where the call fails)
   const long base = (long)blockIdx.x * blockDim.x * kCompactItems;
   if (threadIdx.x == 0) off = F.cnt->tl_base + F.scan_tmp[blockIdx.x];
   __syncthreads();
@@ -782,14 +789,6 @@ __global__ void k_start_write(FrameDev F) {
     __syncthreads();
     if (threadIdx.x == 0) off += tot;
     __syncthreads();
-  }
-}
-
-__global__ void k_start_check(FrameDev F) {
-  F.cnt->n_starts = F.cnt->tl_base + F.cnt->n_new;
-  if (F.cnt->n_starts > F.cap_tl) {
-    atomicOr(&F.cnt->err, kErrCapTracklets);
-    atomicMax(&F.cnt->need_tracklets, F.cnt->n_starts);
   }
 }
 
@@ -1656,6 +1655,63 @@ void init_attributes() {
                                             kRowStatsMaxRows * 12) == cudaSuccess;
 }
 
+// Buffers that a call accumulates into, set for it in one launch: counters, row
+// statistics, scheduling and merge-index counts, and per cluster the owner keys
+// and attachments.  (As a dozen memsets they cost a call without a graph some
+// 30 us of launches.)
+namespace {
+struct InitSeg {
+  unsigned* p;   // 4-byte words (cudaMalloc'd: 16-byte aligned), or bytes in words rounded up
+  long words;
+  unsigned v;
+};
+constexpr int kInitSegs = 14;
+struct InitList {
+  InitSeg s[kInitSegs];
+  int n;
+};
+
+__global__ void __launch_bounds__(kBlock) k_call_init(InitList L) {
+  const long t0 = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long step = (long)gridDim.x * blockDim.x;
+  for (int i = 0; i < L.n; ++i) {
+    const unsigned v = L.s[i].v;
+    const long n4 = L.s[i].words >> 2;
+    uint4* p4 = (uint4*)L.s[i].p;
+    for (long q = t0; q < n4; q += step) p4[q] = make_uint4(v, v, v, v);
+    for (long q = 4 * n4 + t0; q < L.s[i].words; q += step) L.s[i].p[q] = v;
+  }
+}
+}  // namespace
+
+int call_init(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+  const long n = F.n, nrr = (long)P.n_sectors * P.n_rows;
+  InitList L;
+  L.n = 0;
+  auto add = [&](void* p, long bytes, unsigned v) {
+    if (p && bytes > 0) L.s[L.n++] = InitSeg{(unsigned*)p, (bytes + 3) / 4, v};
+  };
+  add(F.cnt, sizeof(Counters), 0u);
+  add(F.row_cnt, 4 * nrr, 0u);
+  add(F.row_zmin, 4 * nrr, 0xFFFFFFFFu);
+  add(F.row_zmax, 4 * nrr, 0u);
+  add(F.st_ord_cnt, 4 * kOrdBuckets, 0u);
+  add(F.out_offset, 4, 0u);
+  add(F.ie_cnt, 4 * (nrr * kMergeZ + 1), 0u);
+  add(F.owner_key, 8 * n, 0u);
+  add(F.sec_owner, 4 * n, 0xFFFFFFFFu);
+  add(F.attach, 4 * n, 0xFFFFFFFFu);
+  add(F.attach_key, 4 * n, 0x7F7F7F7Fu);
+  add(F.taken, n, 0u);
+  if (P.ext_rows > 0) add(F.ft_fixed, n, 0u);
+  if (P.seed_iters > 1) add(F.sused, n, 0u);
+  long words = 0;
+  for (int i = 0; i < L.n; ++i) words += L.s[i].words;
+  k_call_init<<<(unsigned)min((long)sms * 8, (long)blocks_for(words, 8 * kBlock)), kBlock, 0, s>>>(
+      L);
+  return 1;
+}
+
 // Stage launchers; each returns the number of kernels it enqueued.
 int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const long n = F.n;
@@ -1663,7 +1719,9 @@ int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   // rows of one frame: the window of the shared-memory statistics
   const int W = (F.nsrc > 0 ? F.src_nsec : P.n_sectors) * P.n_rows;
   if (n > 0 && g_row_stats_shared && W <= kRowStatsMaxRows) {
-    k_row_stats_sh<<<blocks_for(n, kRowStatsChunk), 256, (size_t)W * 12, s>>>(F, P, W);
+    const int chunk = (int)max((long)kRowStatsMin,
+                               min((long)kRowStatsChunk, (n + sms - 1) / sms));
+    k_row_stats_sh<<<blocks_for(n, chunk), 256, (size_t)W * 12, s>>>(F, P, W, chunk);
     ++k;
   } else if (n > 0) {
     k_row_stats<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F, P);
@@ -1676,8 +1734,7 @@ int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   if (n > 0) {
     k_scatter<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F);
     k_bin_sort<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F);
-    k_row_fill<<<P.n_sectors * P.n_rows, 128, 0, s>>>(F);
-    k += 3;
+    k += 2;
   }
   return k;
 }
@@ -1698,8 +1755,7 @@ int stage_starts(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   k_start_count<<<nb, kBlock, 0, s>>>(F);
   k_scan_partials<<<1, 1024, 0, s>>>(F.scan_tmp, nb, &F.cnt->n_new);
   k_start_write<<<nb, kBlock, 0, s>>>(F);
-  k_start_check<<<1, 1, 0, s>>>(F);
-  return 4;
+  return 3;
 }
 
 // The tracklet constructor of one sector-tracking iteration.  Chains and refits
@@ -1758,11 +1814,10 @@ int stage_reseed(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
     k_start_count<<<nb, kBlock, 0, s>>>(F);
     k_scan_partials<<<1, 1024, 0, s>>>(F.scan_tmp, nb, &F.cnt->n_new);
     k_start_write<<<nb, kBlock, 0, s>>>(F);
-    k_start_check<<<1, 1, 0, s>>>(F);
     k += launch_tracklets<true>(F, P, sms, s);
     k_sel_owner<<<sms * 8, kBlock, 0, s>>>(F, P);
     k_sel_walk<<<sms * 8, kBlock, 0, s>>>(F, P);
-    k += 11;
+    k += 10;
   }
   return k;
 }

@@ -138,6 +138,13 @@ __global__ void k_scan_partials(int* part, int nparts, int* total) {
   if (threadIdx.x == 0) *total = carry;
 }
 
+// Items per warp of the kernels whose warps take up to 32 items, their headers
+// loaded by the lanes side by side, one after the other: fewer where 32 would
+// leave warps without work (the items of a warp are a serial chain).
+__device__ __forceinline__ int warp_share(int n, int warps) {
+  return max(1, min(32, (n + warps - 1) / warps));
+}
+
 // Device-side work queue: each call hands the calling lanes the next item
 // indices of the queue (one atomic per warp), so uneven items (tracklets of
 // 3..150 rows, sectors of 10x different occupancy) balance dynamically across
