@@ -769,6 +769,7 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
     ok &= dalloc(ctx, &R.raw, NR);
     ok &= dalloc(ctx, &R.meas, NR);
     ok &= dalloc(ctx, &R.queue, kRefitQueues);
+    ok &= dalloc(ctx, &R.order, T);
     ok &= dalloc(ctx, &R.acc, NR);
     ok &= dalloc(ctx, &R.z0, T);
     ok &= dalloc(ctx, &R.ckpt, T * 3 * kCkptSeg * kCkptF);

@@ -246,18 +246,18 @@ __global__ void k_st_gather(FrameDev F, KParams P) {
 // because what bounds the kernel is the serial chain of a track's steps: as
 // two nested loops per track the lanes of a warp did not reconverge between
 // tracks and passes of unequal length, and a step cost 5 us instead of 0.8.
-__global__ void __launch_bounds__(256) k_sector_refit(FrameDev F, KParams P) {
+__global__ void __launch_bounds__(256) k_sector_refit(FrameDev F, KParams P, int stat) {
   const int ns = F.cnt->n_tracks;
   if (F.cnt->err) return;
   const int NR = P.n_rows;
-  bool busy = false, inward = false;
+  bool busy = false, inward = false, first = true;
   int i = 0, sec = 0, nk = 0, left = 0;
   const float4* pos = nullptr;
   float4 nxt;
   Trk<float> t;
   for (;;) {
     if (!busy) {
-      const int q = queue_next(&F.cnt->queue[kQSectorRefit]);
+      const int q = next_item(&F.cnt->queue[kQSectorRefit], first, stat);
       if (q >= ns) break;
       i = F.st_order[q];
       const int ti = F.st_tl[i];
@@ -869,11 +869,11 @@ __global__ void k_head_write(FrameDev F, KParams P) {
 }
 
 // Processing order of the fit kernels: a stable partition of the fit tracks,
-// loopers first.  On this GPU an FP64 update costs the whole warp the FP64
-// pipe's time even when only one lane needs it, so loopers share warps; each
-// part keeps list order (sector-major), which keeps the cluster accesses of a
-// warp close together.  The two parts are served by two work queues (see
-// fit_next).  No result depends on the order.
+// loopers first.  A looper's update costs its whole warp about twice the other
+// update's time, so loopers share warps, and the longer work starts first; each
+// part keeps list order (sector-major) but for the order by stations within a
+// stretch (k_fit_order), which keeps the cluster accesses of a warp close
+// together.  No result depends on the order.
 __device__ __forceinline__ int looper_flag(const FrameDev& F, int f) {
   const int nf = min(F.cnt->n_merged, (int)F.cap_ft);
   return (!F.cnt->err && f < nf) ? F.ft_looper[f] : 0;
@@ -898,46 +898,25 @@ __global__ void k_looper_write(FrameDev F) {
   F.ft_order[fl ? lr : F.cnt->n_loopers + (f - lr)] = f;
 }
 
-// Next fit track for the calling lane from the two queues of a fit kernel:
-// loopers hold ft_order[0, nL), the other tracks ft_order[nL, nf).  Half of
-// the warps (chosen pseudo-randomly over the grid) serve the looper queue
-// first, the rest the other queue first; each turns to the other queue when
-// its own is empty, so that the (narrow) FP64 pipe is in use while the other
-// tracks are fitted rather than only at one end of the kernel.  Returns nf
-// when both queues are empty.
-__device__ __forceinline__ int fit_next(Counters* cnt, int qL, int qN, int nL, int nf) {
-  const unsigned gw = (unsigned)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const bool looper_home = nL > 0 && ((gw * 2654435761u) >> 31) == 0u;
-  if (looper_home) {
-    const int q = queue_next(&cnt->queue[qL]);
-    if (q < nL) return q;
-    const int r = nL + queue_next(&cnt->queue[qN]);
-    return r < nf ? r : nf;
-  }
-  const int r = nL + queue_next(&cnt->queue[qN]);
-  if (r < nf) return r;
-  const int q = nL > 0 ? queue_next(&cnt->queue[qL]) : nL;
-  return q < nL ? q : nf;
+// The fit kernels take ft_order: loopers in [0, nL), the other tracks in [nL,
+// nf).  Iteration 3 comes in three parts: kPart 0 takes all, 1 the other tracks
+// only, 2 the loopers only.  Part 1 carries no looper update, so it fits in 80
+// registers and keeps half as many warps again in flight as the full kernel:
+// two launches are the faster form where a kernel's time is its throughput
+// (iteration 3 of two full frames: 0.77 ms, one launch 0.87), one launch where it
+// is the longest track's chain of steps (a central event: 0.28 against 0.16 ms),
+// which the second launch would wait for again.
+//
+// Parts 0 and iterations 1 and 2 number the other tracks from the next multiple
+// of 32 on, so that no warp starts with both kinds (on a frame of a few dozen
+// tracks every warp would, and pay for both updates in each step).
+__device__ __forceinline__ int fit_total(int nL, int nf) { return nf + ((32 - (nL & 31)) & 31); }
+__device__ __forceinline__ int fit_position(int q, int nL) {  // -1: no track
+  const int pad = (32 - (nL & 31)) & 31;
+  return q < nL ? q : q < nL + pad ? -1 : q - pad;
 }
 
-// The fit kernels come in three parts: kPart 0 takes both queues (fit_next),
-// 1 the other tracks only, 2 the loopers only.  Without a correction map
-// iteration 3 runs as part 1 then part 2: part 1 carries neither the looper
-// update nor the map evaluation, so it fits in 80 registers and keeps half
-// as many warps again in flight as the full kernel (iteration 3: 6.7 -> 5.3
-// ms per batch).  The order of the tracks changes no result.
-template <int kPart>
-__device__ __forceinline__ int fit_next_part(Counters* cnt, int qL, int qN, int nL, int nf) {
-  if (kPart == 1) {
-    const int r = nL + queue_next(&cnt->queue[qN]);
-    return r < nf ? r : nf;
-  }
-  if (kPart == 2) {
-    const int q = queue_next(&cnt->queue[qL]);
-    return q < nL ? q : nf;
-  }
-  return fit_next(cnt, qL, qN, nL, nf);
-}
+constexpr long kFit3Split = 4000000;  // clusters of a call from which on iteration 3 is split
 
 // Looper flag of fit track f in part kPart (compile-time in parts 1 and 2).
 template <int kPart>
@@ -1469,7 +1448,7 @@ __device__ __forceinline__ void ext_candidates(FrameDev& F, const KParams& P, co
 // next station's record is requested one step ahead.  The end state of
 // iteration 1 goes to ft_end2 for k_fit2.
 template <bool kMap, bool kExt>
-__global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M) {
+__global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M, int stat) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1486,18 +1465,20 @@ __global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M
   float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float* store = nullptr;
   Lin L;
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     const bool fetch = refill(phase != kFitIdle, done, all_done);
     if (all_done) break;
     if (phase == kFitIdle) {
       if (!fetch) continue;
-      const int q = fit_next(F.cnt, kQFit12, kQFit12N, nL, nf);
-      if (q >= nf) {
+      const int q = next_item(&F.cnt->queue[kQFit1], first, stat);
+      if (q >= fit_total(nL, nf)) {
         done = true;
         continue;
       }
-      f = F.ft_order[q];
+      const int pos = fit_position(q, nL);
+      if (pos < 0) continue;
+      f = F.ft_order[pos];
       lp = F.ft_looper[f] != 0;
       ns = F.ft_nst[f];
       F.ft_ok[f] = 0;
@@ -1573,7 +1554,7 @@ __global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M
 enum : int { kFit2Idle = 0, kFit2St, kFit2Out };
 
 template <bool kMap, bool kExt>
-__global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M) {
+__global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M, int stat) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1592,18 +1573,20 @@ __global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M
   float sn[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // the next station's prediction
   uint8_t* flag = nullptr;
   Lin L;
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     const bool fetch = refill(phase != kFit2Idle, done, all_done);
     if (all_done) break;
     if (phase == kFit2Idle) {
       if (!fetch) continue;
-      const int q = fit_next(F.cnt, kQFit2, kQFit2N, nL, nf);
-      if (q >= nf) {
+      const int q = next_item(&F.cnt->queue[kQFit2], first, stat);
+      if (q >= fit_total(nL, nf)) {
         done = true;
         continue;
       }
-      f = F.ft_order[q];
+      const int pos = fit_position(q, nL);
+      if (pos < 0) continue;
+      f = F.ft_order[pos];
       if (!F.ft_ok[f]) continue;
       lp = F.ft_looper[f] != 0;
       ns = F.ft_nst[f];
@@ -1805,7 +1788,7 @@ __global__ void k_amb_resolve(FrameDev F, KParams P, MapDev M, int round) {
 // solving), simple cut.
 template <bool kMap, bool kExt, int kPart>
 __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
-    k_fit3(FrameDev F, KParams P, MapDev M) {
+    k_fit3(FrameDev F, KParams P, MapDev M, int stat) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1814,9 +1797,14 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
   if (F.cnt->err) return;
   const int NR = P.n_rows;
   const int nL = min(F.cnt->n_loopers, nf);
-  for (int q = fit_next_part<kPart>(F.cnt, kQFit3, kQFit3N, nL, nf); q < nf;
-       q = fit_next_part<kPart>(F.cnt, kQFit3, kQFit3N, nL, nf)) {
-    const int f = F.ft_order[q];
+  bool first = true;
+  for (;;) {
+    const int q = (kPart == 1 ? nL : 0) +
+                  next_item(&F.cnt->queue[kPart == 1 ? kQFit3N : kQFit3], first, stat);
+    if (q >= (kPart == 2 ? nL : kPart == 1 ? nf : fit_total(nL, nf))) break;
+    const int pos = kPart == 0 ? fit_position(q, nL) : q;
+    if (pos < 0) continue;
+    const int f = F.ft_order[pos];
     const bool lp = fit_looper<kPart>(F, f);  // FP64 updates (low-pT looper)
     F.ft_n[f] = 0;
     if (!F.ft_ok[f]) continue;
@@ -2180,16 +2168,33 @@ __global__ void __launch_bounds__(256, 2) k_refit_prep(RefitDev R, KParams P, in
   }
 }
 
+// Order of the tracks for the four passes, stretch by stretch: loopers (by
+// their start parameters; the passes judge at every update) first, each part by
+// clusters, so that the lanes of a warp run the same update and end together.
+__global__ void __launch_bounds__(kBlock) k_refit_order(RefitDev R, KParams P) {
+  constexpr int kHalf = kOrdBuckets / 2;
+  for (int c0 = blockIdx.x * kOrdChunk; c0 < R.n_tracks; c0 += gridDim.x * kOrdChunk)
+    order_chunk(
+        (int)min((long)kOrdChunk, R.n_tracks - c0), [&](int q) { return c0 + q; },
+        [&](int t) {
+          const int ns = max(0, min(kMaxRows, R.offset[t + 1] - R.offset[t]));
+          const bool looper =
+              P.looper_qpt > 0.0f && fabsf(R.in_par[(long)t * 5 + 4]) > P.looper_qpt;
+          return (looper ? kHalf - 1 : -1) + min(kHalf - 1, ns * kHalf / kMaxRows);
+        },
+        R.order + c0);
+}
+
 __device__ __forceinline__ float* refit_ckpt(const RefitDev& R, int t, int it, int seg) {
   return R.ckpt + (((long)t * 3 + it) * kCkptSeg + seg) * kCkptF;
 }
 
-__global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P) {
+__global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P, int stat) {
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = R.row_x[r];
   __syncthreads();
   const int half = P.n_phi;
-  bool busy = false;
+  bool busy = false, first = true;
   int t = 0, k = 0, ns = 0, sec = 0;
   const float2* raw = nullptr;
   const float4* meas = nullptr;
@@ -2198,8 +2203,9 @@ __global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P) {
   Trk<float> t0;
   for (;;) {
     if (!busy) {
-      t = queue_next(&R.queue[0]);
+      t = next_item(&R.queue[0], first, stat);
       if (t >= R.n_tracks) break;
+      t = R.order[t];
       const int o0 = R.offset[t];
       ns = R.offset[t + 1] - o0;
       if (ns < 1 || ns > kMaxRows) continue;
@@ -2249,11 +2255,11 @@ __global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P) {
 // Iteration IT of the refit (0: inward, 1: outward with the interpolation
 // flags, 2: inward with the cuts).
 template <int IT, bool kMap>
-__global__ void __launch_bounds__(128, 4) k_refit_iter(RefitDev R, KParams P, int* steps3) {
+__global__ void __launch_bounds__(128, 4) k_refit_iter(RefitDev R, KParams P, int* steps3, int stat) {
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = R.row_x[r];
   __syncthreads();
-  bool busy = false;
+  bool busy = false, first = true;
   int t = 0, j = 0, ns = 0, o0 = 0, n = 0, out_sec = 0;
   const float4* meas = nullptr;
   float4 nxt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -2264,8 +2270,9 @@ __global__ void __launch_bounds__(128, 4) k_refit_iter(RefitDev R, KParams P, in
   Trk<float> out;  // the state after the last cluster used
   for (;;) {
     if (!busy) {
-      t = queue_next(&R.queue[1 + IT]);
+      t = next_item(&R.queue[1 + IT], first, stat);
       if (t >= R.n_tracks) break;
+      t = R.order[t];
       if (R.ok[t] != IT + 1) continue;
       o0 = R.offset[t];
       ns = R.offset[t + 1] - o0;
@@ -2683,23 +2690,29 @@ __global__ void __launch_bounds__(256) k_grad_reduce(RefitDev R) {
 
 }  // namespace
 
+template <bool kMap>
+static void refit_passes(RefitDev& R, const KParams& P, int* steps3, unsigned g, int sms,
+                         cudaStream_t s) {
+  k_refit_iter<0, kMap><<<g, 128, 0, s>>>(R, P, steps3,
+                                          resident_lanes<k_refit_iter<0, kMap>>(128, 0, g, sms));
+  k_refit_iter<1, kMap><<<g, 128, 0, s>>>(R, P, steps3,
+                                          resident_lanes<k_refit_iter<1, kMap>>(128, 0, g, sms));
+  k_refit_iter<2, kMap><<<g, 128, 0, s>>>(R, P, steps3,
+                                          resident_lanes<k_refit_iter<2, kMap>>(128, 0, g, sms));
+}
+
 int refit_forward(RefitDev& R, const KParams& P, int* steps3, int sms, cudaStream_t s) {
   if (R.n_tracks <= 0) return 0;
   // (no more blocks than there are tracks for)
   const unsigned g = (unsigned)min((long)sms * 4, (long)blocks_for(R.n_tracks, 32));
   k_refit_prep<<<(unsigned)min((long)sms * 16, (long)blocks_for(R.n_tracks, 8)), 256, 0, s>>>(
       R, P, steps3);
-  k_refit_start<<<g, 128, 0, s>>>(R, P);
-  if (R.map.on) {
-    k_refit_iter<0, true><<<g, 128, 0, s>>>(R, P, steps3);
-    k_refit_iter<1, true><<<g, 128, 0, s>>>(R, P, steps3);
-    k_refit_iter<2, true><<<g, 128, 0, s>>>(R, P, steps3);
-  } else {
-    k_refit_iter<0, false><<<g, 128, 0, s>>>(R, P, steps3);
-    k_refit_iter<1, false><<<g, 128, 0, s>>>(R, P, steps3);
-    k_refit_iter<2, false><<<g, 128, 0, s>>>(R, P, steps3);
-  }
-  return 5;
+  k_refit_order<<<(unsigned)min((long)sms * 4, (long)blocks_for(R.n_tracks, kOrdChunk)), kBlock, 0,
+                  s>>>(R, P);
+  k_refit_start<<<g, 128, 0, s>>>(R, P, resident_lanes<k_refit_start>(128, 0, g, sms));
+  if (R.map.on) refit_passes<true>(R, P, steps3, g, sms, s);
+  else refit_passes<false>(R, P, steps3, g, sms, s);
+  return 6;
 }
 
 int refit_backward(RefitDev& R, const KParams& P, const int* steps3, int sms, cudaStream_t s) {
@@ -2749,7 +2762,9 @@ int stage_sector_refit(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   k_order_scatter<<<sms * 4, kBlock, 0, s>>>(F.st_obucket, F.st_oslot, F.st_ord_cnt,
                                              &F.cnt->n_tracks, F.cap_tl, &F.cnt->err, F.st_order);
   k_st_gather<<<sms * 8, kBlock, 0, s>>>(F, P);
-  k_sector_refit<<<persistent_grid(F.lc, kLSectorRefit, sms), F.lc.block[kLSectorRefit], 0, s>>>(F, P);
+  const unsigned g = persistent_grid(F.lc, kLSectorRefit, sms);
+  const int b = F.lc.block[kLSectorRefit];
+  k_sector_refit<<<g, b, 0, s>>>(F, P, resident_lanes<k_sector_refit>(b, 0, g, sms));
   return 6;
 }
 
@@ -2800,11 +2815,11 @@ int fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   // two parts, as iteration 3 is, they measured slower: 22.4 -> 25.1 ms per
   // batch, the two kinds of track no longer sharing the warps)
   if (P.ext_rows > 0) {
-    k_fit1<kMap, true><<<g, b, 0, s>>>(F, P, F.map);
-    k_fit2<kMap, true><<<g, b, 0, s>>>(F, P, F.map);
+    k_fit1<kMap, true><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit1<kMap, true>>(b, 0, g, sms));
+    k_fit2<kMap, true><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit2<kMap, true>>(b, 0, g, sms));
   } else {
-    k_fit1<kMap, false><<<g, b, 0, s>>>(F, P, F.map);
-    k_fit2<kMap, false><<<g, b, 0, s>>>(F, P, F.map);
+    k_fit1<kMap, false><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit1<kMap, false>>(b, 0, g, sms));
+    k_fit2<kMap, false><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit2<kMap, false>>(b, 0, g, sms));
   }
   k_inner_cand<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
   return 5;  // the station lists, the order, iterations 1 and 2, the candidate search
@@ -2826,18 +2841,29 @@ int stage_ambiguity2(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   return k;
 }
 
-template <bool kMap, bool kExt>
-int fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+template <bool kMap, bool kExt, int kPart>
+void launch_fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const unsigned g = persistent_grid(F.lc, kLFit3, sms);
   const int b = F.lc.block[kLFit3];
-  if constexpr (kMap && kExt) {
-    k_fit3<kMap, kExt, 0><<<g, b, 0, s>>>(F, P, F.map);
+  k_fit3<kMap, kExt, kPart><<<g, b, 0, s>>>(F, P, F.map,
+                                            resident_lanes<k_fit3<kMap, kExt, kPart>>(b, 0, g, sms));
+}
+
+template <bool kMap, bool kExt>
+int fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+  if (kMap && kExt) {  // (its part 1 would spill)
+    launch_fit3<kMap, kExt, 0>(F, P, sms, s);
     return 1;
-  } else {
-    k_fit3<kMap, kExt, 1><<<g, b, 0, s>>>(F, P, F.map);
-    k_fit3<kMap, kExt, 2><<<g, b, 0, s>>>(F, P, F.map);
-    return 2;
   }
+  if constexpr (!(kMap && kExt)) {
+    if (F.n >= kFit3Split) {
+      launch_fit3<kMap, kExt, 1>(F, P, sms, s);
+      launch_fit3<kMap, kExt, 2>(F, P, sms, s);
+      return 2;
+    }
+    launch_fit3<kMap, kExt, 0>(F, P, sms, s);
+  }
+  return 1;
 }
 
 int stage_fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {

@@ -54,10 +54,8 @@ struct LaunchCfg {
 };
 
 // Work queues: counters of the dynamic item fetching (zeroed per call).
-// The fit kernels keep two queues each: loopers (kQFit12, kQFit3) and the
-// other tracks (kQFit12N, kQFit3N).
 enum QueueSlot : int {
-  kQTracklets = 0, kQSectorRefit, kQMerge, kQFit12, kQFit3, kQFit12N, kQFit3N, kQFit2, kQFit2N,
+  kQTracklets = 0, kQSectorRefit, kQMerge, kQFit1, kQFit2, kQFit3, kQFit3N,
   kQTlDown, kQTlUp, kQTlRefit, kQNum
 };
 
@@ -360,6 +358,7 @@ struct RefitDev {
   float2* raw;             // [cap_refs] cluster y, and z in the frame of the track's innermost side
   float4* meas;            // [cap_refs] (x displacement, y, z of the corrected cluster, station
                            // word: row in bits 0..7, sector above)
+  int* order;              // [cap] order in which the filter passes take the tracks
   int* queue;              // [kRefitQueues] work-queue heads of the filter passes
   // state kept for freezing and for the adjoint
   float* ref;              // [cap][10]

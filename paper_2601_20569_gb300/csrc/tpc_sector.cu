@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(kBlock) k_tl_order(FrameDev F, KParams P) {
 // sector, so the chain's next row is known); the next link and the cluster's
 // position are requested before the propagation.  The state after the last
 // update is the state at the top hit.
-__global__ void __launch_bounds__(256, 4) k_tl_chain(FrameDev F, KParams P) {
+__global__ void __launch_bounds__(256, 4) k_tl_chain(FrameDev F, KParams P, int stat) {
   const int nst = min(F.cnt->n_starts, (int)F.cap_tl);
   const int tbase = F.cnt->tl_base;
   if (F.cnt->err) return;
@@ -973,14 +973,14 @@ __global__ void __launch_bounds__(256, 4) k_tl_chain(FrameDev F, KParams P) {
   const int* H = nullptr;  // the chain's clusters by row (k_chain_info)
   float yt = 0.0f, zt = 0.0f;  // position of the top hit
   Trk<float> t;
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     bool handover = false;
     const bool fetch = refill(busy, done, all_done);
     if (all_done) break;
     if (!busy) {
       if (!fetch) continue;
-      ti = tbase + queue_next(&F.cnt->queue[kQTracklets]);
+      ti = tbase + next_item(&F.cnt->queue[kQTracklets], first, stat);
       if (ti >= nst) {
         done = true;
         continue;
@@ -1045,7 +1045,7 @@ __global__ void __launch_bounds__(256, 4) k_tl_chain(FrameDev F, KParams P) {
 // the chain's top.  The state at the top hit and that hit's position are left
 // in tl_seed[0..5], tl_chi2 and tl_x for the downward pass.
 template <bool kLeft>
-__global__ void __launch_bounds__(256, 3) k_tl_up(FrameDev F, KParams P) {
+__global__ void __launch_bounds__(256, 3) k_tl_up(FrameDev F, KParams P, int stat) {
   extern __shared__ float tl_sh[];
   float* const S = tl_sh + threadIdx.x;
   const int BS = blockDim.x;
@@ -1064,13 +1064,13 @@ __global__ void __launch_bounds__(256, 3) k_tl_up(FrameDev F, KParams P) {
     S[6 * BS] = y;
     S[7 * BS] = z;
   };
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     const bool fetch = refill(busy, done, all_done);
     if (all_done) break;
     if (!busy) {
       if (!fetch) continue;
-      ti = tbase + queue_next(&F.cnt->queue[kQTlUp]);
+      ti = tbase + next_item(&F.cnt->queue[kQTlUp], first, stat);
       if (ti >= nst) {
         done = true;
         continue;
@@ -1162,7 +1162,7 @@ __device__ __forceinline__ void tl_down_done(const FrameDev& F, const KParams& P
 // the count go to the extension below the start (tl_n = -3; n in tl_rlo).
 constexpr int kTlRefitDone = -3;
 
-__global__ void __launch_bounds__(256, 4) k_tl_refit(FrameDev F, KParams P) {
+__global__ void __launch_bounds__(256, 4) k_tl_refit(FrameDev F, KParams P, int stat) {
   extern __shared__ float tl_sh[];
   float* const S = tl_sh + threadIdx.x;
   const int BS = blockDim.x;
@@ -1182,13 +1182,13 @@ __global__ void __launch_bounds__(256, 4) k_tl_refit(FrameDev F, KParams P) {
     for (int i = 0; i < 15; ++i) S[(5 + i) * BS] = t.c[i];
     S[20 * BS] = t.x;
   };
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     const bool fetch = refill(busy, done, all_done);
     if (all_done) break;
     if (!busy) {
       if (!fetch) continue;
-      ti = tbase + queue_next(&F.cnt->queue[kQTlRefit]);
+      ti = tbase + next_item(&F.cnt->queue[kQTlRefit], first, stat);
       if (ti >= nst) {
         done = true;
         continue;
@@ -1258,7 +1258,7 @@ __global__ void __launch_bounds__(256, 4) k_tl_refit(FrameDev F, KParams P) {
 // Downward pass, second part: extension below the start by the best cluster
 // of each row until max_miss rows in a row have none.
 template <bool kLeft>
-__global__ void __launch_bounds__(256, 3) k_tl_down(FrameDev F, KParams P) {
+__global__ void __launch_bounds__(256, 3) k_tl_down(FrameDev F, KParams P, int stat) {
   extern __shared__ float tl_sh[];
   float* const S = tl_sh + threadIdx.x;
   const int BS = blockDim.x;
@@ -1278,13 +1278,13 @@ __global__ void __launch_bounds__(256, 3) k_tl_down(FrameDev F, KParams P) {
     for (int i = 0; i < 15; ++i) S[(5 + i) * BS] = t.c[i];
     S[20 * BS] = t.x;
   };
-  bool done = false, all_done;
+  bool done = false, all_done, first = true;
   for (;;) {
     const bool fetch = refill(busy, done, all_done);
     if (all_done) break;
     if (!busy) {
       if (!fetch) continue;
-      ti = tbase + queue_next(&F.cnt->queue[kQTlDown]);
+      ti = tbase + next_item(&F.cnt->queue[kQTlDown], first, stat);
       if (ti >= nst) {
         done = true;
         continue;
@@ -1768,11 +1768,11 @@ static int launch_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t
   const unsigned g = persistent_grid(F.lc, kLTracklets, sms);
   k_chain_info<<<sms * 8, kBlock, 0, s>>>(F, P);
   k_tl_order<false><<<sms * 4, kBlock, 0, s>>>(F, P);
-  k_tl_chain<<<g, tb, 0, s>>>(F, P);
-  k_tl_up<kLeft><<<g, tb, sh, s>>>(F, P);
+  k_tl_chain<<<g, tb, 0, s>>>(F, P, resident_lanes<k_tl_chain>(tb, 0, g, sms));
+  k_tl_up<kLeft><<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_up<kLeft>>(tb, sh, g, sms));
   k_tl_order<true><<<sms * 4, kBlock, 0, s>>>(F, P);
-  k_tl_refit<<<g, tb, sh, s>>>(F, P);
-  k_tl_down<kLeft><<<g, tb, sh, s>>>(F, P);
+  k_tl_refit<<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_refit>(tb, sh, g, sms));
+  k_tl_down<kLeft><<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_down<kLeft>>(tb, sh, g, sms));
   return 7;
 }
 

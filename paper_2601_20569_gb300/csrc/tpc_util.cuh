@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "tpc_internal.h"
 
 namespace tpc {
@@ -159,6 +161,22 @@ __device__ __forceinline__ int queue_next(int* q) {
   return base + __popc(mask & ((1u << lane) - 1u));
 }
 
+// Next item of a lane: the first is the lane's own number in the grid, for the
+// `stat` lanes of the blocks that start together; every other one comes from
+// the queue, whose count starts there.  Blocks start one per SM before any SM
+// gets its second, so the first items, the longest ones, are spread evenly over
+// the SMs.  (All from the queue, the blocks that asked first took them: with the
+// 17,000 tracks of an event, too few for every lane, some schedulers had four
+// warps of filter steps and others none.)
+__device__ __forceinline__ int next_item(int* q, bool& first, int stat) {
+  if (first) {
+    first = false;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < stat) return g;
+  }
+  return stat + queue_next(q);
+}
+
 // Refill of the per-lane state machines (all lanes of the warp call it once per
 // loop iteration): lanes without an item wait until kRefill of them do, or until
 // no lane has one, and fetch together.  Loading an item costs as much as a step
@@ -236,6 +254,21 @@ __global__ void k_order_scatter(const int* __restrict__ bucket, const int* __res
 }  // namespace
 
 inline unsigned blocks_for(long n, int b) { return (unsigned)((n + b - 1) / b); }
+
+// Lanes of the blocks of kernel K (block size `block`, shared memory `smem`, a
+// function of the block size) that start together in a grid of `grid` blocks.
+template <auto K>
+inline int resident_lanes(int block, size_t smem, unsigned grid, int sms) {
+  static std::atomic<int> per_sm[kBlock / 32 + 1];  // by warps of the block; 0: not asked yet
+  std::atomic<int>& c = per_sm[min(block, kBlock) / 32];
+  int nb = c.load(std::memory_order_relaxed);
+  if (nb == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, K, block, smem) != cudaSuccess || nb < 1)
+      nb = 1;
+    c.store(nb, std::memory_order_relaxed);
+  }
+  return (int)min((long)grid, (long)nb * sms) * block;
+}
 
 // Persistent grid of a heavy kernel for launch slot `slot`.
 inline unsigned persistent_grid(const LaunchCfg& lc, int slot, int sms) {
