@@ -84,6 +84,8 @@ struct tpc_ctx {
   std::vector<void*> allocs;
   FrameDev F{};
   tpc_map map{};
+  float4* map4 = nullptr;  // the map packed for a call (tracking and refit), map4_cap points
+  long map4_cap = 0;
   Counters host_cnt{};
   cudaStream_t last_stream = nullptr;
   // refit and adjoint
@@ -111,6 +113,9 @@ tpc_status fail(tpc_ctx* c, tpc_status st, const char* fmt, ...) {
   return st;
 }
 
+// Room for the packed form of map m; false without memory.
+bool map_room(tpc_ctx* c, const tpc_map& m);
+
 template <typename T>
 bool dalloc(tpc_ctx* c, T** p, long count) {
   void* v = nullptr;
@@ -121,6 +126,22 @@ bool dalloc(tpc_ctx* c, T** p, long count) {
   }
   c->allocs.push_back(v);
   *p = (T*)v;
+  return true;
+}
+
+bool map_room(tpc_ctx* c, const tpc_map& m) {
+  const long n = m.coeff ? (long)m.n_z * m.n_r * m.n_phi : 0;
+  if (n <= c->map4_cap) return true;
+  void* v = nullptr;
+  if (cudaMalloc(&v, n * sizeof(float4)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  // (cudaFree waits for the work in flight that may read the smaller one)
+  cudaFree(c->map4);
+  c->map4 = (float4*)v;
+  c->map4_cap = n;
+  ++c->lc_version;  // captured graphs hold the pointer by value: recapture
   return true;
 }
 
@@ -282,7 +303,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.ldn, n);
   ok &= dalloc(ctx, &F.cup, n);
   ok &= dalloc(ctx, &F.cdn, n);
-  ok &= dalloc(ctx, &F.flags, n);
+  ok &= dalloc(ctx, &F.flags, n / 32 + 64);
   ok &= dalloc(ctx, &F.scan_tmp, (F.cap_bins + n) / 256 + 4096);
   ok &= dalloc(ctx, &F.starts, F.cap_tl);
   ok &= dalloc(ctx, &F.tl_par, F.cap_tl * 5);
@@ -412,6 +433,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.out_key, FT);
   ok &= dalloc(ctx, &F.attach, n);
   ok &= dalloc(ctx, &F.attach_key, n);
+  if (map) ok &= map_room(ctx, *map);
   if (!ok) {
     tpc_destroy(ctx);
     return TPC_ERR_OOM;
@@ -439,6 +461,7 @@ tpc_status tpc_set_map(tpc_ctx* ctx, const tpc_map* map) {
     if (map->coeff && (map->n_phi < 1 || map->n_r < 4 || map->n_z < 4 || !(map->r_max > map->r_min) ||
                        !(map->z_max > map->z_min)))
       return fail(ctx, TPC_ERR_INVALID_ARG, "invalid map shape");
+    if (!map_room(ctx, *map)) return fail(ctx, TPC_ERR_OOM, "map buffer");
     ctx->map = *map;
   } else {
     ctx->map = tpc_map{};
@@ -457,6 +480,7 @@ tpc_status enqueue_chain(tpc_ctx* ctx, FrameDev& F, const KParams& Pc, cudaStrea
                          bool events, long* launches) {
   long k = ctx->opt.mode == 0 ? strict::call_init(F, Pc, ctx->sms, s)
                               : fast::call_init(F, Pc, ctx->sms, s);
+  if (F.map.on) k += fast::map_pack(F.map, ctx->map4, s);
   if (events) CK(cudaEventRecord(ctx->ev[0], s));
   for (int i = 0; i < kNumStages; ++i) {
     const StageFn fn = ctx->opt.mode == 0 ? kStages[i].strict_fn : kStages[i].fast_fn;
@@ -478,6 +502,7 @@ tpc_status run_chain(tpc_ctx* ctx, FrameDev& F, int nf, cudaStream_t s, tpc_trac
   KParams Pc = ctx->P;
   Pc.n_sectors = ctx->n_sectors * nf;
   F.map = make_mapdev(ctx->map);
+  F.map.c4 = ctx->map4;
   ctx->tracked = false;
   ctx->last_nf = nf;
   ctx->last_stream = s;
@@ -803,7 +828,10 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
   R.in_zsh = in->z_shift;
   R.row_x = F.row_x;
   R.freeze = freeze ? 1 : 0;
+  if (!map_room(ctx, mp)) return fail(ctx, TPC_ERR_OOM, "map buffer");
   R.map = make_mapdev(mp);
+  R.map.c4 = ctx->map4;
+  if (R.map.on) fast::map_pack(R.map, ctx->map4, s);
   CK(cudaMemsetAsync(R.queue, 0, sizeof(int) * kRefitQueues, s));
   const int k = ctx->opt.mode == 0 ? strict::refit_forward(R, ctx->P, ctx->steps3, ctx->sms, s)
                                    : fast::refit_forward(R, ctx->P, ctx->steps3, ctx->sms, s);
@@ -1051,6 +1079,7 @@ const char* tpc_last_error(const tpc_ctx* ctx) {
 void tpc_destroy(tpc_ctx* ctx) {
   if (!ctx) return;
   for (void* p : ctx->allocs) cudaFree(p);
+  cudaFree(ctx->map4);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);

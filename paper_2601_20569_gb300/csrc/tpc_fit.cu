@@ -93,17 +93,43 @@ __device__ __forceinline__ void map_eval(const MapDev& M, const KParams& P, int 
   int pidx[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) pidx[e] = phi_index(sp.ip, e, M.nphi);
-  for (int comp = 0; comp < 3; ++comp) {
-    float acc = 0.0f;
-    for (int a = 0; a < 4; ++a)
-      for (int b = 0; b < 4; ++b) {
-        const float wzr = sp.wz[a] * sp.wr[b];
-        const float* row = M.c + (((long)comp * M.nz + (sp.iz + a)) * M.nr + (sp.ir + b)) * M.nphi;
+  // one 16-byte load per control point gives its three components (the packed
+  // map of 18 x 16 x 20 control points, 92 KB, stays in L1); each component's sum
+  // runs in the order z, r, phi
+  // (the z loop stays a loop, its weights handed down: 64 loads in flight at once
+  // would hold 160 registers)
+  float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
+  float wz = sp.wz[0], wz1 = sp.wz[1], wz2 = sp.wz[2];
+#pragma unroll 1
+  for (int a = 0; a < 4; ++a) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc = acc + wzr * sp.wp[e] * __ldg(row + pidx[e]);
+    for (int b = 0; b < 4; ++b) {
+      const float wzr = wz * sp.wr[b];
+      const float4* row = M.c4 + ((long)(sp.iz + a) * M.nr + (sp.ir + b)) * M.nphi;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float4 v = __ldg(row + pidx[e]);
+        const float w = wzr * sp.wp[e];
+        a0 = a0 + w * v.x;
+        a1 = a1 + w * v.y;
+        a2 = a2 + w * v.z;
       }
-    D[comp] = acc;
+    }
+    wz = wz1;
+    wz1 = wz2;
+    wz2 = sp.wz[3];
   }
+  D[0] = a0;
+  D[1] = a1;
+  D[2] = a2;
+}
+
+// The map's control points with their components side by side, packed anew for
+// every call (the caller may change the coefficients between calls).
+__global__ void k_map_pack(MapDev M, float4* c4) {
+  const int n = M.nz * M.nr * M.nphi;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    c4[i] = make_float4(M.c[i], M.c[n + i], M.c[2 * n + i], 0.0f);
 }
 
 // Corrected measurement projected back onto the pad row along the reference.
@@ -1689,7 +1715,10 @@ __global__ void k_inner_cand(FrameDev F, KParams P, MapDev M) {
   for (long w = (long)blockIdx.x * blockDim.x + threadIdx.x; w < tot;
        w += (long)gridDim.x * blockDim.x) {
     const int f = (int)(w / P.inner_rows), k = (int)(w % P.inner_rows);
-    if (!F.ft_ok[f] || !inner_station(F, P, f, k)) continue;
+    if (!F.ft_ok[f] || !inner_station(F, P, f, k)) {
+      F.ft_ncand[(long)f * F.nslot + k] = 0;  // (the ambiguity looks at the count only)
+      continue;
+    }
     const float* ip = F.ft_ipol + ((long)f * kMaxInner + k) * kIpolF;
     Interp I;
     I.y = ip[0];
@@ -1709,15 +1738,17 @@ __global__ void k_inner_cand(FrameDev F, KParams P, MapDev M) {
 // Work item w of the second ambiguity: (fit track, candidate slot).  Slots
 // 0..inner_rows-1 are the inner stations, the next ext_rows slots the rows
 // extrapolated below the track, the ext_rows after them the rows extrapolated
-// above it (Phase III); returns -1 for an unused slot.
+// above it (Phase III); returns -1 for an unused extrapolation slot (an unused
+// inner slot has no candidates).
 __device__ __forceinline__ int amb_per(const KParams& P) { return P.inner_rows + 2 * P.ext_rows; }
 
-__device__ __forceinline__ long amb_slot(const FrameDev& F, const KParams& P, long w, int& f) {
+__device__ __forceinline__ long amb_slot(const FrameDev& F, const KParams& P, long w, int& f,
+                                         int& k) {
   const int per = amb_per(P);
   f = (int)(w / per);
-  const int k = (int)(w % per);
+  k = (int)(w % per);
+  if (k < P.inner_rows) return (long)f * F.nslot + k;
   if (!F.ft_ok[f]) return -1;
-  if (k < P.inner_rows) return inner_station(F, P, f, k) ? (long)f * F.nslot + k : -1;
   const int e = k - P.inner_rows;
   if (e < P.ext_rows) return e < F.ft_next[f] ? (long)f * F.nslot + kMaxInner + e : -1;
   const int eo = e - P.ext_rows;
@@ -1730,10 +1761,9 @@ __global__ void k_amb_bid(FrameDev F, KParams P, int round) {
   const long tot = (long)nf * amb_per(P);
   for (long w = (long)blockIdx.x * blockDim.x + threadIdx.x; w < tot;
        w += (long)gridDim.x * blockDim.x) {
-    int f;
-    const long sk = amb_slot(F, P, w, f);
-    if (sk < 0) continue;
-    if (F.ft_assigned[sk] >= 0 || F.ft_ncand[sk] <= round) continue;
+    int f, k;
+    const long sk = amb_slot(F, P, w, f, k);
+    if (sk < 0 || F.ft_ncand[sk] <= round || F.ft_assigned[sk] >= 0) continue;
     const int c = F.ft_cand[sk * kMaxCand + round];
     if (F.taken[c]) continue;
     atomicMin(&F.bid[c], pack_chi_key(F.ft_cchi[sk * kMaxCand + round], F.ft_key[f]));
@@ -1754,11 +1784,14 @@ __global__ void k_amb_resolve(FrameDev F, KParams P, MapDev M, int round) {
   const long tot = (long)nf * amb_per(P);
   for (long w = (long)blockIdx.x * blockDim.x + threadIdx.x; w < tot;
        w += (long)gridDim.x * blockDim.x) {
-    int f;
-    const long sk = amb_slot(F, P, w, f);
+    int f, k;
+    const long sk = amb_slot(F, P, w, f, k);
     if (sk < 0) continue;
+    const bool more = F.ft_ncand[sk] > round;
+    if (!kLast && !more) continue;
+    // (an unused inner slot: ncand is 0, assigned and ft_ok stand for themselves)
     int got = F.ft_assigned[sk];
-    if (got < 0 && F.ft_ncand[sk] > round) {
+    if (more && got < 0) {
       const int c = F.ft_cand[sk * kMaxCand + round];
       if (!F.taken[c] &&
           F.bid[c] == pack_chi_key(F.ft_cchi[sk * kMaxCand + round], F.ft_key[f])) {
@@ -1767,8 +1800,7 @@ __global__ void k_amb_resolve(FrameDev F, KParams P, MapDev M, int round) {
         F.bid[c] = ~0ull;
       }
     }
-    const int k = (int)(w % amb_per(P));
-    if (kLast && k < P.inner_rows) {
+    if (kLast && k < P.inner_rows && F.ft_ok[f] && inner_station(F, P, f, k)) {
       float4* m = F.ft_meas + (long)f * kMaxRows + k;
       if (got < 0) {
         m->w = __uint_as_float(__float_as_uint(m->w) & ~kStHave);
@@ -2689,6 +2721,11 @@ __global__ void __launch_bounds__(256) k_grad_reduce(RefitDev R) {
 }
 
 }  // namespace
+
+int map_pack(const MapDev& M, float4* c4, cudaStream_t s) {
+  k_map_pack<<<blocks_for((long)M.nz * M.nr * M.nphi, 256), 256, 0, s>>>(M, c4);
+  return 1;
+}
 
 template <bool kMap>
 static void refit_passes(RefitDev& R, const KParams& P, int* steps3, unsigned g, int sms,

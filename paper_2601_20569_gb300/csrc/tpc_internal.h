@@ -114,7 +114,8 @@ struct MapDev {
   int nphi, nr, nz;
   float rmin, zmin, zmax;
   float phi_scale, r_scale, z_scale;
-  const float* c;
+  const float* c;    // [3][nz][nr][nphi]
+  const float4* c4;  // [nz][nr][nphi] (dx, dy, dz, -): packed for the call (k_map_pack)
 };
 
 // Small device-side counters read back at the end of a call.
@@ -184,7 +185,7 @@ struct FrameDev {
   int* cup;
   int* cdn;
   // a4
-  int* flags;              // [n] scratch for compaction
+  int* flags;              // [n / 32 + 64] start-hit flags, one bit per sorted cluster
   int* scan_tmp;           // block partials
   int* starts;             // [cap_tl]
   // a5

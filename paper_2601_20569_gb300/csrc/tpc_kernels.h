@@ -11,6 +11,7 @@ namespace tpc {
 // Each launcher enqueues one stage on stream s and returns its kernel count.
 #define TPC_DECLARE_LAUNCHERS                                                       \
   void init_attributes();                                                          \
+  int map_pack(const MapDev& M, float4* c4, cudaStream_t s);                      \
   int call_init(FrameDev& F, const KParams& P, int sms, cudaStream_t s);          \
   int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s);         \
   int stage_links(FrameDev& F, const KParams& P, int sms, cudaStream_t s);        \

@@ -142,10 +142,12 @@ __global__ void k_cr_legs(FrameDev F, KParams P, RemovalParams R) {
 // One tube cross-section: the clusters of batch row rr within h of (yc, zc).
 // Where protection 2 depends on the occupancy, one scan of the window that
 // covers both the occupancy window and the larger of the two possible tubes
-// counts the occupancy and lists the tube candidates (up to kCrList; a denser
-// window is scanned again once h is known).
-constexpr int kCrList = 12;
-
+// counts the occupancy and marks the clusters of both tubes.  The window's whole z
+// strips are one contiguous run of the sorted order, walked in one loop that the
+// lanes of a warp run together, with the tubes as bit masks; where it holds
+// more than 32 clusters, the bins of the window are walked strip by strip (and
+// again once h is known).  (Strip by strip with a list in local memory for all:
+// 0.60 ms on a 4e6-cluster frame.)
 __device__ __forceinline__ void cr_tube(const FrameDev& F, const KParams& P,
                                         const RemovalParams& R, int rr, float yc, float zc,
                                         bool protect) {
@@ -154,39 +156,41 @@ __device__ __forceinline__ void cr_tube(const FrameDev& F, const KParams& P,
   const float h0 = protect ? R.protect : R.remove;
   const float fac = protect ? R.p2_grow : R.p2_shrink;
   const unsigned bit = protect ? 1u : 4u;
-  float h = h0;
+  const float hg = h0 * fac, w = R.occ_w;
+  bool grown = false, by_occ = false;  // half-width hg instead of h0; by the occupancy
   if (R.mode >= 2) {
-    if (r < P.inner_rows || fabsf(yc) > F.row_x[r] * P.tan_half - R.edge) {
-      h = h0 * fac;
-    } else {
-      const float w = R.occ_w;
-      const float hg = h0 * fac;
-      const float hm = hg > h0 ? hg : h0;  // the larger tube the occupancy may select
-      const float wb = hm > w ? hm : w;
-      int occ = 0, nc = 0;
-      bool over = false;
-      int cand[kCrList];
-      for_window(F.bin_first, g, yc - wb, yc + wb, zc - wb, zc + wb, [&](int k) {
-        const float2 pk = F.syz[k];
-        const float dy = fabsf(pk.x - yc), dz = fabsf(pk.y - zc);
-        if (dy <= w && dz <= w) ++occ;
-        if (dy <= hm && dz <= hm) {
-          if (nc < kCrList)
-            cand[nc++] = k;
-          else
-            over = true;
-        }
-      });
-      if (occ > R.occ_max) h = hg;
-      if (!over) {
-        for (int j = 0; j < nc; ++j) {
-          const float2 pk = F.syz[cand[j]];
-          if (fabsf(pk.x - yc) <= h && fabsf(pk.y - zc) <= h) atomicOr(&F.cr_flags[cand[j]], bit);
-        }
-        return;
-      }
-    }
+    if (r < P.inner_rows || fabsf(yc) > F.row_x[r] * P.tan_half - R.edge) grown = true;
+    else by_occ = true;
   }
+  const float wb = by_occ ? fmaxf(w, fmaxf(h0, hg)) : grown ? hg : h0;
+  if (g.ncl == 0 || !(yc - wb <= yc + wb) || !(zc - wb <= zc + wb)) return;
+  const int iz0 = bin_of(zc - wb, g.z0, g.invDz, g.nZ), iz1 = bin_of(zc + wb, g.z0, g.invDz, g.nZ);
+  const int lo = F.bin_first[g.bin0 + iz0 * g.nY];
+  const int n = F.bin_first[g.bin0 + (iz1 + 1) * g.nY] - lo;
+  if (n <= 32) {
+    int occ = 0;
+    unsigned in0 = 0u, ing = 0u;  // within h0, within hg
+    for (int c = 0; c < n; ++c) {
+      const float2 pk = F.syz[lo + c];
+      const float dy = fabsf(pk.x - yc), dz = fabsf(pk.y - zc);
+      if (dy <= w && dz <= w) ++occ;
+      if (dy <= h0 && dz <= h0) in0 |= 1u << c;
+      if (dy <= hg && dz <= hg) ing |= 1u << c;
+    }
+    if (by_occ) grown = occ > R.occ_max;
+    for (unsigned m = grown ? ing : in0; m; m &= m - 1u)
+      atomicOr(&F.cr_flags[lo + __ffs(m) - 1], bit);
+    return;
+  }
+  if (by_occ) {
+    int occ = 0;
+    for_window(F.bin_first, g, yc - w, yc + w, zc - w, zc + w, [&](int k) {
+      const float2 pk = F.syz[k];
+      if (fabsf(pk.x - yc) <= w && fabsf(pk.y - zc) <= w) ++occ;
+    });
+    grown = occ > R.occ_max;
+  }
+  const float h = grown ? hg : h0;
   for_window(F.bin_first, g, yc - h, yc + h, zc - h, zc + h, [&](int k) {
     const float2 pk = F.syz[k];
     if (fabsf(pk.x - yc) <= h && fabsf(pk.y - zc) <= h) atomicOr(&F.cr_flags[k], bit);

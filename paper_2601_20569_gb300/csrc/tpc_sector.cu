@@ -129,16 +129,20 @@ __global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int
   }
 }
 
-// One block: bin layout of every (sector,row) and the row/bin offsets.  A thread
-// lays out consecutive rows, one block scan over the threads' sums gives the
-// offsets (a scan per 1024 rows, with its barriers, took 13 us for a frame).
+// One block: bin layout of every (sector,row) and the row/bin offsets.  A warp
+// takes a run of consecutive rows, 32 at a time with a scan of its own, and one
+// scan over the warps' sums gives the offsets (a block scan per 1024 rows, with
+// its barriers, took 13 us for a frame).
 __global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
   __shared__ int sh[32];
   const int nrr = P.n_sectors * P.n_rows;
-  const int per = (nrr + (int)blockDim.x - 1) / (int)blockDim.x;
-  const int lo = min(nrr, (int)threadIdx.x * per), hi = min(nrr, lo + per);
-  int nb = 0, nc = 0;  // bins and clusters of the thread's rows
-  for (int rr = lo; rr < hi; ++rr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int per = (nrr + 32 * nw - 1) / (32 * nw) * 32;
+  const int lo = min(nrr, warp * per), hi = min(nrr, lo + per);
+  int nb = 0, nc = 0;  // bins and clusters of the warp's rows so far
+  for (int r0 = lo; r0 < hi; r0 += 32) {
+    const int rr = min(r0 + lane, hi - 1);
+    const bool mine = r0 + lane < hi;
     RowGrid g{};
     const int r = rr % P.n_rows;
     const int cnt = F.row_cnt[rr];
@@ -169,16 +173,29 @@ __global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
     g.z0 = zlo;
     g.invDz = zr > 0.0f ? (float)nZ / zr : 0.0f;
     g.ncl = cnt;
-    g.bin0 = nb;
-    F.rows[rr] = g;
-    F.row_first[rr] = nc;
-    nb += nY * nZ;
-    nc += cnt;
+    int ib = mine ? nY * nZ : 0, ic = mine ? cnt : 0;  // inclusive scans
+    const int vb = ib, vc = ic;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int yb = __shfl_up_sync(0xffffffffu, ib, o), yc = __shfl_up_sync(0xffffffffu, ic, o);
+      if (lane >= o) {
+        ib += yb;
+        ic += yc;
+      }
+    }
+    if (mine) {
+      g.bin0 = nb + ib - vb;
+      F.rows[rr] = g;
+      F.row_first[rr] = nc + ic - vc;
+    }
+    nb += __shfl_sync(0xffffffffu, ib, 31);
+    nc += __shfl_sync(0xffffffffu, ic, 31);
   }
   int tot_b, tot_c;
-  const int ob = block_exscan(nb, sh, &tot_b);
-  const int oc = block_exscan(nc, sh, &tot_c);
-  for (int rr = lo; rr < hi; ++rr) {
+  const int eb = block_exscan(lane == 31 ? nb : 0, sh, &tot_b);
+  const int ec = block_exscan(lane == 31 ? nc : 0, sh, &tot_c);
+  const int ob = __shfl_sync(0xffffffffu, eb, 0), oc = __shfl_sync(0xffffffffu, ec, 0);
+  for (int rr = lo + lane; rr < hi; rr += 32) {
     F.rows[rr].bin0 += ob;
     F.row_first[rr] += oc;
   }
@@ -346,60 +363,19 @@ __device__ __forceinline__ void links_one(const FrameDev& F, const KParams& P, l
   }
 }
 
-// The same search over whole z strips.  A row's clusters are sorted strip by
-// strip, so the strips the window reaches are one contiguous run: two bin
-// offsets instead of two per strip, and one loop that the lanes of a warp run
-// together (neighbouring sorted clusters have neighbouring runs of nearly the
-// same length).  The clusters inside the window are kept as bit masks over the
-// runs, and the pairs of the two masks tested in a loop of their own, ids read
-// on exact ties only.  It visits a superset of the clusters links_one visits,
-// tests them alike, and the best pair is a minimum under a total order: the
-// same links.  Testing all y bins of the strips pays while they are few (a row
-// of a 2.8 ms frame has five or six): rows with more than kRunMaxY, and runs of
-// more than 32 clusters, take links_one (returns false).
-constexpr int kRunMaxY = 9;
-
-template <bool kLeft>
-__device__ __forceinline__ bool links_run(const FrameDev& F, const KParams& P, long k, int& bu,
-                                          int& bd) {
-  const int rr = F.srow[k];
-  const int r = rr % P.n_rows;
-  bu = -1;
-  bd = -1;
-  if (r < 1 || r > P.n_rows - 2 || (kLeft && F.sused[k])) return true;
-  const float2 pc = F.syz[k];
-  const float yc = pc.x, zc = pc.y;
-  const RowGrid gd = F.rows[rr - 1], gu = F.rows[rr + 1];
-  if (gd.ncl == 0 || gu.ncl == 0) return true;
-  const float m = 0.01f;
-  const float zlo = zc - P.link_wz - m, zhi = zc + P.link_wz + m;
-  if (!(zlo <= zhi)) return true;
-  const int* bf = F.bin_first;
-  const int d0 = bf[gd.bin0 + bin_of(zlo, gd.z0, gd.invDz, gd.nZ) * gd.nY];
-  const int nd = bf[gd.bin0 + (bin_of(zhi, gd.z0, gd.invDz, gd.nZ) + 1) * gd.nY] - d0;
-  const int u0 = bf[gu.bin0 + bin_of(zlo, gu.z0, gu.invDz, gu.nZ) * gu.nY];
-  const int nu = bf[gu.bin0 + (bin_of(zhi, gu.z0, gu.invDz, gu.nZ) + 1) * gu.nY] - u0;
-  if (gd.nY > kRunMaxY || gu.nY > kRunMaxY || nd > 32 || nu > 32) return false;
-  unsigned md = 0u, mu = 0u;
-  for (int c = 0; c < nd; ++c) {
-    const float2 p = F.syz[d0 + c];
-    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
-        !(kLeft && F.sused[d0 + c]))
-      md |= 1u << c;
-  }
-  if (md == 0u) return true;
-  for (int c = 0; c < nu; ++c) {
-    const float2 p = F.syz[u0 + c];
-    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
-        !(kLeft && F.sused[u0 + c]))
-      mu |= 1u << c;
-  }
+// Best pair of the clusters marked in the masks md (row below, dn(c) the sorted
+// cluster of bit c) and mu (row above): every upper with every lower one, input
+// ids read on exact ties only.
+template <typename Dn, typename Up>
+__device__ __forceinline__ void links_pairs(const FrameDev& F, const KParams& P, int r, float yc,
+                                            float zc, unsigned md, unsigned mu, Dn&& dn, Up&& up,
+                                            int& bu, int& bd) {
   const float xd = F.row_x[r - 1], xc = F.row_x[r], xu = F.row_x[r + 1];
   const float f = (xc - xd) / (xu - xd);
   float best = 0.0f;
   unsigned dm = md;
-  while (mu) {  // all pairs: the lower mask once per upper cluster
-    const int u = u0 + __ffs(mu) - 1, d = d0 + __ffs(dm) - 1;
+  while (mu) {  // the lower mask once per upper cluster
+    const int u = up(__ffs(mu) - 1), d = dn(__ffs(dm) - 1);
     const float2 pu = F.syz[u], pd = F.syz[d];
     const float yp = pd.x + (pu.x - pd.x) * f;
     const float zp = pd.y + (pu.y - pd.y) * f;
@@ -423,17 +399,115 @@ __device__ __forceinline__ bool links_run(const FrameDev& F, const KParams& P, l
       mu &= mu - 1u;
     }
   }
+}
+
+// The same search over whole z strips.  A row's clusters are sorted strip by
+// strip, so the strips the window reaches are one contiguous run: two bin
+// offsets instead of two per strip, and one loop that the lanes of a warp run
+// together (neighbouring sorted clusters have neighbouring runs of nearly the
+// same length).  The clusters inside the window are kept as bit masks over the
+// runs, and the pairs of the two masks tested in a loop of their own (links_pairs).
+// It visits a superset of the clusters links_one visits, tests them alike, and
+// the best pair is a minimum under a total order: the same links.  Testing all
+// y bins of the strips pays up to the length of a mask: longer runs take
+// links_flat (returns false).  (Two full frames / a dense central event, limit
+// 12: 1.71 / 0.14 ms, 24: 1.56 / 0.16, 32: 1.47 / 0.17.)
+constexpr int kRunWhole = 32;
+
+template <bool kLeft>
+__device__ __forceinline__ bool links_run(const FrameDev& F, const KParams& P, long k, int& bu,
+                                          int& bd) {
+  const int rr = F.srow[k];
+  const int r = rr % P.n_rows;
+  bu = -1;
+  bd = -1;
+  if (r < 1 || r > P.n_rows - 2 || (kLeft && F.sused[k])) return true;
+  const float2 pc = F.syz[k];
+  const float yc = pc.x, zc = pc.y;
+  const RowGrid gd = F.rows[rr - 1], gu = F.rows[rr + 1];
+  if (gd.ncl == 0 || gu.ncl == 0) return true;
+  const float m = 0.01f;
+  const float zlo = zc - P.link_wz - m, zhi = zc + P.link_wz + m;
+  if (!(zlo <= zhi)) return true;
+  const int* bf = F.bin_first;
+  const int d0 = bf[gd.bin0 + bin_of(zlo, gd.z0, gd.invDz, gd.nZ) * gd.nY];
+  const int nd = bf[gd.bin0 + (bin_of(zhi, gd.z0, gd.invDz, gd.nZ) + 1) * gd.nY] - d0;
+  const int u0 = bf[gu.bin0 + bin_of(zlo, gu.z0, gu.invDz, gu.nZ) * gu.nY];
+  const int nu = bf[gu.bin0 + (bin_of(zhi, gu.z0, gu.invDz, gu.nZ) + 1) * gu.nY] - u0;
+  if (nd > kRunWhole || nu > kRunWhole) return false;
+  unsigned md = 0u, mu = 0u;
+  for (int c = 0; c < nd; ++c) {
+    const float2 p = F.syz[d0 + c];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
+        !(kLeft && F.sused[d0 + c]))
+      md |= 1u << c;
+  }
+  if (md == 0u) return true;
+  for (int c = 0; c < nu; ++c) {
+    const float2 p = F.syz[u0 + c];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz &&
+        !(kLeft && F.sused[u0 + c]))
+      mu |= 1u << c;
+  }
+  links_pairs(F, P, r, yc, zc, md, mu, [&](int c) { return d0 + c; }, [&](int c) { return u0 + c; },
+              bu, bd);
   return true;
 }
 
+// The same over the window's y bins of up to kStrips strips per row, for clusters
+// that links_run leaves (dense regions, rows of many y bins).  More than 32
+// candidates or kStrips strips take links_one (returns false).
 template <bool kLeft>
-// (40 registers, held by the launch bounds; 46 without them: 1.79 against 1.63 ms
-// for two full frames)
+__device__ __forceinline__ bool links_flat(const FrameDev& F, const KParams& P, long k, int& bu,
+                                          int& bd) {
+  const int rr = F.srow[k];
+  const int r = rr % P.n_rows;
+  bu = -1;
+  bd = -1;
+  const float2 pc = F.syz[k];
+  const float yc = pc.x, zc = pc.y;
+  const RowGrid gd = F.rows[rr - 1], gu = F.rows[rr + 1];
+  const float m = 0.01f;
+  const float ylo = yc - P.link_wy - m, yhi = yc + P.link_wy + m;
+  const float zlo = zc - P.link_wz - m, zhi = zc + P.link_wz + m;
+  if (!(ylo <= yhi)) return true;
+  const int dz0 = bin_of(zlo, gd.z0, gd.invDz, gd.nZ), dz1 = bin_of(zhi, gd.z0, gd.invDz, gd.nZ);
+  const int uz0 = bin_of(zlo, gu.z0, gu.invDz, gu.nZ), uz1 = bin_of(zhi, gu.z0, gu.invDz, gu.nZ);
+  if (dz1 - dz0 >= kStrips || uz1 - uz0 >= kStrips) return false;
+  const StripRun rd = strip_run(F.bin_first, gd, bin_of(ylo, gd.y0, gd.invDy, gd.nY),
+                                bin_of(yhi, gd.y0, gd.invDy, gd.nY), dz0, dz1);
+  const StripRun ru = strip_run(F.bin_first, gu, bin_of(ylo, gu.y0, gu.invDy, gu.nY),
+                                bin_of(yhi, gu.y0, gu.invDy, gu.nY), uz0, uz1);
+  if (rd.n > 32 || ru.n > 32) return false;
+  unsigned md = 0u, mu = 0u;
+  for (int c = 0; c < rd.n; ++c) {
+    const int d = rd.at(c);
+    const float2 p = F.syz[d];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz && !(kLeft && F.sused[d]))
+      md |= 1u << c;
+  }
+  if (md == 0u) return true;
+  for (int c = 0; c < ru.n; ++c) {
+    const int u = ru.at(c);
+    const float2 p = F.syz[u];
+    if (fabsf(p.x - yc) <= P.link_wy && fabsf(p.y - zc) <= P.link_wz && !(kLeft && F.sused[u]))
+      mu |= 1u << c;
+  }
+  links_pairs(F, P, r, yc, zc, md, mu, [&](int c) { return rd.at(c); },
+              [&](int c) { return ru.at(c); }, bu, bd);
+  return true;
+}
+
+// (40 registers, held by the launch bounds; without them 46, and 10 % slower on
+// two full frames.  Two full frames: 2.13 ms with links_one for all clusters, 1.47
+// with the runs; a central event 0.23 -> 0.17 ms.)
+template <bool kLeft>
 __global__ void __launch_bounds__(kBlock) k_links(FrameDev F, KParams P) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= F.n || F.cnt->err) return;
   int bu, bd;
-  if (!links_run<kLeft>(F, P, k, bu, bd)) links_one<kLeft>(F, P, k, bu, bd);
+  if (!links_run<kLeft>(F, P, k, bu, bd) && !links_flat<kLeft>(F, P, k, bu, bd))
+    links_one<kLeft>(F, P, k, bu, bd);
   F.lup[k] = bu;
   F.ldn[k] = bd;
 }
@@ -750,6 +824,10 @@ __device__ __forceinline__ bool is_start(const FrameDev& F, long k) {
   return F.cdn[k] < 0 && u >= 0 && F.cup[u] >= 0;
 }
 
+// The count pass leaves its flags as one word per 32 clusters, from which the
+// write pass places the start hits without looking at the links again.
+static_assert(kBlock * kCompactItems == 1024, "one flag word per lane of a warp");
+
 __global__ void k_start_count(FrameDev F) {
   __shared__ int sh[32];
   const long base = (long)blockIdx.x * blockDim.x * kCompactItems;
@@ -757,7 +835,10 @@ __global__ void k_start_count(FrameDev F) {
   if (!F.cnt->err)
     for (int j = 0; j < kCompactItems; ++j) {
       const long k = base + (long)j * blockDim.x + threadIdx.x;
-      if (k < F.n && is_start(F, k)) ++c;
+      const bool f = k < F.n && is_start(F, k);
+      const unsigned m = __ballot_sync(0xffffffffu, f);
+      if ((threadIdx.x & 31) == 0) F.flags[k >> 5] = (int)m;
+      c += f;
     }
   int tot;
   block_exscan(c, sh, &tot);
@@ -765,8 +846,8 @@ __global__ void k_start_count(FrameDev F) {
 }
 
 __global__ void k_start_write(FrameDev F) {
-  __shared__ int sh[32];
-  __shared__ int off;
+  __shared__ unsigned word[32];
+  __shared__ int before[32];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int ns = F.cnt->tl_base + F.cnt->n_new;
     F.cnt->n_starts = ns;
@@ -777,18 +858,23 @@ __global__ void k_start_write(FrameDev F) {
   }
   if (F.cnt->err) return;  // (differing between blocks only where the call fails)
   const long base = (long)blockIdx.x * blockDim.x * kCompactItems;
-  if (threadIdx.x == 0) off = F.cnt->tl_base + F.scan_tmp[blockIdx.x];
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    const unsigned m = (unsigned)F.flags[(base >> 5) + lane];
+    int x = __popc(m);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    word[lane] = m;
+    before[lane] = F.cnt->tl_base + F.scan_tmp[blockIdx.x] + x - __popc(m);
+  }
   __syncthreads();
-  for (int j = 0; j < kCompactItems; ++j) {
-    const long k = base + (long)j * blockDim.x + threadIdx.x;
-    const int flag = (k < F.n && is_start(F, k)) ? 1 : 0;
-    int tot;
-    const int ex = block_exscan(flag, sh, &tot);
-    const int pos = off + ex;
-    if (flag && pos < F.cap_tl) F.starts[pos] = (int)k;
-    __syncthreads();
-    if (threadIdx.x == 0) off += tot;
-    __syncthreads();
+  for (int w = threadIdx.x >> 5; w < 32; w += blockDim.x >> 5) {
+    const unsigned m = word[w];
+    const int pos = before[w] + __popc(m & ((1u << lane) - 1u));
+    if ((m >> lane & 1u) && pos < F.cap_tl) F.starts[pos] = (int)(base + 32 * w + lane);
   }
 }
 
@@ -1373,6 +1459,9 @@ __global__ void k_sel_owner(FrameDev F, KParams P) {
 // Outer-to-inner walk of every tracklet's hits.  The rows are taken in
 // groups of kWalkGroup: their hit indices, then those hits' owner keys, are
 // requested together before the (sequential) keep decisions of the group.
+// (List order: ordered by rows within stretches, as the constructor's kernels
+// are, the lanes fill better but neighbouring tracklets' owner keys no longer
+// share cache lines: 1.17 instead of 0.77 ms on two full frames.)
 constexpr int kWalkGroup = 16;
 
 __global__ void k_sel_walk(FrameDev F, KParams P) {
@@ -1815,9 +1904,8 @@ int stage_reseed(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
     k_scan_partials<<<1, 1024, 0, s>>>(F.scan_tmp, nb, &F.cnt->n_new);
     k_start_write<<<nb, kBlock, 0, s>>>(F);
     k += launch_tracklets<true>(F, P, sms, s);
-    k_sel_owner<<<sms * 8, kBlock, 0, s>>>(F, P);
-    k_sel_walk<<<sms * 8, kBlock, 0, s>>>(F, P);
-    k += 10;
+    k += stage_select(F, P, sms, s);
+    k += 8;
   }
   return k;
 }
