@@ -418,7 +418,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.cr_cx, FT);
   ok &= dalloc(ctx, &F.cr_cy, FT);
   ok &= dalloc(ctx, &F.cr_zk, FT);
-  ok &= dalloc(ctx, &F.cr_bin_items, FT);
+  ok &= dalloc(ctx, &F.cr_rec, 2 * FT);
   ok &= dalloc(ctx, &F.out_par, FT * 5);
   ok &= dalloc(ctx, &F.out_cov, FT * 15);
   ok &= dalloc(ctx, &F.out_chi2, FT);

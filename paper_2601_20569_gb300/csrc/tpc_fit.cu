@@ -593,127 +593,140 @@ __global__ void __launch_bounds__(256, 4) k_merge_best(FrameDev F, KParams P) {
         F.st_bestchi[am] = 0.0f;
       }
     }
-    for (unsigned todo = __ballot_sync(gmask, live) & gmask; todo; todo &= todo - 1) {
-      const int a = __shfl_sync(gmask, am, (__ffs(todo) - 1) & (G - 1), G);
-      const int keyA = F.st_key[a];
-      unsigned long long best = ~0ull;
-      int bb = -1;
-      // the pair test needs 1 <= rmin(B) - rmax(A) <= merge_max_gap: only
-      // those rows of the index are visited
-      const int r0 = F.st_rmax[a] + 1;
-      const int r1 = min(F.st_rmax[a] + P.merge_max_gap, P.n_rows - 1);
-      const float x0 = F.row_x[r0], x1 = F.row_x[r1];
-      const int sa = F.st_sector[a];
-      const int side = sa / half, ph = sa % half;
-      const float* oe = F.st_oe + (long)a * kStateF;
-      const float zwin = P.merge_dz + fabsf(oe[3]) * P.merge_zspan;
-      const float oz = oe[1];
-      // A's state and z bins in the three sectors: lanes 0-2 of the group hold
-      // one sector each and hand it to the lanes by shuffles (with fewer lanes
-      // every lane computes the three); no bins where A cannot be turned into
-      // the sector, as the test fails there
+    // A's state and z bins in the three sectors searched: lane 3 e + q of the
+    // group prepares sector q of the round's e-th end (kSetup ends at once; with
+    // fewer than four lanes every lane prepares the three of each end itself) and
+    // hands them to the lanes by shuffles; no bins where A cannot be turned into
+    // the sector, as the test fails there
+    constexpr int kSetup = G >= 4 ? G / 3 : 1;
+    for (unsigned todo = __ballot_sync(gmask, live) & gmask; todo;) {
+      const int slot = gl / 3;  // the lane's end among the next kSetup
+      unsigned mine = todo;
+      if (G >= 4)
+        for (int e = 0; e < slot && mine; ++e) mine &= mine - 1;
       MergeA ma{};
-      int sq[3], zq[3], nq[3];
-      int nr = 0;
       int my_s = 0, my_z = 0, my_n = 0;
+      const int ae = __shfl_sync(gmask, am, mine ? (__ffs(mine) - 1) & (G - 1) : 0, G);
+      auto setup = [&](int a, int q) {
+        const float* oe = F.st_oe + (long)a * kStateF;
+        const int sa = F.st_sector[a], rmx = F.st_rmax[a];
+        const float zwin = P.merge_dz + fabsf(oe[3]) * P.merge_zspan;
+        ma = merge_a(oe, q, P);
+        my_s = sa / half * half + (sa % half + (q == 0 ? 0 : q == 1 ? 1 : half - 1)) % half;
+        float zlo, zhi;
+        merge_window(ma, F.row_x[rmx + 1], F.row_x[min(rmx + P.merge_max_gap, P.n_rows - 1)], P,
+                     zlo, zhi);
+        zlo = fmaxf(zlo, oe[1] - zwin - 0.01f);
+        zhi = fminf(zhi, oe[1] + zwin + 0.01f);
+        my_z = merge_zbin(F, my_s, zlo);
+        my_n = ma.ok && zlo <= zhi ? merge_zbin(F, my_s, zhi) - my_z + 1 : 0;
+      };
+      if (G >= 4 && slot < kSetup && mine) setup(ae, gl - 3 * slot);
+#pragma unroll 1
+      for (int e = 0; e < kSetup && todo; ++e, todo &= todo - 1) {
+        const int a = __shfl_sync(gmask, am, (__ffs(todo) - 1) & (G - 1), G);
+        const int keyA = F.st_key[a];
+        unsigned long long best = ~0ull;
+        int bb = -1;
+        // the pair test needs 1 <= rmin(B) - rmax(A) <= merge_max_gap: only
+        // those rows of the index are visited
+        const int r0 = F.st_rmax[a] + 1;
+        const int r1 = min(F.st_rmax[a] + P.merge_max_gap, P.n_rows - 1);
+        const float* oe = F.st_oe + (long)a * kStateF;
+        const float zwin = P.merge_dz + fabsf(oe[3]) * P.merge_zspan;
+        const float oz = oe[1];
+        int sq[3], zq[3], nq[3];
+        int nr = 0;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        if (G < 4 || gl == q) {
-          ma = merge_a(oe, q, P);
-          my_s = side * half + (ph + (q == 0 ? 0 : q == 1 ? 1 : half - 1)) % half;
-          float zlo, zhi;
-          merge_window(ma, x0, x1, P, zlo, zhi);
-          zlo = fmaxf(zlo, oz - zwin - 0.01f);
-          zhi = fminf(zhi, oz + zwin + 0.01f);
-          my_z = merge_zbin(F, my_s, zlo);
-          my_n = ma.ok && zlo <= zhi ? merge_zbin(F, my_s, zhi) - my_z + 1 : 0;
-        }
-        if (G < 4) {
-          sq[q] = my_s;
-          zq[q] = my_z;
-          nq[q] = my_n;
-        } else {
-          sq[q] = __shfl_sync(gmask, my_s, q, G);
-          zq[q] = __shfl_sync(gmask, my_z, q, G);
-          nq[q] = __shfl_sync(gmask, my_n, q, G);
-        }
-        nr += nq[q];
-      }
-      for (int j0 = 0; j0 < nr; j0 += G) {
-        int lo = 0, cnt = 0, qj = 0;
-        int j = j0 + gl;
-        if (j < nr) {
-          const int q = j < nq[0] ? 0 : j < nq[0] + nq[1] ? 1 : 2;
-          j -= q == 0 ? 0 : q == 1 ? nq[0] : nq[0] + nq[1];
-          const int base = ((q == 0 ? sq[0] : q == 1 ? sq[1] : sq[2]) * kMergeZ +
-                            (q == 0 ? zq[0] : q == 1 ? zq[1] : zq[2]) + j) * P.n_rows;
-          lo = F.ie_first[base + r0];
-          cnt = F.ie_first[base + r1 + 1] - lo;
-          qj = q;
-        }
-        int inc = cnt;  // inclusive scan of the range sizes over the group
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-          const int v = __shfl_up_sync(gmask, inc, o, G);
-          if (gl >= o) inc += v;
-        }
-        const int total = __shfl_sync(gmask, inc, G - 1, G);
-        for (int c0 = 0; c0 < total; c0 += G) {
-          const int c = c0 + gl;
-          int L = 0;  // the range holding candidate c: first lane with inc > c
-#pragma unroll
-          for (int st = G / 2; st >= 1; st >>= 1) {
-            const int v = __shfl_sync(gmask, inc, L + st - 1, G);
-            if (v <= c) L += st;
+        for (int q = 0; q < 3; ++q) {
+          if (G < 4) {
+            setup(a, q);
+            sq[q] = my_s;
+            zq[q] = my_z;
+            nq[q] = my_n;
+          } else {
+            sq[q] = __shfl_sync(gmask, my_s, 3 * e + q, G);
+            zq[q] = __shfl_sync(gmask, my_z, 3 * e + q, G);
+            nq[q] = __shfl_sync(gmask, my_n, 3 * e + q, G);
           }
-          const int excl = __shfl_sync(gmask, inc - cnt, L, G);
-          const int lo_l = __shfl_sync(gmask, lo, L, G);
-          const int q_l = __shfl_sync(gmask, qj, L, G);
-          MergeA mq;
-          if (G >= 4) {
-            mq.y = __shfl_sync(gmask, ma.y, q_l, G);
-            mq.z = __shfl_sync(gmask, ma.z, q_l, G);
-            mq.s0 = __shfl_sync(gmask, ma.s0, q_l, G);
-            mq.c0 = __shfl_sync(gmask, ma.c0, q_l, G);
-            mq.kap = __shfl_sync(gmask, ma.kap, q_l, G);
-            mq.tgl = __shfl_sync(gmask, ma.tgl, q_l, G);
-            mq.x = __shfl_sync(gmask, ma.x, q_l, G);
-            mq.ok = __shfl_sync(gmask, ma.ok, q_l, G);
-          }
-          if (c >= total) continue;
-          // the indexed inner end: (y, z, x, track)
-          const float4 rec = F.ie_rec[lo_l + (c - excl)];
-          if (!(fabsf(rec.y - oz) <= zwin)) continue;  // the full test's z window
-          if (G < 4) mq = merge_a(oe, q_l, P);
-          float yb, zb;
-          if (merge_pos(mq, rec.z, P, yb, zb) &&
-              (fabsf(rec.x - yb) > P.merge_dy + 0.01f + 1e-5f * fabsf(rec.x) ||
-               fabsf(rec.y - zb) > P.merge_dz + 0.01f + 1e-5f * fabsf(rec.y)))
-            continue;
-          const int b = __float_as_int(rec.w);
-          if (b == a || !F.st_ok[b]) continue;
-          float chi2;
-          if (!merge_test(F, P, a, b, chi2)) continue;
-          const unsigned long long kb = pack_chi_key(chi2, F.st_key[b]);
-          if (kb < best) {
-            best = kb;
-            bb = b;
-          }
-          atomicMin(&F.st_bestA[b], pack_chi_key(chi2, keyA));
+          nr += nq[q];
         }
-      }
+        for (int j0 = 0; j0 < nr; j0 += G) {
+          int lo = 0, cnt = 0, qj = 0;
+          int j = j0 + gl;
+          if (j < nr) {
+            const int q = j < nq[0] ? 0 : j < nq[0] + nq[1] ? 1 : 2;
+            j -= q == 0 ? 0 : q == 1 ? nq[0] : nq[0] + nq[1];
+            const int base = ((q == 0 ? sq[0] : q == 1 ? sq[1] : sq[2]) * kMergeZ +
+                              (q == 0 ? zq[0] : q == 1 ? zq[1] : zq[2]) + j) * P.n_rows;
+            lo = F.ie_first[base + r0];
+            cnt = F.ie_first[base + r1 + 1] - lo;
+            qj = q;
+          }
+          int inc = cnt;  // inclusive scan of the range sizes over the group
 #pragma unroll
-      for (int o = G / 2; o >= 1; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(gmask, best, o, G);
-        const int obb = __shfl_xor_sync(gmask, bb, o, G);
-        if (ob < best) {
-          best = ob;
-          bb = obb;
+          for (int o = 1; o < G; o <<= 1) {
+            const int v = __shfl_up_sync(gmask, inc, o, G);
+            if (gl >= o) inc += v;
+          }
+          const int total = __shfl_sync(gmask, inc, G - 1, G);
+          for (int c0 = 0; c0 < total; c0 += G) {
+            const int c = c0 + gl;
+            int L = 0;  // the range holding candidate c: first lane with inc > c
+#pragma unroll
+            for (int st = G / 2; st >= 1; st >>= 1) {
+              const int v = __shfl_sync(gmask, inc, L + st - 1, G);
+              if (v <= c) L += st;
+            }
+            const int excl = __shfl_sync(gmask, inc - cnt, L, G);
+            const int lo_l = __shfl_sync(gmask, lo, L, G);
+            const int q_l = __shfl_sync(gmask, qj, L, G);
+            MergeA mq;
+            if (G >= 4) {
+              mq.y = __shfl_sync(gmask, ma.y, 3 * e + q_l, G);
+              mq.z = __shfl_sync(gmask, ma.z, 3 * e + q_l, G);
+              mq.s0 = __shfl_sync(gmask, ma.s0, 3 * e + q_l, G);
+              mq.c0 = __shfl_sync(gmask, ma.c0, 3 * e + q_l, G);
+              mq.kap = __shfl_sync(gmask, ma.kap, 3 * e + q_l, G);
+              mq.tgl = __shfl_sync(gmask, ma.tgl, 3 * e + q_l, G);
+              mq.x = __shfl_sync(gmask, ma.x, 3 * e + q_l, G);
+              mq.ok = __shfl_sync(gmask, ma.ok, 3 * e + q_l, G);
+            }
+            if (c >= total) continue;
+            // the indexed inner end: (y, z, x, track)
+            const float4 rec = F.ie_rec[lo_l + (c - excl)];
+            if (!(fabsf(rec.y - oz) <= zwin)) continue;  // the full test's z window
+            if (G < 4) mq = merge_a(oe, q_l, P);
+            float yb, zb;
+            if (merge_pos(mq, rec.z, P, yb, zb) &&
+                (fabsf(rec.x - yb) > P.merge_dy + 0.01f + 1e-5f * fabsf(rec.x) ||
+                 fabsf(rec.y - zb) > P.merge_dz + 0.01f + 1e-5f * fabsf(rec.y)))
+              continue;
+            const int b = __float_as_int(rec.w);
+            if (b == a || !F.st_ok[b]) continue;
+            float chi2;
+            if (!merge_test(F, P, a, b, chi2)) continue;
+            const unsigned long long kb = pack_chi_key(chi2, F.st_key[b]);
+            if (kb < best) {
+              best = kb;
+              bb = b;
+            }
+            atomicMin(&F.st_bestA[b], pack_chi_key(chi2, keyA));
+          }
         }
-      }
-      if (gl == 0) {
-        F.st_bestB[a] = bb;
-        F.st_bestchi[a] = bb >= 0 ? o2f((unsigned)(best >> 32)) : 0.0f;
+#pragma unroll
+        for (int o = G / 2; o >= 1; o >>= 1) {
+          const unsigned long long ob = __shfl_xor_sync(gmask, best, o, G);
+          const int obb = __shfl_xor_sync(gmask, bb, o, G);
+          if (ob < best) {
+            best = ob;
+            bb = obb;
+          }
+        }
+        if (gl == 0) {
+          F.st_bestB[a] = bb;
+          F.st_bestchi[a] = bb >= 0 ? o2f((unsigned)(best >> 32)) : 0.0f;
+        }
       }
     }
   }

@@ -97,7 +97,7 @@ constexpr int kMaxBinOcc = 1024;
 constexpr int kStateF = 22;     // p[5], c[15], x, sector (as float)
 constexpr int kSeedF = 8;       // tracklet seed: p[5], x, sector*n_rows + row, valid
 constexpr int kIpolF = 11;      // interpolation record of an inner station
-constexpr int kMergeLanesDefault = 16;  // lanes per outer end in the merge search
+constexpr int kMergeLanesDefault = 32;  // lanes per outer end in the merge search
 constexpr int kLinksLanesDefault = 1;   // lanes per cluster in the neighbour search (32: staged per warp)
 constexpr int kMergeZ = 512;     // z bins per sector of the merge candidate index
 constexpr int kMaxInner = 32;    // inner-region rows supported
@@ -139,6 +139,7 @@ struct Counters {
   int n_removed;     // cluster removal: clusters flagged for removal
   int n_st0;         // edge following: sector tracks before the segments were added
   int n_tl_all;      // edge following: tracklet slots in use before the segments
+  int row_blocks;    // row layout: blocks done
 };
 
 // One frame of a batch call, read in place: the clusters of batch index i
@@ -224,7 +225,8 @@ struct FrameDev {
   float* cr_zk;            // [cap_ft] side * z at the innermost cluster (leg order)
   int* cr_bin_cnt;         // [kCrBins + 1] loopers per (side block, centre bin)
   int* cr_bin_first;       // [kCrBins + 1]
-  int* cr_bin_items;       // [cap_ft]
+  float4* cr_rec;          // [cap_ft][2] loopers in bin order: (q/pT, tan lambda, centre x, y),
+                           // (side * z, key, track, -)
   Counters* cnt;
 
   // a7 sector tracks (capacity cap_tl)

@@ -15,6 +15,7 @@ namespace tpc {
   int call_init(FrameDev& F, const KParams& P, int sms, cudaStream_t s);          \
   int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s);         \
   int stage_links(FrameDev& F, const KParams& P, int sms, cudaStream_t s);        \
+  int stage_find_links(FrameDev& F, const KParams& P, cudaStream_t s);            \
   int stage_starts(FrameDev& F, const KParams& P, int sms, cudaStream_t s);       \
   int stage_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t s);    \
   int stage_select(FrameDev& F, const KParams& P, int sms, cudaStream_t s);       \

@@ -54,7 +54,7 @@ constexpr long kOffBinFirst = kOffBinCnt + align256(sizeof(int) * (kNoAllocBins 
 constexpr long kOffScanTmp = kOffBinFirst + align256(sizeof(int) * (kNoAllocBins + 1));
 constexpr long kScanTmpInts = kNoAllocBins / 256 + 4096;
 constexpr long kOffPerCl = kOffScanTmp + align256(sizeof(int) * kScanTmpInts);
-constexpr long kPerClInts = 9;  // cl_bin, cl_slot, (y, z) [two slots], sid, lup, ldn, cup, cdn
+constexpr long kPerClInts = 7;  // cl_bin, cl_slot, (y, z) [two slots], sid, lup, ldn
 constexpr long kOffSrow = kOffPerCl + kPerClInts * align256(4 * kNoAllocMaxClusters);
 constexpr long kOffSrec = kOffSrow + align256(2 * kNoAllocMaxClusters);
 constexpr long kOffRowFirst = kOffSrec + align256(16 * kNoAllocMaxClusters);
@@ -106,19 +106,20 @@ __global__ void k_links_init(FrameDev F, RowX row_x, int n_rows, long nrr) {
   for (int k = threadIdx.x; k < (int)(sizeof(Counters) / 4); k += blockDim.x) ((int*)F.cnt)[k] = 0;
 }
 
-// Sorted-order links -> caller's input-id order.  Writes nothing when the grid
+// Cleaning (a link stays if its partner links back) and sorted-order links ->
+// caller's input-id order in one pass.  Writes nothing when the grid
 // build or the neighbour finding recorded an error: those kernels then leave
 // the sorted arrays partly unwritten, holding an earlier call's ids, which may
 // lie beyond this call's n.
 __global__ void k_links_to_ids(const Counters* __restrict__ cnt, const int* __restrict__ sid,
-                               const int* __restrict__ cup, const int* __restrict__ cdn, long n,
+                               const int* __restrict__ lup, const int* __restrict__ ldn, long n,
                                int32_t* up, int32_t* dn) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n || cnt->err != 0) return;
   const int id = sid[k];
-  const int u = cup[k], d = cdn[k];
-  up[id] = u >= 0 ? sid[u] : -1;
-  dn[id] = d >= 0 ? sid[d] : -1;
+  const int u = lup[k], d = ldn[k];
+  up[id] = u >= 0 && ldn[u] == (int)k ? sid[u] : -1;
+  dn[id] = d >= 0 && lup[d] == (int)k ? sid[d] : -1;
 }
 
 }  // namespace
@@ -179,8 +180,6 @@ extern "C" tpc_status tpc_links_noalloc(const tpc_geometry* geo, const tpc_optio
   F.sid = per[4];
   F.lup = per[5];
   F.ldn = per[6];
-  F.cup = per[7];
-  F.cdn = per[8];
   F.srow = (uint16_t*)(b + kOffSrow);
   F.srec = (int4*)(b + kOffSrec);
   F.row_first = (int*)(b + kOffRowFirst);
@@ -195,9 +194,9 @@ extern "C" tpc_status tpc_links_noalloc(const tpc_geometry* geo, const tpc_optio
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   strict::stage_grid(F, P, sms > 0 ? sms : 1, s);
-  strict::stage_links(F, P, sms > 0 ? sms : 1, s);
+  strict::stage_find_links(F, P, s);
   if (n > 0)
-    k_links_to_ids<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(F.cnt, F.sid, F.cup, F.cdn, n,
+    k_links_to_ids<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(F.cnt, F.sid, F.lup, F.ldn, n,
                                                                 link_up, link_dn);
   if (cudaGetLastError() != cudaSuccess) return TPC_ERR_CUDA;
   Counters hc;

@@ -129,30 +129,26 @@ __global__ void __launch_bounds__(256) k_row_stats_sh(FrameDev F, KParams P, int
   }
 }
 
-// One block: bin layout of every (sector,row) and the row/bin offsets.  A warp
-// takes a run of consecutive rows, 32 at a time with a scan of its own, and one
-// scan over the warps' sums gives the offsets (a block scan per 1024 rows, with
-// its barriers, took 13 us for a frame).
+// Bin layout of every (sector,row) and the row/bin offsets.  A thread lays out one
+// row; the block that finishes last turns the bin and cluster counts into offsets,
+// each of its warps over a run of consecutive rows with scans of its own.  (As
+// one block of 1024 threads the layouts' divides and roots alone took that SM
+// most of 13 us for a frame's 5,472 rows.)
 __global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
   __shared__ int sh[32];
+  __shared__ bool last;
   const int nrr = P.n_sectors * P.n_rows;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int per = (nrr + 32 * nw - 1) / (32 * nw) * 32;
-  const int lo = min(nrr, warp * per), hi = min(nrr, lo + per);
-  int nb = 0, nc = 0;  // bins and clusters of the warp's rows so far
-  for (int r0 = lo; r0 < hi; r0 += 32) {
-    const int rr = min(r0 + lane, hi - 1);
-    const bool mine = r0 + lane < hi;
+  const int row = blockIdx.x * blockDim.x + threadIdx.x;
+  if (row < nrr) {
     RowGrid g{};
-    const int r = rr % P.n_rows;
-    const int cnt = F.row_cnt[rr];
-    const float x = F.row_x[r];
+    const int cnt = F.row_cnt[row];
+    const float x = F.row_x[row % P.n_rows];
     const float ymax = x * P.tan_half + 0.5f;
     int nZ = 1;
     float zlo = 0.0f, zr = 0.0f;
     if (cnt > 0) {
-      zlo = o2f(F.row_zmin[rr]);
-      zr = o2f(F.row_zmax[rr]) - zlo;
+      zlo = o2f(F.row_zmin[row]);
+      zr = o2f(F.row_zmax[row]) - zlo;
     }
     // about square bins holding grid_occ clusters each (0.5), at least grid_dy
     // wide in y: the search windows (a few cm in y and in z) then cover few
@@ -173,8 +169,36 @@ __global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
     g.z0 = zlo;
     g.invDz = zr > 0.0f ? (float)nZ / zr : 0.0f;
     g.ncl = cnt;
-    int ib = mine ? nY * nZ : 0, ic = mine ? cnt : 0;  // inclusive scans
-    const int vb = ib, vc = ic;
+    g.bin0 = nY * nZ;  // the row's bins, until the offsets are known
+    F.rows[row] = g;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&F.cnt->row_blocks, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int per = (nrr + 32 * nw - 1) / (32 * nw) * 32;
+  const int lo = min(nrr, warp * per), hi = min(nrr, lo + per);
+  int nb = 0, nc = 0;  // bins and clusters of the warp's rows
+  for (int r = lo + lane; r < hi; r += 32) {
+    nb += __ldcg(&F.rows[r].bin0);
+    nc += __ldcg(&F.row_cnt[r]);
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    nb += __shfl_xor_sync(0xffffffffu, nb, o);
+    nc += __shfl_xor_sync(0xffffffffu, nc, o);
+  }
+  int tot_b, tot_c;
+  const int eb = block_exscan(lane == 31 ? nb : 0, sh, &tot_b);
+  const int ec = block_exscan(lane == 31 ? nc : 0, sh, &tot_c);
+  int ob = __shfl_sync(0xffffffffu, eb, 0), oc = __shfl_sync(0xffffffffu, ec, 0);
+  for (int r0 = lo; r0 < hi; r0 += 32) {
+    const int r = r0 + lane;
+    const int vb = r < hi ? __ldcg(&F.rows[r].bin0) : 0, vc = r < hi ? __ldcg(&F.row_cnt[r]) : 0;
+    int ib = vb, ic = vc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int yb = __shfl_up_sync(0xffffffffu, ib, o), yc = __shfl_up_sync(0xffffffffu, ic, o);
@@ -183,21 +207,12 @@ __global__ void __launch_bounds__(1024) k_row_grid(FrameDev F, KParams P) {
         ic += yc;
       }
     }
-    if (mine) {
-      g.bin0 = nb + ib - vb;
-      F.rows[rr] = g;
-      F.row_first[rr] = nc + ic - vc;
+    if (r < hi) {
+      F.rows[r].bin0 = ob + ib - vb;
+      F.row_first[r] = oc + ic - vc;
     }
-    nb += __shfl_sync(0xffffffffu, ib, 31);
-    nc += __shfl_sync(0xffffffffu, ic, 31);
-  }
-  int tot_b, tot_c;
-  const int eb = block_exscan(lane == 31 ? nb : 0, sh, &tot_b);
-  const int ec = block_exscan(lane == 31 ? nc : 0, sh, &tot_c);
-  const int ob = __shfl_sync(0xffffffffu, eb, 0), oc = __shfl_sync(0xffffffffu, ec, 0);
-  for (int rr = lo + lane; rr < hi; rr += 32) {
-    F.rows[rr].bin0 += ob;
-    F.row_first[rr] += oc;
+    ob += __shfl_sync(0xffffffffu, ib, 31);
+    oc += __shfl_sync(0xffffffffu, ic, 31);
   }
   if (threadIdx.x == 0) {
     F.row_first[nrr] = tot_c;
@@ -1816,7 +1831,8 @@ int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
     k_row_stats<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F, P);
     ++k;
   }
-  k_row_grid<<<1, 1024, 0, s>>>(F, P); ++k;
+  k_row_grid<<<blocks_for((long)P.n_sectors * P.n_rows, 1024), 1024, 0, s>>>(F, P);
+  ++k;
   if (n > 0) { k_bin_hist<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F, P); ++k; }
   k_row_scan<<<P.n_sectors * P.n_rows, 256, 0, s>>>(F);
   ++k;
@@ -1828,11 +1844,18 @@ int stage_grid(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   return k;
 }
 
+// The neighbour search alone (lup, ldn not yet cleaned).
+int stage_find_links(FrameDev& F, const KParams& P, cudaStream_t s) {
+  if (F.n <= 0) return 0;
+  launch_links<false>(F, P, F.n, s);
+  return 1;
+}
+
 int stage_links(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   (void)sms;
   const long n = F.n;
   if (n <= 0) return 0;
-  launch_links<false>(F, P, n, s);
+  stage_find_links(F, P, s);
   k_clean<<<blocks_for(n, kBlock), kBlock, 0, s>>>(F);
   return 2;
 }
