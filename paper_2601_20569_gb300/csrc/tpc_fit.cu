@@ -937,30 +937,16 @@ __global__ void k_looper_write(FrameDev F) {
   F.ft_order[fl ? lr : F.cnt->n_loopers + (f - lr)] = f;
 }
 
-// The fit kernels take ft_order: loopers in [0, nL), the other tracks in [nL,
-// nf).  Iteration 3 comes in three parts: kPart 0 takes all, 1 the other tracks
-// only, 2 the loopers only.  Part 1 carries no looper update, so it fits in 80
-// registers and keeps half as many warps again in flight as the full kernel:
-// two launches are the faster form where a kernel's time is its throughput
-// (iteration 3 of two full frames: 0.77 ms, one launch 0.87), one launch where it
-// is the longest track's chain of steps (a central event: 0.28 against 0.16 ms),
-// which the second launch would wait for again.
-//
-// Parts 0 and iterations 1 and 2 number the other tracks from the next multiple
-// of 32 on, so that no warp starts with both kinds (on a frame of a few dozen
-// tracks every warp would, and pay for both updates in each step).
+// The fit kernels take ft_order: loopers in [0, nL), the other tracks in [nL, nf),
+// which are numbered from the next multiple of 32 on, so that no warp starts
+// with both kinds (on a frame of a few dozen tracks every warp would, and pay for
+// both updates in each step).  All in one launch per iteration: iteration 3 in
+// two, the other tracks in 80 registers first, took 0.78 against 0.61 ms on two
+// full frames and 0.24 against 0.17 on a central event.
 __device__ __forceinline__ int fit_total(int nL, int nf) { return nf + ((32 - (nL & 31)) & 31); }
 __device__ __forceinline__ int fit_position(int q, int nL) {  // -1: no track
   const int pad = (32 - (nL & 31)) & 31;
   return q < nL ? q : q < nL + pad ? -1 : q - pad;
-}
-
-constexpr long kFit3Split = 4000000;  // clusters of a call from which on iteration 3 is split
-
-// Looper flag of fit track f in part kPart (compile-time in parts 1 and 2).
-template <int kPart>
-__device__ __forceinline__ bool fit_looper(const FrameDev& F, int f) {
-  return kPart == 2 ? true : kPart == 1 ? false : F.ft_looper[f] != 0;
 }
 
 // ------------------------------------------ a9/a10 linearised three-iteration fit
@@ -1831,9 +1817,8 @@ __global__ void k_amb_resolve(FrameDev F, KParams P, MapDev M, int round) {
 // Iteration 3: inward with the surviving and re-attached clusters (as the
 // station records hold them after iteration 2 and the second ambiguity
 // solving), simple cut.
-template <bool kMap, bool kExt, int kPart>
-__global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
-    k_fit3(FrameDev F, KParams P, MapDev M, int stat) {
+template <bool kMap, bool kExt>
+__global__ void __launch_bounds__(256, 2) k_fit3(FrameDev F, KParams P, MapDev M, int stat) {
   if (!kMap) M.on = 0;  // (the map evaluation is compiled out)
   __shared__ float rx[kMaxRows];
   for (int r = threadIdx.x; r < P.n_rows; r += blockDim.x) rx[r] = F.row_x[r];
@@ -1844,13 +1829,12 @@ __global__ void __launch_bounds__(256, kPart == 1 ? 3 : 2)
   const int nL = min(F.cnt->n_loopers, nf);
   bool first = true;
   for (;;) {
-    const int q = (kPart == 1 ? nL : 0) +
-                  next_item(&F.cnt->queue[kPart == 1 ? kQFit3N : kQFit3], first, stat);
-    if (q >= (kPart == 2 ? nL : kPart == 1 ? nf : fit_total(nL, nf))) break;
-    const int pos = kPart == 0 ? fit_position(q, nL) : q;
+    const int q = next_item(&F.cnt->queue[kQFit3], first, stat);
+    if (q >= fit_total(nL, nf)) break;
+    const int pos = fit_position(q, nL);
     if (pos < 0) continue;
     const int f = F.ft_order[pos];
-    const bool lp = fit_looper<kPart>(F, f);  // FP64 updates (low-pT looper)
+    const bool lp = F.ft_looper[f] != 0;  // FP64 updates (low-pT looper)
     F.ft_n[f] = 0;
     if (!F.ft_ok[f]) continue;
     const int ns = F.ft_nst[f];
@@ -2891,28 +2875,11 @@ int stage_ambiguity2(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   return k;
 }
 
-template <bool kMap, bool kExt, int kPart>
-void launch_fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
-  const unsigned g = persistent_grid(F.lc, kLFit3, sms);
-  const int b = F.lc.block[kLFit3];
-  k_fit3<kMap, kExt, kPart><<<g, b, 0, s>>>(F, P, F.map,
-                                            resident_lanes<k_fit3<kMap, kExt, kPart>>(b, 0, g, sms));
-}
-
 template <bool kMap, bool kExt>
 int fit3(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
-  if (kMap && kExt) {  // (its part 1 would spill)
-    launch_fit3<kMap, kExt, 0>(F, P, sms, s);
-    return 1;
-  }
-  if constexpr (!(kMap && kExt)) {
-    if (F.n >= kFit3Split) {
-      launch_fit3<kMap, kExt, 1>(F, P, sms, s);
-      launch_fit3<kMap, kExt, 2>(F, P, sms, s);
-      return 2;
-    }
-    launch_fit3<kMap, kExt, 0>(F, P, sms, s);
-  }
+  const unsigned g = persistent_grid(F.lc, kLFit3, sms);
+  const int b = F.lc.block[kLFit3];
+  k_fit3<kMap, kExt><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit3<kMap, kExt>>(b, 0, g, sms));
   return 1;
 }
 

@@ -55,7 +55,7 @@ struct LaunchCfg {
 
 // Work queues: counters of the dynamic item fetching (zeroed per call).
 enum QueueSlot : int {
-  kQTracklets = 0, kQSectorRefit, kQMerge, kQFit1, kQFit2, kQFit3, kQFit3N,
+  kQTracklets = 0, kQSectorRefit, kQMerge, kQFit1, kQFit2, kQFit3,
   kQTlDown, kQTlUp, kQTlRefit, kQNum
 };
 

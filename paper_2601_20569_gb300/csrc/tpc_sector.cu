@@ -1016,10 +1016,10 @@ __global__ void k_chain_info(FrameDev F, KParams P) {
 // state they only save and restore (downward: the state at the innermost hit;
 // upward: the state and position at the top hit), field-major so that a
 // warp's accesses hit distinct banks.  It keeps k_tl_refit at 64 registers, four
-// 256-thread blocks per SM.  The searches are held to three blocks (80
-// registers): at 64 they spill, and what they wait for is the chain of loads of
-// a step, not lanes (two full frames: k_tl_up 1.05 -> 0.99 ms, a central event
-// 0.42 -> 0.35 ms with the batched loads of pick).
+// 256-thread blocks per SM.  The searches are held to two or three blocks
+// (launch_tracklets): at 64 registers they spill, and what they wait for is the
+// chain of loads of a step, not lanes (two full frames: k_tl_up 1.05 -> 0.99 ms, a
+// central event 0.42 -> 0.35 ms with the batched loads of pick).
 constexpr int kTlShared = 21;  // saved state: p[5], c[15], x (or p[5], x, y_hit, z_hit)
 
 // Tracklet states between the kernels (tl_n): 0 none yet or rejected; -2 seed
@@ -1145,8 +1145,8 @@ __global__ void __launch_bounds__(256, 4) k_tl_chain(FrameDev F, KParams P, int 
 // Upward pass, second part: extension by the best cluster of each row from
 // the chain's top.  The state at the top hit and that hit's position are left
 // in tl_seed[0..5], tl_chi2 and tl_x for the downward pass.
-template <bool kLeft>
-__global__ void __launch_bounds__(256, 3) k_tl_up(FrameDev F, KParams P, int stat) {
+template <bool kLeft, int kBlocks>
+__global__ void __launch_bounds__(256, kBlocks) k_tl_up(FrameDev F, KParams P, int stat) {
   extern __shared__ float tl_sh[];
   float* const S = tl_sh + threadIdx.x;
   const int BS = blockDim.x;
@@ -1358,8 +1358,8 @@ __global__ void __launch_bounds__(256, 4) k_tl_refit(FrameDev F, KParams P, int 
 
 // Downward pass, second part: extension below the start by the best cluster
 // of each row until max_miss rows in a row have none.
-template <bool kLeft>
-__global__ void __launch_bounds__(256, 3) k_tl_down(FrameDev F, KParams P, int stat) {
+template <bool kLeft, int kBlocks>
+__global__ void __launch_bounds__(256, kBlocks) k_tl_down(FrameDev F, KParams P, int stat) {
   extern __shared__ float tl_sh[];
   float* const S = tl_sh + threadIdx.x;
   const int BS = blockDim.x;
@@ -1873,7 +1873,7 @@ int stage_starts(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
 // The tracklet constructor of one sector-tracking iteration.  Chains and refits
 // are taken by length, which is known beforehand; the searches in list order,
 // where neighbouring tracklets start on the same row.
-template <bool kLeft>
+template <bool kLeft, int kBlocks>
 static int launch_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const int tb = F.lc.block[kLTracklets];
   const size_t sh = sizeof(float) * kTlShared * tb;
@@ -1881,11 +1881,26 @@ static int launch_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t
   k_chain_info<<<sms * 8, kBlock, 0, s>>>(F, P);
   k_tl_order<false><<<sms * 4, kBlock, 0, s>>>(F, P);
   k_tl_chain<<<g, tb, 0, s>>>(F, P, resident_lanes<k_tl_chain>(tb, 0, g, sms));
-  k_tl_up<kLeft><<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_up<kLeft>>(tb, sh, g, sms));
+  k_tl_up<kLeft, kBlocks><<<g, tb, sh, s>>>(
+      F, P, resident_lanes<k_tl_up<kLeft, kBlocks>>(tb, sh, g, sms));
   k_tl_order<true><<<sms * 4, kBlock, 0, s>>>(F, P);
   k_tl_refit<<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_refit>(tb, sh, g, sms));
-  k_tl_down<kLeft><<<g, tb, sh, s>>>(F, P, resident_lanes<k_tl_down<kLeft>>(tb, sh, g, sms));
+  k_tl_down<kLeft, kBlocks><<<g, tb, sh, s>>>(
+      F, P, resident_lanes<k_tl_down<kLeft, kBlocks>>(tb, sh, g, sms));
   return 7;
+}
+
+// The searches at two blocks per SM (up to 128 registers, no spills) where the
+// call is short of tracklets for the lanes and its time is the longest tracklet's
+// chain of steps, at three (80 registers) where it is the throughput: k_tl_up +
+// k_tl_down of a central event 557 us at two, 610 at three; of two full frames 2.33
+// and 1.98 ms.
+constexpr long kFewClusters = 4000000;
+
+template <bool kLeft>
+static int launch_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
+  return F.n < kFewClusters ? launch_tracklets<kLeft, 2>(F, P, sms, s)
+                            : launch_tracklets<kLeft, 3>(F, P, sms, s);
 }
 
 int stage_tracklets(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
