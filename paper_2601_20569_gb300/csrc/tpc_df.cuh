@@ -12,7 +12,8 @@
 // same update on the FP32 pipe with about 2^-46 relative precision per term
 // instead of 2^-53: the rounded results differ from the FP64 update's only
 // where a result lies within that margin of a rounding boundary.  (Strict
-// mode keeps the FP64 update, which the oracle defines.)
+// mode, whose results the oracle defines as the FP64 update's, checks for those
+// and repeats them in FP64: df_update_checked.)
 //
 // Host-compilable, so that a CPU test can compare it with the FP64 update and
 // an extended-precision evaluation.  Every operation is an explicitly rounded
