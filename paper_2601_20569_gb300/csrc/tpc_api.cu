@@ -296,13 +296,15 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.cl_bin, n);
   ok &= dalloc(ctx, &F.cl_slot, n);
   ok &= dalloc(ctx, &F.srec, n);
+  // the links take the grid build's records' place (the records are split into
+  // the sorted arrays before the neighbour search)
+  F.lup = (int*)F.srec;
+  F.ldn = F.lup + n;
+  F.cup = F.ldn + n;
+  F.cdn = F.cup + n;
   ok &= dalloc(ctx, &F.syz, n);
   ok &= dalloc(ctx, &F.sid, n);
   ok &= dalloc(ctx, &F.srow, n);
-  ok &= dalloc(ctx, &F.lup, n);
-  ok &= dalloc(ctx, &F.ldn, n);
-  ok &= dalloc(ctx, &F.cup, n);
-  ok &= dalloc(ctx, &F.cdn, n);
   ok &= dalloc(ctx, &F.flags, n / 32 + 64);
   ok &= dalloc(ctx, &F.scan_tmp, (F.cap_bins + n) / 256 + 4096);
   ok &= dalloc(ctx, &F.starts, F.cap_tl);

@@ -176,7 +176,8 @@ struct FrameDev {
   int* cl_slot;            // [n]
   long cap_bins;
   int4* srec;              // [n] grid build: (y, z, input id, bin) scattered to the sorted
-                           // positions, ordered in each bin and split into syz / sid
+                           // positions, ordered in each bin and split into syz / sid (then
+                           // the room of lup, ldn, cup and cdn)
   float2* syz;             // [n] sorted (y, z)
   int* sid;                // sorted -> input id
   uint16_t* srow;          // sorted -> sector*n_rows + row
