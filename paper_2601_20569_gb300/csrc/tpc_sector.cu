@@ -860,18 +860,28 @@ __global__ void k_start_count(FrameDev F) {
   if (threadIdx.x == 0) F.scan_tmp[blockIdx.x] = tot;
 }
 
+// Whether there is room is decided by every thread from the counts, which are
+// final before the launch.  The error word is raised here, so it must not decide:
+// threads of one block could read different values of it, and those that went on
+// would place hits by shared words that the others had not written.  (An earlier
+// kernel's error is read once per block.)
 __global__ void k_start_write(FrameDev F) {
   __shared__ unsigned word[32];
   __shared__ int before[32];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const int ns = F.cnt->tl_base + F.cnt->n_new;
-    F.cnt->n_starts = ns;
-    if (ns > F.cap_tl) {
-      atomicOr(&F.cnt->err, kErrCapTracklets);
-      atomicMax(&F.cnt->need_tracklets, ns);
+  __shared__ int failed;
+  const int ns = F.cnt->tl_base + F.cnt->n_new;
+  if (threadIdx.x == 0) {
+    failed = F.cnt->err;
+    if (blockIdx.x == 0) {
+      F.cnt->n_starts = ns;
+      if (ns > F.cap_tl) {
+        atomicOr(&F.cnt->err, kErrCapTracklets);
+        atomicMax(&F.cnt->need_tracklets, ns);
+      }
     }
   }
-  if (F.cnt->err) return;  // (differing between blocks only where the call fails)
+  __syncthreads();
+  if (failed || ns > F.cap_tl) return;  // (the same for the whole block)
   const long base = (long)blockIdx.x * blockDim.x * kCompactItems;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 32) {
@@ -888,8 +898,8 @@ __global__ void k_start_write(FrameDev F) {
   __syncthreads();
   for (int w = threadIdx.x >> 5; w < 32; w += blockDim.x >> 5) {
     const unsigned m = word[w];
-    const int pos = before[w] + __popc(m & ((1u << lane) - 1u));
-    if ((m >> lane & 1u) && pos < F.cap_tl) F.starts[pos] = (int)(base + 32 * w + lane);
+    const int pos = before[w] + __popc(m & ((1u << lane) - 1u));  // (< ns <= cap_tl)
+    if (m >> lane & 1u) F.starts[pos] = (int)(base + 32 * w + lane);
   }
 }
 

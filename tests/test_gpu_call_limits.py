@@ -1,0 +1,51 @@
+"""Calls at the limits of a context, and what they leave for the next one."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_2601_20569_gb300 import synth
+from paper_2601_20569_gb300.options import TrackerOptions
+
+pytestmark = pytest.mark.gpu
+
+RX = synth.row_x()
+
+
+def tracks(tr, dev):
+    tr.track(*dev)
+    return {k: v.cpu().numpy().copy() for k, v in tr.result().items()}
+
+
+def same(a, b):
+    return all(np.array_equal(a[k].view(np.uint8), b[k].view(np.uint8)) for k in a)
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("iters", [1, 2])
+def test_tracklet_capacity_exceeded_then_a_valid_call(iters, graphs):
+    """More start hits than tracklet slots, in the first sector-tracking iteration and
+    (one slot short of both iterations' hits) in the second: the call reports the
+    size it needs, and a call that fits gives a fresh context's tracks."""
+    from paper_2601_20569_gb300 import tpc
+
+    f = synth.generate("central_event", n_primaries=900, looper_frac=0.2, seed=21)
+    s = synth.generate("one_sector", n_primaries=40)
+    opts = TrackerOptions(seed_iters=iters)
+    roomy = tpc.Tracker(RX, opts, mode=0, cap_clusters=f.n)
+    dev = roomy.to_device(f.y, f.z, f.q, f.row, f.sector)
+    sdev = roomy.to_device(s.y, s.z, s.q, s.row, s.sector)
+    want = tracks(roomy, sdev)
+    roomy.track(*dev)
+    need = len(roomy.debug("starts"))
+    first = int(roomy.debug("pass_start")[1]) if iters > 1 else need
+    assert need >= first > 64 and (iters == 1 or need > first)
+    roomy.close()
+    for cap in {first - 1, need - 1, first // 3}:
+        tr = tpc.Tracker(RX, opts, mode=0, cap_clusters=f.n, cap_tracklets=cap, use_graphs=graphs)
+        for _ in range(3):
+            with pytest.raises(tpc.TpcError) as e:
+                tr.track(*dev)
+            assert e.value.status == 3 and e.value.needed == (first if cap < first else need)
+            assert same(tracks(tr, sdev), want)
+        tr.close()
