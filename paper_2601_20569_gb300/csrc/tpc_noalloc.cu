@@ -94,8 +94,15 @@ struct RowX {
   float x[kMaxRows];
 };
 
+// What the grid build accumulates into.  The bin counts (1.8 MB) are cleared here
+// although every complete call leaves them at zero: a call stopped between its
+// kernels, or two calls that overlapped against the rules, would otherwise spoil
+// every later one.
+constexpr long kBinCntVecs = (kOffBinFirst - kOffBinCnt) / 16;  // (the pad to 256 bytes too)
+
 __global__ void k_links_init(FrameDev F, RowX row_x, int n_rows, long nrr) {
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kBinCntVecs) ((int4*)F.bin_cnt)[i] = make_int4(0, 0, 0, 0);
   if (i < nrr) {
     F.row_cnt[i] = 0;
     F.row_zmin[i] = 0xFFFFFFFFu;
@@ -185,10 +192,11 @@ extern "C" tpc_status tpc_links_noalloc(const tpc_geometry* geo, const tpc_optio
   F.row_first = (int*)(b + kOffRowFirst);
 
   // clear what the grid build accumulates into and set the geometry in one
-  // launch (the bin counts are zero from the start and left so by every call)
+  // launch
   RowX row_x;
   std::memcpy(row_x.x, geo->row_x, sizeof(float) * geo->n_rows);
-  k_links_init<<<(unsigned)((nrr + 255) / 256), 256, 0, s>>>(F, row_x, geo->n_rows, nrr);
+  static_assert(kBinCntVecs >= kNoAllocMaxRows, "one thread per bin vector covers the rows");
+  k_links_init<<<(unsigned)((kBinCntVecs + 255) / 256), 256, 0, s>>>(F, row_x, geo->n_rows, nrr);
   int sms = 1;
   int dev = 0;
   cudaGetDevice(&dev);

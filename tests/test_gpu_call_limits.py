@@ -1,6 +1,9 @@
 """Calls at the limits of a context, and what they leave for the next one."""
 from __future__ import annotations
 
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -49,3 +52,32 @@ def test_tracklet_capacity_exceeded_then_a_valid_call(iters, graphs):
             assert e.value.status == 3 and e.value.needed == (first if cap < first else need)
             assert same(tracks(tr, sdev), want)
         tr.close()
+
+
+def run_with_internals(name, tmp_path, frame, opts):
+    """Builds tests/cpp/<name>.cu, which includes a host source file of the library,
+    against libtpc.so and runs it on a frame; returns the words it prints."""
+    from paper_2601_20569_gb300 import build, tpc
+
+    data = tmp_path / "frame.bin"
+    with open(data, "wb") as out:
+        np.array([frame.n, len(RX)], np.int64).tofile(out)
+        out.write(bytes(tpc.make_options(opts, mode=0, cap_clusters=frame.n)))
+        for a, dt in ((RX, np.float32), (frame.y, np.float32), (frame.z, np.float32),
+                      (frame.row, np.uint8), (frame.sector, np.uint8)):
+            np.ascontiguousarray(a, dtype=dt).tofile(out)
+    exe = tmp_path / name
+    here = os.path.dirname(os.path.abspath(__file__))
+    subprocess.check_call([build._nvcc()] + build.COMMON +
+                          [os.path.join(here, "cpp", name + ".cu"), "-o", str(exe), "-L" + build.HERE,
+                           "-l:libtpc.so", "-Xlinker", "-rpath=" + build.HERE])
+    r = subprocess.run([str(exe), str(data)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.split()
+
+
+def test_links_after_stale_bin_counts(tmp_path):
+    f = synth.generate("one_sector")
+    v = run_with_internals("links_scratch", tmp_path, f, TrackerOptions())
+    assert v[0] == "links" and int(v[1]) > 0.5 * f.n
+    assert v[2] == "changed" and int(v[3]) == 0
