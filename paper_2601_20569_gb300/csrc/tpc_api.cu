@@ -94,6 +94,7 @@ struct tpc_ctx {
   bool refit_done = false;
   int64_t refit_gen = 0;  // successful tpc_refit calls so far
   bool tracked = false;  // the last tracking call succeeded (its tracks are resident)
+  bool clean = false;    // bin counts zero and bids empty, as a complete chain leaves them
   int last_nf = 1;       // frames of that call
   long refit_tracks = -1, refit_refs = -1;
   int* steps3 = nullptr;
@@ -142,6 +143,20 @@ bool map_room(tpc_ctx* c, const tpc_map& m) {
   c->map4 = (float4*)v;
   c->map4_cap = n;
   ++c->lc_version;  // captured graphs hold the pointer by value: recapture
+  return true;
+}
+
+// The buffers that the chain itself keeps from call to call: zero bin counts
+// (k_row_scan), empty bids (k_amb_resolve).  Set at the start, and again after a
+// call that stopped part-way (waiting for what it left in flight).
+bool clean_kept(tpc_ctx* c) {
+  FrameDev& F = c->F;
+  if (cudaDeviceSynchronize() != cudaSuccess ||
+      cudaMemset(F.bin_cnt, 0, sizeof(int) * (F.cap_bins + 1)) != cudaSuccess ||
+      cudaMemset(F.bid, 0xFF, sizeof(unsigned long long) * c->cap_n) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess)
+    return false;
+  c->clean = true;
   return true;
 }
 
@@ -440,11 +455,7 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
     tpc_destroy(ctx);
     return TPC_ERR_OOM;
   }
-  // kept by the chain itself from call to call: zero bin counts (k_row_scan),
-  // empty bids (k_amb_resolve)
-  if (cudaMemset(F.bin_cnt, 0, sizeof(int) * (F.cap_bins + 1)) != cudaSuccess ||
-      cudaMemset(F.bid, 0xFF, sizeof(unsigned long long) * n) != cudaSuccess ||
-      cudaDeviceSynchronize() != cudaSuccess) {
+  if (!clean_kept(ctx)) {
     tpc_destroy(ctx);
     return TPC_ERR_CUDA;
   }
@@ -508,6 +519,12 @@ tpc_status run_chain(tpc_ctx* ctx, FrameDev& F, int nf, cudaStream_t s, tpc_trac
   ctx->tracked = false;
   ctx->last_nf = nf;
   ctx->last_stream = s;
+  if (!ctx->clean) {
+    cudaGetLastError();  // (the incomplete call has reported it)
+    if (!clean_kept(ctx))
+      return fail(ctx, TPC_ERR_CUDA, "buffers of an incomplete call could not be reset");
+  }
+  ctx->clean = false;  // (until this call's kernels are known to be done)
   long launches = 0;
   const bool graph = ctx->opt.use_graphs && !ctx->prof;
   if (graph) {
@@ -556,6 +573,7 @@ tpc_status run_chain(tpc_ctx* ctx, FrameDev& F, int nf, cudaStream_t s, tpc_trac
       }
     }
   }
+  ctx->clean = true;
   ctx->launches_last = launches;
   const Counters& c = ctx->host_cnt;
   std::memset(out, 0, sizeof(*out));

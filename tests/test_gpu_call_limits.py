@@ -81,3 +81,10 @@ def test_links_after_stale_bin_counts(tmp_path):
     v = run_with_internals("links_scratch", tmp_path, f, TrackerOptions())
     assert v[0] == "links" and int(v[1]) > 0.5 * f.n
     assert v[2] == "changed" and int(v[3]) == 0
+
+
+def test_call_after_an_interrupted_one(tmp_path):
+    f = synth.generate("central_event", n_primaries=300, seed=8)
+    v = run_with_internals("interrupted_call", tmp_path, f, TrackerOptions())
+    assert v[0] == "tracks" and int(v[1]) > 100
+    assert v[4] == "changed" and int(v[5]) == 0
