@@ -185,7 +185,9 @@ tpc_status tpc_track_timeframe(tpc_ctx* ctx, const tpc_clusters* clusters, tpc_t
  * may be NULL; where given (tracks merged across the central electrode), each
  * track's clusters on the side other than its innermost cluster's enter the
  * refit and the adjoint with their z plus the shift.  `in` and its arrays must
- * stay valid until the matching tpc_refit_backward.  Synchronous.
+ * stay valid until the matching tpc_refit_backward.  A track that cannot be
+ * refitted (no cluster or more than 160, a row that the geometry does not have,
+ * a step that fails) gets chi2 0 and n_clusters 0.  Synchronous.
  * Not in the paper: the differentiable form serves distortion calibration
  * (Sec. 2 names the space-charge correction maps as the limiting factor). */
 tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* clusters, const tpc_tracks* in,

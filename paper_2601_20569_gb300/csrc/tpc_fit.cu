@@ -2158,7 +2158,8 @@ __device__ __forceinline__ void lin_start2(Lin& L, const Trk<float>& s, const fl
 // (As one kernel of four loops per track the lanes of a warp did not reconverge:
 // 4.9 ms for the 3,900 tracks of an event in strict mode.)
 // R.ok counts the passes done: a pass takes a track only if the one before it
-// succeeded.
+// succeeded (-1 from the preparation: a cluster's row is none of the detector's,
+// and the passes hold the rows' x in shared memory; the track is not fitted).
 __global__ void __launch_bounds__(256, 2) k_refit_prep(RefitDev R, KParams P, int* steps3) {
   const MapDev M = R.map;
   const int lane = threadIdx.x & 31;
@@ -2179,12 +2180,15 @@ __global__ void __launch_bounds__(256, 2) k_refit_prep(RefitDev R, KParams P, in
     float zsh;
     int zside;
     refit_shift(R, P, t, zsh, zside);
+    bool bad = false;
     for (int k = lane; k < ns; k += 32) {
       const int c = R.ids[o0 + k];
       const int s = R.sector[c], row = R.row[c];
       const float y = R.y[c], z = track_z(R.z[c], s, zside, zsh, P);
       float4 m = make_float4(0.0f, y, z, __int_as_float(s << 8 | row));
-      if (M.on) {
+      if (row >= P.n_rows) {
+        bad = true;
+      } else if (M.on) {
         float D[3];
         map_eval<true>(M, P, s, R.row_x[row], y, z - z0, D);
         m.x = D[0];
@@ -2194,6 +2198,7 @@ __global__ void __launch_bounds__(256, 2) k_refit_prep(RefitDev R, KParams P, in
       R.raw[o0 + k] = make_float2(y, z);
       R.meas[o0 + k] = m;
     }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) R.ok[t] = -1;
   }
 }
 
@@ -2238,6 +2243,10 @@ __global__ void __launch_bounds__(128, 4) k_refit_start(RefitDev R, KParams P, i
       const int o0 = R.offset[t];
       ns = R.offset[t + 1] - o0;
       if (ns < 1 || ns > kMaxRows) continue;
+      if (R.ok[t] < 0) {
+        R.ok[t] = 0;
+        continue;
+      }
       raw = R.raw + o0;
       meas = R.meas + o0;
       nyz = raw[0];

@@ -88,3 +88,54 @@ def test_call_after_an_interrupted_one(tmp_path):
     v = run_with_internals("interrupted_call", tmp_path, f, TrackerOptions())
     assert v[0] == "tracks" and int(v[1]) > 100
     assert v[4] == "changed" and int(v[5]) == 0
+
+
+REFIT_KEYS = ("cl_offset", "cl_ids", "params", "x", "sector")
+
+
+def refit_setup(n_primaries=300, cap_clusters=None, **opts):
+    import torch
+
+    from paper_2601_20569_gb300 import tpc
+
+    f = synth.generate("central_event", distort=True, n_primaries=n_primaries)
+    tr = tpc.Tracker(RX, TrackerOptions(**opts), mode=0, cap_clusters=cap_clusters or f.n)
+    coeff = torch.as_tensor(f.map).cuda()
+    tr.set_map(coeff)
+    dev = tr.to_device(f.y, f.z, f.q, f.row, f.sector)
+    tr.track(*dev)
+    return f, tr, dev, coeff, {k: tr.result()[k].clone() for k in REFIT_KEYS}
+
+
+def first_tracks(t, n):
+    refs = int(t["cl_offset"][n])
+    return {"cl_offset": t["cl_offset"][:n + 1].clone(), "cl_ids": t["cl_ids"][:refs].clone(),
+            **{k: t[k][:n].clone() for k in ("params", "x", "sector")}}
+
+
+@pytest.mark.parametrize("row", [152, 159, 160, 255])
+def test_refit_skips_a_track_with_a_row_that_does_not_exist(row):
+    f, tr, dev, coeff, t = refit_setup()
+    keys = ("chi2", "n_clusters", "params", "cov")
+    want = {k: tr.refit(dev, t, coeff)[k].clone() for k in keys}
+    nt = int(t["params"].shape[0])
+    bad = nt // 2
+    assert int(want["n_clusters"][bad]) > 0
+    rows = dev[3].clone()
+    o = int(t["cl_offset"][bad])
+    ids = t["cl_ids"].clone()
+    # (clusters may be shared by tracks: the bad one gets a copy of its own)
+    c = int(ids[o + 3])
+    more = [x if x is None else x.new_empty(x.shape[0] + 1) for x in dev]
+    for a, b in zip(more, dev):
+        a[:-1] = b
+        a[-1] = b[c]
+    more[3][:-1] = rows
+    more[3][-1] = row
+    ids[o + 3] = f.n
+    got = tr.refit(tuple(more), dict(t, cl_ids=ids), coeff)
+    assert int(got["n_clusters"][bad]) == 0 and float(got["chi2"][bad]) == 0.0
+    keep = [i for i in range(nt) if i != bad and int(want["n_clusters"][i]) > 0]
+    for k in keys:
+        assert np.array_equal(got[k][keep].cpu().numpy().view(np.uint8),
+                              want[k][keep].cpu().numpy().view(np.uint8)), k
