@@ -833,6 +833,9 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
     R.cap_refs = NR;
     ctx->refit_alloc = true;
   }
+  // (before the previous refit's record changes: it can still be differentiated
+  // after a refit refused here)
+  if (!map_room(ctx, mp)) return fail(ctx, TPC_ERR_OOM, "map buffer");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   ctx->last_stream = s;
   R.n_tracks = in->n_tracks;
@@ -848,7 +851,6 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* cl, const tpc_tracks* in,
   R.in_zsh = in->z_shift;
   R.row_x = F.row_x;
   R.freeze = freeze ? 1 : 0;
-  if (!map_room(ctx, mp)) return fail(ctx, TPC_ERR_OOM, "map buffer");
   R.map = make_mapdev(mp);
   R.map.c4 = ctx->map4;
   if (R.map.on) fast::map_pack(R.map, ctx->map4, s);

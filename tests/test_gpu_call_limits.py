@@ -139,3 +139,24 @@ def test_refit_skips_a_track_with_a_row_that_does_not_exist(row):
     for k in keys:
         assert np.array_equal(got[k][keep].cpu().numpy().view(np.uint8),
                               want[k][keep].cpu().numpy().view(np.uint8)), k
+
+
+def test_refit_without_room_for_its_map_leaves_the_last_one():
+    """A refit refused for want of memory for its map (1.3 TB here; nothing is
+    launched) does not touch the refit before it, which can still be
+    differentiated: the gradient's FP64 sums differ by their order only."""
+    import torch
+
+    from paper_2601_20569_gb300 import tpc
+
+    f, tr, dev, coeff, t = refit_setup()
+    nt = int(t["params"].shape[0])
+    w = torch.linspace(0.5, 1.5, nt, device="cuda")
+    tr.refit(dev, t, coeff)
+    want = tr.refit_backward(w).cpu().numpy()
+    huge = coeff.new_zeros(1).expand(3, 20000, 2000, 2000)
+    with pytest.raises(tpc.TpcError) as e:
+        tr.refit(dev, first_tracks(t, nt // 3), huge)
+    assert e.value.status == 5
+    got = tr.refit_backward(w, tuple(coeff.shape)).cpu().numpy()
+    assert np.abs(got - want).max() <= 2.0 ** -23 * np.abs(want).max()
