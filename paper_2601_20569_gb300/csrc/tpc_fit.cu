@@ -127,8 +127,9 @@ __device__ __forceinline__ void map_eval(const MapDev& M, const KParams& P, int 
 // The map's control points with their components side by side, packed anew for
 // every call (the caller may change the coefficients between calls).
 __global__ void k_map_pack(MapDev M, float4* c4) {
-  const int n = M.nz * M.nr * M.nphi;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+  const long n = (long)M.nz * M.nr * M.nphi;
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x)
     c4[i] = make_float4(M.c[i], M.c[n + i], M.c[2 * n + i], 0.0f);
 }
 

@@ -160,3 +160,29 @@ def test_refit_without_room_for_its_map_leaves_the_last_one():
     assert e.value.status == 5
     got = tr.refit_backward(w, tuple(coeff.shape)).cpu().numpy()
     assert np.abs(got - want).max() <= 2.0 ** -23 * np.abs(want).max()
+
+
+def test_map_of_more_than_2_31_coefficients():
+    """A constant map of 7.2e8 control points, read at its far end (every cluster of
+    side A lies above its z range): the shift of a small constant map.  The spline
+    weights sum to 1 within a few 2^-24, a correction of 0.25 cm to 1e-7 cm."""
+    import torch
+
+    f, tr, dev, coeff, t = refit_setup(n_primaries=100)
+    side_a = torch.nonzero(t["sector"] < 18).flatten().cpu().numpy()
+    assert len(side_a) > 20
+    out = []
+    for shape in ((2000, 2000, 180), (20, 16, 18)):
+        c = torch.zeros((3,) + shape, device="cuda")
+        c[2] = 0.25
+        r = tr.refit(dev, t, c, z_range=(-1000.0, 1.0))
+        out.append({k: r[k].cpu().numpy()[side_a].copy() for k in ("params", "n_clusters")})
+        del c, r
+    plain = tr.refit(dev, t, coeff.new_zeros(coeff.shape))["params"].cpu().numpy()[side_a]
+    big, small = out
+    fitted = (big["n_clusters"] > 0) & (big["n_clusters"] == small["n_clusters"])
+    assert fitted.sum() > 0.9 * len(side_a)
+    assert np.abs(np.median(big["params"][fitted, 1] - plain[fitted, 1]) - 0.25) < 0.01
+    assert np.abs(big["params"] - small["params"])[fitted, 1].max() < 1e-3
+    tr.close()
+    torch.cuda.empty_cache()
