@@ -197,7 +197,10 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* clusters, const tpc_track
  * respect to the map control points, references and decisions held fixed:
  * a hand-written adjoint sweeping iterations 3, 2, 1 in reverse with the
  * filter recomputed from checkpoints every 16 stations; per-track work in
- * FP32, the cross-track reduction in FP64.  dL_dchi2: device float[n_tracks];
+ * FP32, the cross-track reduction in FP64.  The first call allocates the step
+ * records of the refit's tracks, 46 KB each (at most 32,768 tracks at a time,
+ * 1.5 GB; fewer where there is no memory for them) and keeps them with the
+ * context.  dL_dchi2: device float[n_tracks];
  * dL_dmap: device float[3*n_z*n_r*n_phi] (overwritten).  TPC_ERR_STATE
  * without a preceding refit that used a map. */
 tpc_status tpc_refit_backward(tpc_ctx* ctx, const float* dL_dchi2, float* dL_dmap,

@@ -146,6 +146,31 @@ bool map_room(tpc_ctx* c, const tpc_map& m) {
   return true;
 }
 
+// Room for the adjoint's step records: as many tracks at a time as the refit has,
+// at most kAdjChunk, and half as many as often as there is no memory for them (the
+// adjoint runs over the tracks in chunks of R.chunk).  False without memory for one.
+bool record_room(tpc_ctx* c) {
+  RefitDev& R = c->R;
+  const long want = R.n_tracks < (long)kAdjChunk ? (R.n_tracks > 0 ? R.n_tracks : 1) : (long)kAdjChunk;
+  if (want <= R.chunk) return true;
+  // (rounded up to a power of two, so that refits of growing size seldom allocate)
+  long tracks = 256;
+  while (tracks < want) tracks *= 2;
+  cudaFree(R.rec);
+  R.rec = nullptr;
+  R.chunk = 0;
+  for (; tracks >= 1; tracks /= 2) {
+    void* v = nullptr;
+    if (cudaMalloc(&v, (size_t)tracks * kRecTrackBytes) == cudaSuccess) {
+      R.rec = (float4*)v;
+      R.chunk = (int)tracks;
+      return true;
+    }
+    cudaGetLastError();
+  }
+  return false;
+}
+
 // The buffers that the chain itself keeps from call to call: zero bin counts
 // (k_row_scan), empty bids (k_amb_resolve).  Set at the start, and again after a
 // call that stopped part-way (waiting for what it left in flight).
@@ -900,10 +925,7 @@ tpc_status tpc_refit_backward(tpc_ctx* ctx, const float* dl_dchi2, float* dl_dma
   R.ncoef = (int)ncoef;
   R.gblocks = ctx->sms;
   R.smem_max = smem_max;
-  if (!R.rec) {
-    const long tracks = R.cap < (long)kAdjChunk ? R.cap : (long)kAdjChunk;
-    if (!dalloc(ctx, &R.rec, tracks * 3 * kMaxRows * kRecV)) return fail(ctx, TPC_ERR_OOM, "adjoint records");
-  }
+  if (!record_room(ctx)) return fail(ctx, TPC_ERR_OOM, "adjoint records");
   if ((long)R.gblocks * ncoef > ctx->gpart_cap) {
     if (!dalloc(ctx, &R.gpart, (long)R.gblocks * ncoef)) return fail(ctx, TPC_ERR_OOM, "gradient partials");
     ctx->gpart_cap = (long)R.gblocks * ncoef;
@@ -1102,6 +1124,7 @@ void tpc_destroy(tpc_ctx* ctx) {
   if (!ctx) return;
   for (void* p : ctx->allocs) cudaFree(p);
   cudaFree(ctx->map4);
+  cudaFree(ctx->R.rec);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);

@@ -2780,7 +2780,7 @@ int refit_backward(RefitDev& R, const KParams& P, const int* steps3, int sms, cu
   int k = 0;
   long t0 = 0;
   do {
-    const int tn = (int)min(R.n_tracks - t0, (long)kAdjChunk);
+    const int tn = (int)min(R.n_tracks - t0, (long)R.chunk);
     if (tn > 0) {
       k_refit_replay<<<blocks_for((long)tn * 3 * kCkptSeg, 128), 128, 0, s>>>(R, P, steps3,
                                                                               (int)t0, tn);
@@ -2792,7 +2792,7 @@ int refit_backward(RefitDev& R, const KParams& P, const int* steps3, int sms, cu
     else
       k_refit_scatter<false><<<R.gblocks, 32 * warps, scat, s>>>(R, P, steps3, (int)t0, tn);
     ++k;
-    t0 += kAdjChunk;
+    t0 += R.chunk;
   } while (t0 < R.n_tracks);
   k_grad_reduce<<<blocks_for(R.ncoef, 32), 256, 0, s>>>(R);
   return k + 1;

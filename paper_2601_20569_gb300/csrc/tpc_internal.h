@@ -336,8 +336,9 @@ constexpr int kCkptF = 27;                             // p[5], c[15], ref[5], x
 
 constexpr int kRefitQueues = 4;   // start pass, iterations 1-3
 constexpr int kRecV = 6;          // float4 per step record of the adjoint
-// Tracks per chunk of the adjoint, which bounds its step records: 3 kMaxRows
-// steps of 96 bytes each at most, 1.5 GB.
+// Step records of a track in the adjoint: 3 kMaxRows steps of 96 bytes at most.
+constexpr long kRecTrackBytes = 3L * kMaxRows * kRecV * 16;
+// Most tracks per chunk of the adjoint: 1.5 GB of records.
 constexpr int kAdjChunk = 32768;
 
 // Refit of given tracks (fixed clusters) and its adjoint.
@@ -382,8 +383,9 @@ struct RefitDev {
   float* out_x;
   // adjoint
   const float* dl_dchi2;   // [n_tracks]
-  float4* rec;             // [min(cap, kAdjChunk)][3 kMaxRows][kRecV] adjoint: step
-                           // records of one chunk of tracks
+  float4* rec;             // [chunk][3 kMaxRows][kRecV] adjoint: step records of one chunk
+                           // of tracks
+  int chunk;               // tracks per chunk (a power of two, as memory allowed)
   double* gpart;           // [blocks][ncoef]
   float* dl_dmap;          // [ncoef]
   int ncoef;

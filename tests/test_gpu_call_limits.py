@@ -186,3 +186,48 @@ def test_map_of_more_than_2_31_coefficients():
     assert np.abs(big["params"] - small["params"])[fitted, 1].max() < 1e-3
     tr.close()
     torch.cuda.empty_cache()
+
+
+def test_adjoint_takes_memory_for_its_tracks_only():
+    """A context for up to 45,000 tracks, a refit of 200 of them: 200 step records of
+    46 KB (in steps of 2 MB, rounded up to 256) and the gradient's partial sums (21 MB)."""
+    import torch
+
+    f, tr, dev, coeff, t = refit_setup(n_primaries=300, cap_clusters=1_650_000)
+    few = first_tracks(t, 200)
+    w = torch.ones(200, device="cuda")
+    tr.refit(dev, few, coeff)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    tr.refit_backward(w)
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20
+
+
+def test_adjoint_in_the_memory_there_is():
+    """33,000 tracks with room for a quarter of their step records: the gradient of
+    the same refit with all of them (FP64 sums in another order)."""
+    import torch
+
+    f, tr, dev, coeff, t = refit_setup(n_primaries=1500, cap_clusters=3_500_000)
+    nt, nr = int(t["params"].shape[0]), int(t["cl_ids"].shape[0])
+    rep = -(-33000 // nt)
+    many = {k: t[k].repeat((rep,) + (1,) * (t[k].dim() - 1)) for k in ("cl_ids", "params", "x", "sector")}
+    step = torch.arange(rep, device="cuda", dtype=torch.int32)[:, None] * nr
+    many["cl_offset"] = torch.cat([(t["cl_offset"][:-1] + step).reshape(-1),
+                                   torch.tensor([rep * nr], device="cuda", dtype=torch.int32)])
+    w = torch.linspace(0.5, 1.5, rep * nt, device="cuda")
+    from paper_2601_20569_gb300 import tpc
+
+    tight = tpc.Tracker(RX, TrackerOptions(), mode=0, cap_clusters=3_500_000)
+    got = []
+    for x in (tr, tight):
+        x.refit(dev, many, coeff)
+        hog = None
+        if x is tight:  # (memory taken, not touched)
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            hog = torch.empty(torch.cuda.mem_get_info()[0] - (700 << 20), dtype=torch.uint8, device="cuda")
+        got.append(x.refit_backward(w).cpu().numpy().astype(np.float64))
+        del hog
+    torch.cuda.empty_cache()
+    assert np.abs(got[0] - got[1]).max() <= 2.0 ** -23 * np.abs(got[0]).max()
