@@ -157,7 +157,9 @@ typedef struct {
 
 /* Create a context: copies the geometry, derives the model constants from
  * bz and the options, allocates device buffers for opt->cap_clusters
- * clusters.  map may be NULL.  Sec. 2 (sector structure), Sec. 5 (the
+ * clusters (506 bytes per cluster and some 100 MB with the default capacities for
+ * tracklets and tracks; 16 bytes per control point of the largest map used).
+ * map may be NULL.  Sec. 2 (sector structure), Sec. 5 (the
  * deterministic mode is mode 0). */
 tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
                     const tpc_options* opt, tpc_ctx** out);

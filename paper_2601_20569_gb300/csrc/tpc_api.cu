@@ -377,7 +377,6 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   F.tl_order = F.st_tl;  // (the sector-track list comes after the constructor)
   ok &= dalloc(ctx, &F.st_off, T);
   F.cap_pos = n + n / 4 + 4096;
-  ok &= dalloc(ctx, &F.st_pos, F.cap_pos);
   ok &= dalloc(ctx, &F.st_order, T);
   ok &= dalloc(ctx, &F.st_obucket, T);
   ok &= dalloc(ctx, &F.st_oslot, T);
@@ -432,7 +431,12 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.ft_st_cl, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_st_rs, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_meas, FT * kMaxRows);
-  ok &= dalloc(ctx, &F.ft_store, FT * kMaxRows * 5);
+  // iteration 1's predictions, which iteration 2 reads; before that the kept
+  // clusters' positions, after it the clusters used lie there
+  const long store4 = (FT * kMaxRows * 5 + 3) / 4;  // in float4
+  ok &= dalloc(ctx, &F.st_pos, store4 > F.cap_pos ? store4 : F.cap_pos);
+  F.ft_store = (float*)F.st_pos;
+  F.ft_used = (int*)F.st_pos;
   ok &= dalloc(ctx, &F.ft_flag, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_end2, FT * kStateF);
   F.nslot = kMaxInner + 2 * opt->ext_rows;
@@ -444,14 +448,13 @@ tpc_status tpc_init(const tpc_geometry* geo, float bz_tesla, const tpc_map* map,
   ok &= dalloc(ctx, &F.ft_next, FT);
   ok &= dalloc(ctx, &F.ft_nout, FT);
   ok &= dalloc(ctx, &F.ft_ext_sec, FT * (opt->ext_rows > 0 ? 2 * opt->ext_rows : 1));
-  ok &= dalloc(ctx, &F.ft_ipol, FT * kMaxInner * kIpolF);
+  ok &= dalloc(ctx, &F.ft_ref34, FT);
   ok &= dalloc(ctx, &F.ft_fixed, n + 3);  // (cleared in words)
   ok &= dalloc(ctx, &F.bid, n);
   ok &= dalloc(ctx, &F.taken, n + 3);  // (cleared in words)
   ok &= dalloc(ctx, &F.ft_n, FT);
   ok &= dalloc(ctx, &F.ft_chi2, FT);
   ok &= dalloc(ctx, &F.ft_out, FT * kStateF);
-  ok &= dalloc(ctx, &F.ft_used, FT * kMaxRows);
   ok &= dalloc(ctx, &F.ft_outidx, FT);
   ok &= dalloc(ctx, &F.cr_cls, FT);
   ok &= dalloc(ctx, &F.ft_side0, FT);

@@ -1572,6 +1572,15 @@ __global__ void __launch_bounds__(256, 2) k_fit1(FrameDev F, KParams P, MapDev M
   }
 }
 
+// Interpolation record of inner station k of track f, from k_fit2 for k_inner_cand:
+// (y, z, Cyy, Cyz, Czz, reference y, z, sin phi; the reference's tan(lambda) and
+// q/pT do not change along a track, and x is the row's).  It lies where the
+// station's candidates' chi2 go, which the thread that reads it then writes.
+static_assert(kMaxCand * sizeof(float) == 2 * sizeof(float4), "interpolation record");
+__device__ __forceinline__ float4* ipol_rec(const FrameDev& F, int f, int k) {
+  return (float4*)(F.ft_cchi + ((long)f * F.nslot + k) * kMaxCand);
+}
+
 // Iteration 2 (outward) as the same kind of state machine: interpolation with
 // the stored predictions, flags of outliers, inner-row candidates (Sec. 3,
 // Phases I and II), then (kExt) the Phase III extrapolation above the
@@ -1625,6 +1634,7 @@ __global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M
       Trk<float> s1;
       get_state(F.ft_end2 + (long)f * kStateF, s1);
       lin_start(L, s1, st_sector(nxt), P);
+      F.ft_ref34[f] = make_float2(L.r[3], L.r[4]);
       k = 0;
       phase = kFit2St;
       continue;
@@ -1677,11 +1687,9 @@ __global__ void __launch_bounds__(256, 2) k_fit2(FrameDev F, KParams P, MapDev M
       if (ok && inner) {
         // Phase II candidates of this inner station: the search runs later in
         // k_inner_cand, over all (track, inner station) pairs at once
-        float* ip = F.ft_ipol + ((long)f * kMaxInner + k) * kIpolF;
-        ip[0] = I.y; ip[1] = I.z; ip[2] = I.c00; ip[3] = I.c01; ip[4] = I.c11;
-        ip[5] = L.t.x;
-#pragma unroll
-        for (int i = 0; i < 5; ++i) ip[6 + i] = L.r[i];
+        float4* ip = ipol_rec(F, f, k);
+        ip[0] = make_float4(I.y, I.z, I.c00, I.c01);
+        ip[1] = make_float4(I.c11, L.r[0], L.r[1], L.r[2]);
       }
     }
     if (have) update_as(L.t, residual(L.t, my, mz, P), lp);
@@ -1719,18 +1727,13 @@ __global__ void k_inner_cand(FrameDev F, KParams P, MapDev M) {
       F.ft_ncand[(long)f * F.nslot + k] = 0;  // (the ambiguity looks at the count only)
       continue;
     }
-    const float* ip = F.ft_ipol + ((long)f * kMaxInner + k) * kIpolF;
-    Interp I;
-    I.y = ip[0];
-    I.z = ip[1];
-    I.c00 = ip[2];
-    I.c01 = ip[3];
-    I.c11 = ip[4];
-    float ref[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) ref[i] = ip[6 + i];
+    const float4* ip = ipol_rec(F, f, k);
+    const float4 u = ip[0], v = ip[1];
+    const float2 w34 = F.ft_ref34[f];
+    const Interp I{u.x, u.y, u.z, u.w, v.x};
+    const float ref[5] = {v.y, v.z, v.w, w34.x, w34.y};
     const int rs = F.ft_st_rs[(long)f * kMaxRows + k];
-    inner_candidates(F, P, M, f, k, rs, ip[5], ref, I, F.ft_z0[f],
+    inner_candidates(F, P, M, f, k, rs, F.row_x[rs % P.n_rows], ref, I, F.ft_z0[f],
                      row_shift(rs / P.n_rows, shift_side(F, f), F.ft_zsh[f], P));
   }
 }

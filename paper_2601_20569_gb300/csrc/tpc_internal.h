@@ -96,7 +96,6 @@ constexpr int kMaxBinOcc = 1024;
 
 constexpr int kStateF = 22;     // p[5], c[15], x, sector (as float)
 constexpr int kSeedF = 8;       // tracklet seed: p[5], x, sector*n_rows + row, valid
-constexpr int kIpolF = 11;      // interpolation record of an inner station
 constexpr int kMergeLanesDefault = 32;  // lanes per outer end in the merge search
 constexpr int kLinksLanesDefault = 1;   // lanes per cluster in the neighbour search (32: staged per warp)
 constexpr int kMergeZ = 512;     // z bins per sector of the merge candidate index
@@ -235,7 +234,8 @@ struct FrameDev {
   int* st_off;             // first entry of the track's kept-cluster positions (-1: none,
                            // a segment found by the edge following)
   float4* st_pos;          // [cap_pos] (x, y, z, sector*n_rows + row bits) of kept clusters,
-                           // outermost first per track
+                           // outermost first per track (up to the station lists; in the
+                           // place of ft_store, which iteration 1 fills)
   long cap_pos;
   int* st_order;           // order in which the sector refit takes the tracks
   int* st_obucket;         // scheduling bucket
@@ -295,21 +295,22 @@ struct FrameDev {
   int nslot;
   uint8_t* ft_ncand;       // [cap_ft][nslot]
   int* ft_cand;            // [cap_ft][nslot][kMaxCand]
-  float* ft_cchi;          // [cap_ft][nslot][kMaxCand]
+  float* ft_cchi;          // [cap_ft][nslot][kMaxCand] (before the search: the inner stations'
+                           // interpolation records)
   int* ft_assigned;        // [cap_ft][nslot]
   int* ft_next;            // [cap_ft] rows extrapolated below the innermost station
   int* ft_nout;            // [cap_ft] rows extrapolated above the outermost station
   uint16_t* ft_ext_sec;    // [cap_ft][2 ext_rows] sector of each extrapolated row (inward,
                            // then outward): the extrapolation may cross a sector edge
-  float* ft_ipol;          // [cap_ft][kMaxInner][kIpolF] iteration-2 interpolation at inner
-                           // stations (y, z, Cyy, Cyz, Czz, x, reference p[5]) for k_inner_cand
+  float2* ft_ref34;        // [cap_ft] iteration 2's reference tan(lambda) and q/pT
   uint8_t* ft_fixed;       // [n] sorted cluster held by a station outside the inner region
   unsigned long long* bid; // [n] per sorted cluster
   uint8_t* taken;          // [n]
   int* ft_n;               // iteration 3 results
   float* ft_chi2;
   float* ft_out;           // [cap_ft][kStateF]
-  int* ft_used;            // [cap_ft][kMaxRows] sorted clusters, outermost first
+  int* ft_used;            // [cap_ft][kMaxRows] sorted clusters, outermost first (iteration 3
+                           // on; in the place of ft_store)
   // a11 outputs
   int* ft_outidx;          // compaction index of accepted fit tracks
   float* out_par;

@@ -231,3 +231,23 @@ def test_adjoint_in_the_memory_there_is():
         del hog
     torch.cuda.empty_cache()
     assert np.abs(got[0] - got[1]).max() <= 2.0 ** -23 * np.abs(got[0]).max()
+
+
+@pytest.mark.parametrize("ext", [0, 8])
+def test_device_memory_of_a_context(ext):
+    """What tpc.h states per cluster of capacity, and the candidates of the
+    extrapolated rows; each of some hundred buffers rounded up to 2 MB at most."""
+    import torch
+
+    from paper_2601_20569_gb300 import tpc
+
+    n = 40_000_000
+    tpc.Tracker(RX, TrackerOptions(), mode=0, cap_clusters=1024).close()  # (loads the library)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    tr = tpc.Tracker(RX, TrackerOptions(ext_rows=ext), mode=0, cap_clusters=n)
+    used = free - torch.cuda.mem_get_info()[0]
+    tr.close()
+    tracks = n / 40 + 4096
+    per_ext_row = 2 * (8 * 8 + 4 + 1 + 2)  # candidates, chi2, assignment, count, sector
+    assert used < 512 * n + ext * per_ext_row * tracks + (256 << 20)
