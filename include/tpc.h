@@ -199,7 +199,8 @@ tpc_status tpc_refit(tpc_ctx* ctx, const tpc_clusters* clusters, const tpc_track
  * respect to the map control points, references and decisions held fixed:
  * a hand-written adjoint sweeping iterations 3, 2, 1 in reverse with the
  * filter recomputed from checkpoints every 16 stations; per-track work in
- * FP32, the cross-track reduction in FP64.  The first call allocates the step
+ * FP32, the reduction over clusters and tracks in FP64 (a track's clusters of one
+ * map cell first in three FP32 words, which is finer).  The first call allocates the step
  * records of the refit's tracks, 46 KB each (at most 32,768 tracks at a time,
  * 1.5 GB; fewer where there is no memory for them) and keeps them with the
  * context.  dL_dchi2: device float[n_tracks];

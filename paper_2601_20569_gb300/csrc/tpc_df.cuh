@@ -87,6 +87,21 @@ TPC_DF void df_dot2(float a, float x, float b, float y, float& hi, float& lo) {
   lo = df_add(e, df_add(pe, qe));
 }
 
+// hi + mid + lo += a * b: a sum of products in three floats, where a pair would
+// lose FP64's last bits.  The product and its sums into hi and mid are exact; only
+// the sums into lo round.  With S the sum of the n terms' magnitudes, a term leaves
+// at most 2^-24 S from hi, so |mid| <= 2 n 2^-24 S, |lo| <= 4 n^2 2^-48 S, and the n
+// times two roundings at lo come to 8 n^3 2^-72 S at most: below the n 2^-53 S of a
+// sum in FP64 for n < 256.  Products below 2^-102 lose what is below 2^-149.
+TPC_DF void tf_add_product(float& hi, float& mid, float& lo, float a, float b) {
+  float p, pe, e0, e1, e2;
+  two_prod(a, b, p, pe);
+  two_sum(hi, p, hi, e0);
+  two_sum(mid, e0, mid, e1);
+  two_sum(mid, pe, mid, e2);
+  lo = df_add(lo, df_add(e1, e2));
+}
+
 // fl(v +- ((kh + kl) * x + (gh + gl) * y)) (kSub: minus): the two products of
 // a double-float by a float (the hi part's product exact, the lo part's
 // rounded), their sum with v compensated, one final rounding.

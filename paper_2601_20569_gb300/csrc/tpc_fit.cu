@@ -2601,13 +2601,17 @@ __global__ void __launch_bounds__(kRevBlock) k_refit_reverse(RefitDev R, const i
 // then the warp takes the clusters in track order, each lane holding two of the
 // cell's 64 control points for the three components.  A track stays about ten
 // clusters in one cell, so the lanes sum in registers and add to the FP64
-// accumulators only where the cell changes.  Those sums are kept as float pairs
-// (TwoProduct / TwoSum, 2^-46 relative): this GPU's FP64 rate is 1/60 of its
-// FP32 rate, and 192 FP64 operations per cluster would cost more than the whole
-// sweep.  kShared: the block's accumulators lie in shared memory; a map too large
-// for that has them in the block's partial sums in global memory.
+// accumulators only where the cell changes.  Those sums are kept in three floats
+// (tf_add_product: finer than FP64 up to a track's 160 clusters): this GPU's FP64
+// rate is 1/60 of its FP32 rate, and 192 FP64 operations per cluster would cost
+// more than the whole sweep.  Clusters whose gradients leave the range in which that holds (kSumLow,
+// kSumHigh; infinities and NaN) are added term by term in FP64.  kShared: the
+// block's accumulators lie in shared memory; a map too large for that has them in
+// the block's partial sums in global memory.
 constexpr int kScatWarps = 16;
 constexpr int kScatF = 16;  // floats per staged cluster: wz[4], wr[4], wp[4], g[3], cell
+constexpr unsigned kSumLow = (127u - 40u) << 23;    // 2^-40: 2^-149 is 2^-109 of the largest
+constexpr unsigned kSumHigh = (127u + 100u) << 23;  // 2^100: 160 terms do not overflow
 
 template <bool kShared>
 __global__ void __launch_bounds__(32 * kScatWarps) k_refit_scatter(RefitDev R, KParams P,
@@ -2632,23 +2636,27 @@ __global__ void __launch_bounds__(32 * kScatWarps) k_refit_scatter(RefitDev R, K
     const int n3 = steps3[t];
     const float z0 = R.z0[t];
     const float4* rec = adj_rec(R, q);
-    float hi[6], lo[6];  // [component][point]
+    float hi[6], mid[6], lo[6];  // [component][point]
     int cell = -1;
+    auto point = [&](int c, int e) {  // the lane's control point e of cell c
+      const int zr = c / M.nphi;      // (z, r) cell corner
+      return ((zr / M.nr + la) * M.nr + (zr % M.nr + lb)) * M.nphi +
+             phi_index(c % M.nphi, lh + e, M.nphi);
+    };
     auto flush = [&]() {
       if (cell < 0) return;
-      const int nphi = M.nphi, ip = cell % nphi;
-      const int zr = cell / nphi;  // (z, r) cell corner
-      const int row = ((zr / M.nr + la) * M.nr + (zr % M.nr + lb)) * nphi;
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const int at = row + phi_index(ip, lh + e, nphi);
+        const int at = point(cell, e);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          atomicAdd(&gacc[c * ncomp + at], (double)hi[2 * c + e] + (double)lo[2 * c + e]);
+          atomicAdd(&gacc[c * ncomp + at],
+                    (double)hi[2 * c + e] + ((double)mid[2 * c + e] + (double)lo[2 * c + e]));
       }
     };
     for (int k0 = 0; k0 < ns; k0 += 32) {
       const int k = k0 + lane;
+      unsigned gmax = 0u;  // largest magnitude of the gradients (as bits: NaN above infinity)
       if (k < ns) {
         const float2 yz = R.raw[o0 + k];
         const int w = __float_as_int(R.meas[o0 + k].w);
@@ -2674,33 +2682,42 @@ __global__ void __launch_bounds__(32 * kScatWarps) k_refit_scatter(RefitDev R, K
         d[12] = gx;
         d[13] = gy;
         d[14] = gz;
+        gmax = max(__float_as_uint(fabsf(gx)),
+                   max(__float_as_uint(fabsf(gy)), __float_as_uint(fabsf(gz))));
         // (phi_index wraps its argument, so the cell's phi can be wrapped here)
         const int ipw = ((sp.ip % M.nphi) + M.nphi) % M.nphi;
         d[15] = __int_as_float((sp.iz * M.nr + sp.ir) * M.nphi + ipw);
       }
       __syncwarp();
-      const int m = min(32, ns - k0);
+      gmax = __reduce_max_sync(0xffffffffu, gmax);
+      const int m = gmax != 0u ? min(32, ns - k0) : 0;
+      const bool wide = gmax < kSumLow || gmax >= kSumHigh;
       for (int i = 0; i < m; ++i) {
         const float* d = st + i * kScatF;
         const int c = __float_as_int(d[15]);
+        const float wzr = d[la] * d[4 + lb];
+        if (wide) {
+#pragma unroll 1
+          for (int eg = 0; eg < 6; ++eg) {
+            const int e = eg & 1, g = eg >> 1;
+            if (d[12 + g] != 0.0f)
+              atomicAdd(&gacc[g * ncomp + point(c, e)],
+                        (double)(wzr * d[8 + lh + e]) * (double)d[12 + g]);
+          }
+          continue;
+        }
         if (c != cell) {
           flush();
           cell = c;
 #pragma unroll
-          for (int e = 0; e < 6; ++e) hi[e] = lo[e] = 0.0f;
+          for (int e = 0; e < 6; ++e) hi[e] = mid[e] = lo[e] = 0.0f;
         }
-        const float wzr = d[la] * d[4 + lb];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const float w = wzr * d[8 + lh + e];
 #pragma unroll
-          for (int g = 0; g < 3; ++g) {
-            float p, pe, s, se;
-            two_prod(w, d[12 + g], p, pe);
-            two_sum(hi[2 * g + e], p, s, se);
-            lo[2 * g + e] = df_add(lo[2 * g + e], df_add(se, pe));
-            hi[2 * g + e] = s;
-          }
+          for (int g = 0; g < 3; ++g)
+            tf_add_product(hi[2 * g + e], mid[2 * g + e], lo[2 * g + e], w, d[12 + g]);
         }
       }
       __syncwarp();

@@ -251,3 +251,24 @@ def test_device_memory_of_a_context(ext):
     tracks = n / 40 + 4096
     per_ext_row = 2 * (8 * 8 + 4 + 1 + 2)  # candidates, chi2, assignment, count, sector
     assert used < 512 * n + ext * per_ext_row * tracks + (256 << 20)
+
+
+@pytest.mark.parametrize("shape", [(20, 16, 18), (20, 24, 20)])  # sums in shared memory, in global
+def test_adjoint_of_very_small_and_large_weights(shape):
+    """The gradient is linear in the weights, and a power of two scales every float
+    exactly: with weights outside the three-float sums' range (term by term in FP64)
+    it is the scaled gradient, within one rounding to float and, where elements
+    cancel, the FP64 sums' 2^-53 of the terms (at most 2^-40 of the largest)."""
+    import torch
+
+    f, tr, dev, coeff, t = refit_setup(n_primaries=400)
+    coeff = torch.as_tensor(0.05 * np.random.default_rng(2).standard_normal((3,) + shape),
+                            dtype=torch.float32).cuda()
+    nt = int(t["params"].shape[0])
+    w = torch.linspace(0.5, 1.5, nt, device="cuda")
+    tr.refit(dev, t, coeff)
+    want = tr.refit_backward(w).cpu().numpy().astype(np.float64)
+    assert np.abs(want).max() > 1.0
+    for k in (-70, 105):
+        got = tr.refit_backward(w * 2.0 ** k).cpu().numpy().astype(np.float64) * 2.0 ** -k
+        assert np.all(np.abs(got - want) <= 2.0 ** -23 * np.abs(want) + 2.0 ** -40 * np.abs(want).max())
