@@ -2802,9 +2802,11 @@ int refit_backward(RefitDev& R, const KParams& P, const int* steps3, int sms, cu
     warps = kScatWarps;
   }
   const size_t scat = (shared ? acc : 0) + warps * stage;
+  // (process-wide attributes: the same values in every call, whatever its map, so that
+  // no other context's thread lowers a limit between this call's set and launch)
   cudaFuncSetAttribute(k_refit_reverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rev);
   cudaFuncSetAttribute(k_refit_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       shared ? (int)scat : 0);
+                       R.smem_max);
   int k = 0;
   long t0 = 0;
   do {

@@ -281,10 +281,12 @@ def test_adjoint_of_an_infinite_weight():
     import torch
 
     f, tr, dev, _, t = refit_setup(n_primaries=300, final_chi2=1.5, int_chi2=3.0)
-    # (28,800 control points: cells of 9 cm in r and 14 cm in z)
+    # (28,800 coefficients; the ranges beyond every cluster: a clamped one would have
+    # weights of exactly 0, and 0 x infinity in their place)
     coeff = torch.as_tensor(0.02 * np.random.default_rng(4).standard_normal((3, 40, 20, 12)),
                             dtype=torch.float32).cuda()
-    n = tr.refit(dev, t, coeff)["n_clusters"].cpu().numpy().copy()
+    n = tr.refit(dev, t, coeff, r_range=(80.0, 270.0),
+                 z_range=(-300.0, 300.0))["n_clusters"].cpu().numpy().copy()
     have = np.diff(t["cl_offset"].cpu().numpy())
     nt = len(n)
     assert np.sum(n) < 0.8 * np.sum(have[n > 0])
@@ -296,3 +298,44 @@ def test_adjoint_of_an_infinite_weight():
         inf = tr.refit_backward(w).cpu().numpy()
         assert not np.isfinite(inf).all()
         assert np.isfinite(inf[one == 0.0]).all(), int(i)
+
+
+def test_adjoints_of_two_contexts_on_two_threads():
+    """Maps of 138 KB, 14 KB and 230 KB of accumulators (the last beyond shared
+    memory) side by side: the attributes of the kernels belong to the process."""
+    import threading
+
+    import torch
+
+    f, tr, dev, coeff, t = refit_setup(n_primaries=60)
+    rng = np.random.default_rng(6)
+    nt = int(t["params"].shape[0])
+    failed = []
+
+    def worker(shape):
+        from paper_2601_20569_gb300 import tpc
+
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                c = torch.as_tensor(0.02 * rng_maps[shape]).cuda()
+                w = torch.ones(nt, device="cuda")
+                x = tpc.Tracker(RX, TrackerOptions(), mode=0, cap_clusters=f.n)
+                x.refit(dev, t, c)
+                want = x.refit_backward(w).cpu().numpy()
+                for _ in range(400):
+                    got = x.refit_backward(w).cpu().numpy()
+                    if np.abs(got - want).max() > 2.0 ** -23 * np.abs(want).max():
+                        failed.append((shape, "gradient"))
+                x.close()
+        except Exception as e:  # (reported by the test's own thread)
+            failed.append((shape, repr(e)))
+
+    shapes = [(20, 16, 18), (6, 6, 16), (20, 24, 20)]
+    rng_maps = {s: rng.standard_normal((3,) + s).astype(np.float32) for s in shapes}
+    threads = [threading.Thread(target=worker, args=(s,)) for s in shapes]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed[:3]
