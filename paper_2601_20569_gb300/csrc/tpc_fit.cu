@@ -1041,21 +1041,17 @@ __device__ __forceinline__ bool lin_propagate(Lin& L, float xnew, const KParams&
 }
 
 // Station change: rotation (when the sector changes) and propagation.  The
-// optional records receive the rotation Jacobian (jrec, *rotated set) and the
-// propagation Jacobian (frec) for the adjoint.
+// optional records receive the rotation Jacobian (jrec, untouched without a
+// rotation) and the propagation Jacobian (frec) for the adjoint.
 __device__ __forceinline__ bool lin_goto(Lin& L, int sector, float x, const KParams& P,
-                                         float* jrec = nullptr, bool* rotated = nullptr,
-                                         StepJ* frec = nullptr) {
-  if (rotated) *rotated = false;
+                                         float* jrec = nullptr, StepJ* frec = nullptr) {
   if (sector != L.sector) {
     const int half = P.n_phi;
     const int ds = ((sector % half) - (L.sector % half) + half) % half;
     if (ds == 1) {
       if (!lin_rotate(L, 1, P, jrec)) return false;
-      if (rotated) *rotated = true;
     } else if (ds == half - 1) {
       if (!lin_rotate(L, -1, P, jrec)) return false;
-      if (rotated) *rotated = true;
     } else if (ds != 0) {
       return false;
     }
@@ -2482,7 +2478,7 @@ __global__ void __launch_bounds__(128, 4) k_refit_replay(RefitDev R, KParams P,
     float k0[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, k1[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     float q0 = 0.0f, q1 = 0.0f, gy = no_step(), gz = 0.0f;
     bool go = true;
-    if (j != 0) go = lin_goto(L, w >> 8, R.row_x[w & 0xFF], P, jr, nullptr, &S);
+    if (j != 0) go = lin_goto(L, w >> 8, R.row_x[w & 0xFF], P, jr, &S);
     if (go && !(it == 2 && (R.flag[o0 + k] || !R.acc[o0 + k]))) {
       // the measurement with its derivative by the x displacement
       float my = m.y, mz = m.z, snp1 = L.r[2];
@@ -2885,9 +2881,6 @@ int fit12(FrameDev& F, const KParams& P, int sms, cudaStream_t s) {
   const int b = F.lc.block[kLFit12];
   k_fit_stations<kMap><<<sms * 8, kBlock, 0, s>>>(F, P, F.map);
   k_fit_order<<<sms * 4, kBlock, 0, s>>>(F);
-  // iterations 1 and 2 keep loopers and other tracks in one launch (split in
-  // two parts, as iteration 3 is, they measured slower: 22.4 -> 25.1 ms per
-  // batch, the two kinds of track no longer sharing the warps)
   if (P.ext_rows > 0) {
     k_fit1<kMap, true><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit1<kMap, true>>(b, 0, g, sms));
     k_fit2<kMap, true><<<g, b, 0, s>>>(F, P, F.map, resident_lanes<k_fit2<kMap, true>>(b, 0, g, sms));

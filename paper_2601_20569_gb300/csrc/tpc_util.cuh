@@ -81,19 +81,6 @@ __device__ __forceinline__ StripRun strip_run(const int* __restrict__ bin_first,
   return r;
 }
 
-// for_window over such runs (the same clusters in the same order).
-template <typename Fn>
-__device__ __forceinline__ void for_window_flat(const int* __restrict__ bin_first, const RowGrid& g,
-                                           float ylo, float yhi, float zlo, float zhi, Fn&& fn) {
-  if (g.ncl == 0 || !(ylo <= yhi) || !(zlo <= zhi)) return;
-  const int iy0 = bin_of(ylo, g.y0, g.invDy, g.nY), iy1 = bin_of(yhi, g.y0, g.invDy, g.nY);
-  const int iz0 = bin_of(zlo, g.z0, g.invDz, g.nZ), iz1 = bin_of(zhi, g.z0, g.invDz, g.nZ);
-  for (int iz = iz0; iz <= iz1; iz += kStrips) {
-    const StripRun r = strip_run(bin_first, g, iy0, iy1, iz, iz1);
-    for (int c = 0; c < r.n; ++c) fn(r.at(c));
-  }
-}
-
 __device__ __forceinline__ int block_exscan(int v, int* sh_warp, int* total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int x = v;

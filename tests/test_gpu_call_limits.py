@@ -311,6 +311,7 @@ def test_adjoints_of_two_contexts_on_two_threads():
     rng = np.random.default_rng(6)
     nt = int(t["params"].shape[0])
     failed = []
+    torch.cuda.synchronize()
 
     def worker(shape):
         from paper_2601_20569_gb300 import tpc
