@@ -340,3 +340,63 @@ def test_adjoints_of_two_contexts_on_two_threads():
     for th in threads:
         th.join()
     assert not failed, failed[:3]
+
+
+@pytest.mark.parametrize("length", [1, 2, 15, 16, 17, 31, 32, 33, 48, 49, 64, 65, 100])
+def test_adjoint_of_tracks_of_one_length(length):
+    """The adjoint against the FP64 tape for tracks cut to one length, each with a norm
+    of its own.  With clusters of 3 cm resolution the fit follows no cluster, so
+    residuals stay near the map's random 0.2 cm at every length; the forward states
+    round by up to 4 x 2^-24 x 250 cm per step, over 100 steps 10 times that: 6e-4 cm,
+    below 5e-3 of the residuals."""
+    import torch
+
+    import oracle
+    from paper_2601_20569_gb300 import tpc
+    from tests.test_gpu_refit import device_tracks, host_tracks
+
+    f, tr, dev, _, t = refit_setup(n_primaries=250)
+    tr.close()
+    dmap = (0.6 * np.random.default_rng(11).standard_normal((3, 20, 16, 18))).astype(np.float32)
+    h = host_tracks(t)
+    sel = np.nonzero(np.diff(h["offset"]) >= length)[0][:150]
+    assert len(sel) > 30
+    h = host_tracks(t, sel)
+    ids = np.concatenate([h["ids"][o:o + length] for o in h["offset"][:-1]])
+    h = dict(h, ids=ids, offset=np.arange(0, len(ids) + 1, length, dtype=np.int32))
+    opts = TrackerOptions(sigma_y=3.0, sigma_z=3.0).as_dict()
+    x = tpc.Tracker(RX, opts, mode=0, cap_clusters=f.n)
+    w = np.random.default_rng(12).uniform(0.5, 1.5, len(sel))
+    out = x.refit(dev, device_tracks(h), torch.as_tensor(dmap).cuda())
+    r = oracle.refit(f.y, f.z, f.row, f.sector, RX, opts, h, dist_map=dmap, mode="f32")
+    assert np.array_equal(out["n_clusters"].cpu().numpy(), r["rf_n"])
+    assert (r["rf_n"] > 0).sum() > 0.8 * len(sel)
+    g = x.refit_backward(torch.as_tensor(w, dtype=torch.float32).cuda()).cpu().numpy().ravel()
+    tape = oracle.refit(f.y, f.z, f.row, f.sector, RX, opts, h, dist_map=dmap, frozen=r, weights=w,
+                        mode="tape")["grad"]
+    assert np.linalg.norm(tape) > 0
+    assert np.linalg.norm(g - tape) < 5e-3 * np.linalg.norm(tape)
+    x.close()
+
+
+def test_refit_with_a_larger_map_between_replayed_graphs():
+    """A refit whose map needs more room than the tracker's replaces the packed map
+    that a captured chain reads: the chain is captured again."""
+    import torch
+
+    from paper_2601_20569_gb300 import tpc
+
+    f = synth.generate("central_event", n_primaries=300, distort=True)
+    rng = np.random.default_rng(9)
+    small, large = (torch.as_tensor((0.05 * rng.standard_normal(s)).astype(np.float32)).cuda()
+                    for s in ((3, 5, 6, 7), (3, 40, 30, 36)))
+    tr = tpc.Tracker(RX, TrackerOptions(), mode=0, cap_clusters=f.n, use_graphs=True)
+    tr.set_map(small)
+    dev = tr.to_device(f.y, f.z, f.q, f.row, f.sector)
+    want = tracks(tr, dev)
+    assert same(tracks(tr, dev), want)
+    t = {k: tr.result()[k].clone() for k in REFIT_KEYS}
+    tr.refit(dev, t, large)
+    hold = torch.full((1 << 20,), float("nan"), device="cuda")  # (the freed room's next user)
+    assert same(tracks(tr, dev), want) and same(tracks(tr, dev), want)
+    assert bool(torch.isnan(hold).all())
