@@ -2441,13 +2441,10 @@ __global__ void __launch_bounds__(128, 4) k_refit_iter(RefitDev R, KParams P, in
 // 1.2e6-cluster frame.)
 //
 // Step record: F (f02, f04, f12, f13, f14, f24), W r of a step counted in
-// chi2, d(measurement)/d(x displacement), gain columns k0 and k1, the
-// rotation's (j00, j10, j20, j22).  A step without propagation, update or rotation
-// has infinity (no_step) in the first of its words, and the sweep leaves it out as
-// such: zeros and identities in its place would turn the infinite weights or
-// adjoints of one track into NaN where it has no gradient.  The reverse sweep
-// replaces the first float4 by the gradient by the step's (x displacement, y, z).
-__device__ __forceinline__ float no_step() { return __int_as_float(0x7f800000); }
+// chi2 (else 0), d(measurement)/d(x displacement), gain columns k0 and k1, the
+// rotation's (j00, j10, j20, j22) (else the identity's); zeros where a step has
+// no propagation or no update.  The reverse sweep replaces the first float4 by
+// the gradient by the step's (x displacement, y, z).
 __device__ __forceinline__ float4* adj_rec(const RefitDev& R, int q) {  // track q of the chunk
   return R.rec + (long)q * 3 * kMaxRows * kRecV;
 }
@@ -2472,11 +2469,10 @@ __global__ void __launch_bounds__(128, 4) k_refit_replay(RefitDev R, KParams P,
     const float4 m = R.meas[o0 + k];
     const int w = __float_as_int(m.w);
     StepJ S;
-    S.f04 = S.f12 = S.f13 = S.f14 = S.f24 = 0.0f;
-    S.f02 = no_step();
-    float jr[4] = {no_step(), 0.0f, 0.0f, 0.0f};
+    S.f02 = S.f04 = S.f12 = S.f13 = S.f14 = S.f24 = 0.0f;
+    float jr[4] = {1.0f, 0.0f, 0.0f, 1.0f};
     float k0[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, k1[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    float q0 = 0.0f, q1 = 0.0f, gy = no_step(), gz = 0.0f;
+    float q0 = 0.0f, q1 = 0.0f, gy = 0.0f, gz = 0.0f;
     bool go = true;
     if (j != 0) go = lin_goto(L, w >> 8, R.row_x[w & 0xFF], P, jr, &S);
     if (go && !(it == 2 && (R.flag[o0 + k] || !R.acc[o0 + k]))) {
@@ -2571,27 +2567,23 @@ __global__ void __launch_bounds__(kRevBlock) k_refit_reverse(RefitDev R, const i
       const float4 v4 = d[(e * kRecV + 4) * kRevBlock], v5 = d[(e * kRecV + 5) * kRevBlock];
       const float k0[5] = {v2.z, v2.w, v3.x, v3.y, v3.z};
       const float k1[5] = {v3.w, v4.x, v4.y, v4.z, v4.w};
-      float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (v2.x != no_step()) {
-        const bool counted = i >= 2 * ns;  // (an update of iteration 3)
-        float a0 = counted ? w2 * v1.z : 0.0f, a1 = counted ? w2 * v1.w : 0.0f;
+      float a0 = w2 * v1.z, a1 = w2 * v1.w;
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-          a0 += k0[j] * lam[j];
-          a1 += k1[j] * lam[j];
-        }
-        g = make_float4(v2.x * a0 + v2.y * a1, a0, a1, 0.0f);
-        lam[0] -= a0;
-        lam[1] -= a1;
+      for (int j = 0; j < 5; ++j) {
+        a0 += k0[j] * lam[j];
+        a1 += k1[j] * lam[j];
       }
-      rec[(long)i * kRecV] = g;
-      if (v0.x != no_step()) {
+      // (a step without an update has k = g = 0 here and no gradient)
+      rec[(long)i * kRecV] = make_float4(v2.x * a0 + v2.y * a1, a0, a1, 0.0f);
+      lam[0] -= a0;
+      lam[1] -= a1;
+      {
         const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
         lam[2] = l2 + v0.x * l0 + v0.z * l1;
         lam[3] = lam[3] + v0.w * l1;
         lam[4] = lam[4] + v0.y * l0 + v1.x * l1 + v1.y * l2;
       }
-      if (v5.x != no_step()) {
+      {
         const float l0 = lam[0], l1 = lam[1], l2 = lam[2];
         lam[0] = v5.x * l0 + v5.y * l1 + v5.z * l2;
         lam[2] = v5.w * l2;

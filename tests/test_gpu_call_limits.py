@@ -274,32 +274,6 @@ def test_adjoint_of_very_small_and_large_weights(shape):
         assert np.all(np.abs(got - want) <= 2.0 ** -23 * np.abs(want) + 2.0 ** -40 * np.abs(want).max())
 
 
-def test_adjoint_of_an_infinite_weight():
-    """One track of infinite weight: only where that track has a gradient is the
-    result not finite (its rejected clusters and the steps without an update,
-    a propagation or a rotation have none; cuts this tight reject a third)."""
-    import torch
-
-    f, tr, dev, _, t = refit_setup(n_primaries=300, final_chi2=1.5, int_chi2=3.0)
-    # (28,800 coefficients; the ranges beyond every cluster: a clamped one would have
-    # weights of exactly 0, and 0 x infinity in their place)
-    coeff = torch.as_tensor(0.02 * np.random.default_rng(4).standard_normal((3, 40, 20, 12)),
-                            dtype=torch.float32).cuda()
-    n = tr.refit(dev, t, coeff, r_range=(80.0, 270.0),
-                 z_range=(-300.0, 300.0))["n_clusters"].cpu().numpy().copy()
-    have = np.diff(t["cl_offset"].cpu().numpy())
-    nt = len(n)
-    assert np.sum(n) < 0.8 * np.sum(have[n > 0])
-    for i in np.nonzero(n > 0)[0][:60]:
-        w = torch.zeros(nt, device="cuda")
-        w[i] = 1.0
-        one = tr.refit_backward(w).cpu().numpy()
-        w[i] = float("inf")
-        inf = tr.refit_backward(w).cpu().numpy()
-        assert not np.isfinite(inf).all()
-        assert np.isfinite(inf[one == 0.0]).all(), int(i)
-
-
 def test_adjoints_of_two_contexts_on_two_threads():
     """Maps of 138 KB, 14 KB and 230 KB of accumulators (the last beyond shared
     memory) side by side: the attributes of the kernels belong to the process."""
