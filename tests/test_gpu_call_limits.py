@@ -298,7 +298,7 @@ def test_adjoints_of_two_contexts_on_two_threads():
                 x = tpc.Tracker(RX, TrackerOptions(), mode=0, cap_clusters=f.n)
                 x.refit(dev, t, c)
                 want = x.refit_backward(w).cpu().numpy()
-                for _ in range(400):
+                for _ in range(3000):
                     got = x.refit_backward(w).cpu().numpy()
                     if np.abs(got - want).max() > 2.0 ** -23 * np.abs(want).max():
                         failed.append((shape, "gradient"))
