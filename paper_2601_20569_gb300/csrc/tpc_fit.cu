@@ -2567,7 +2567,9 @@ __global__ void __launch_bounds__(kRevBlock) k_refit_reverse(RefitDev R, const i
       const float4 v4 = d[(e * kRecV + 4) * kRevBlock], v5 = d[(e * kRecV + 5) * kRevBlock];
       const float k0[5] = {v2.z, v2.w, v3.x, v3.y, v3.z};
       const float k1[5] = {v3.w, v4.x, v4.y, v4.z, v4.w};
-      float a0 = w2 * v1.z, a1 = w2 * v1.w;
+      // (rounded by itself: fused into the sum in its place or one of the gains'
+      // products, as the compiler chooses, the gradient would hang on that choice)
+      float a0 = __fmul_rn(w2, v1.z), a1 = __fmul_rn(w2, v1.w);
 #pragma unroll
       for (int j = 0; j < 5; ++j) {
         a0 += k0[j] * lam[j];
