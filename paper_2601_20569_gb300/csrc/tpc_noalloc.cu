@@ -97,7 +97,7 @@ struct RowX {
 // What the grid build accumulates into.  The bin counts (1.8 MB) are cleared here
 // although every complete call leaves them at zero: a call stopped between its
 // kernels, or two calls that overlapped against the rules, would otherwise spoil
-// every later one.
+// every later one.  (A one-sector call 77.7 -> 78.3 us.)
 constexpr long kBinCntVecs = (kOffBinFirst - kOffBinCnt) / 16;  // (the pad to 256 bytes too)
 
 __global__ void k_links_init(FrameDev F, RowX row_x, int n_rows, long nrr) {
