@@ -99,6 +99,7 @@ struct tpc_ctx {
   long refit_tracks = -1, refit_refs = -1;
   int* steps3 = nullptr;
   long gpart_cap = 0;
+  long rec_want = 0;  // tracks for which the adjoint's chunk (R.chunk) was settled
   std::string err = "ok";
 };
 
@@ -148,22 +149,26 @@ bool map_room(tpc_ctx* c, const tpc_map& m) {
 
 // Room for the adjoint's step records: as many tracks at a time as the refit has,
 // at most kAdjChunk, and half as many as often as there is no memory for them (the
-// adjoint runs over the tracks in chunks of R.chunk).  False without memory for one.
+// adjoint runs over the tracks in chunks of R.chunk; a chunk that memory has cut
+// short stays until a larger refit asks).  False without memory for one.
 bool record_room(tpc_ctx* c) {
   RefitDev& R = c->R;
   const long want = R.n_tracks < (long)kAdjChunk ? (R.n_tracks > 0 ? R.n_tracks : 1) : (long)kAdjChunk;
-  if (want <= R.chunk) return true;
+  if (want <= c->rec_want) return true;
   // (rounded up to a power of two, so that refits of growing size seldom allocate)
   long tracks = 256;
   while (tracks < want) tracks *= 2;
   cudaFree(R.rec);
   R.rec = nullptr;
   R.chunk = 0;
+  c->rec_want = 0;
+  const long all = tracks;
   for (; tracks >= 1; tracks /= 2) {
     void* v = nullptr;
     if (cudaMalloc(&v, (size_t)tracks * kRecTrackBytes) == cudaSuccess) {
       R.rec = (float4*)v;
       R.chunk = (int)tracks;
+      c->rec_want = all;
       return true;
     }
     cudaGetLastError();
@@ -928,11 +933,12 @@ tpc_status tpc_refit_backward(tpc_ctx* ctx, const float* dl_dchi2, float* dl_dma
   R.ncoef = (int)ncoef;
   R.gblocks = ctx->sms;
   R.smem_max = smem_max;
-  if (!record_room(ctx)) return fail(ctx, TPC_ERR_OOM, "adjoint records");
+  // (the sums first: the records make do with what is left)
   if ((long)R.gblocks * ncoef > ctx->gpart_cap) {
     if (!dalloc(ctx, &R.gpart, (long)R.gblocks * ncoef)) return fail(ctx, TPC_ERR_OOM, "gradient partials");
     ctx->gpart_cap = (long)R.gblocks * ncoef;
   }
+  if (!record_room(ctx)) return fail(ctx, TPC_ERR_OOM, "adjoint records");
   R.dl_dchi2 = dl_dchi2;
   R.dl_dmap = dl_dmap;
   cudaStream_t s = (cudaStream_t)cuda_stream;

@@ -2603,10 +2603,11 @@ __global__ void __launch_bounds__(kRevBlock) k_refit_reverse(RefitDev R, const i
 // (tf_add_product: finer than FP64 up to a track's 160 clusters): this GPU's FP64
 // rate is 1/60 of its FP32 rate, and 192 FP64 operations per cluster would cost
 // more than the whole sweep.  (Against float pairs, which fall short of FP64, the
-// adjoint of 3.1e5 tracks takes 14.1 instead of 11.8 ms.)  Clusters whose gradients leave the range in which that holds (kSumLow,
-// kSumHigh; infinities and NaN) are added term by term in FP64.  kShared: the
-// block's accumulators lie in shared memory; a map too large for that has them in
-// the block's partial sums in global memory.
+// adjoint of 3.1e5 tracks takes 14.1 instead of 11.8 ms.)  Clusters whose gradients
+// leave the range in which that holds (kSumLow, kSumHigh; infinities and NaN) are
+// added term by term in FP64.  kShared: the block's accumulators lie in shared
+// memory; a map too large for that has them in the block's partial sums in global
+// memory.
 constexpr int kScatWarps = 16;
 constexpr int kScatF = 16;  // floats per staged cluster: wz[4], wr[4], wp[4], g[3], cell
 constexpr unsigned kSumLow = (127u - 40u) << 23;    // 2^-40: 2^-149 is 2^-109 of the largest
